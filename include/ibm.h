@@ -141,10 +141,10 @@ ibm_status ibm_set_markers(ibm_grid *g, int n, const double *X0, const double *U
 ibm_status ibm_set_wall_temperature(ibm_grid *g, const double *Tw);
 
 /* Stopping rule of the quadrature solve A~ eps~ = 1 (Sec. 2.2): the
- * iterative solver (more than 160 markers) stops when
+ * solver of more than 160 markers stops when
  * max_k |1 - (A~ eps~)_k| <= tol, after at most maxit iterations
- * (IBM_ERR_NOCONV otherwise); the direct solver (up to 160 markers) refines
- * to its rounding floor and checks the same bound.  Defaults 1e-12 and 4000.
+ * (IBM_ERR_NOCONV otherwise); up to 160 markers the solution is refined
+ * to its rounding floor and the same bound checked.  Defaults 1e-12 and 4000.
  * Takes effect from the next ibm_set_markers (and every step of a moving
  * body).  Errors: IBM_ERR_ARG (tol outside (0, 1) or maxit < 1). */
 ibm_status ibm_set_quadrature(ibm_grid *g, double tol, int maxit);

@@ -325,6 +325,7 @@ struct QuadBuffers {
     double *r, *z, *p, *q;   // cap each
     int *iters;              // CG iterations of the last solve
     double *resid;           // true residual of the last solve
+    const int *order = nullptr;   // the markers in bin order, or null
 };
 
 int quad_row_width(int dim);

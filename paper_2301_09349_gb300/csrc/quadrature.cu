@@ -7,12 +7,22 @@
 // Because Phi is a tensor product, A~_kl = prod_d sum_i phi(r_k,d(i))
 // phi(r_l,d(i)) over the three support columns of k on each axis.  Rows are
 // assembled in ELL form (column-major, one warp per marker, neighbours
-// found through the marker bins in a fixed order).  Up to 160 markers a
-// single CTA factors the dense matrix (Cholesky in FP32, refined to the FP64
-// solution); above, a single CTA
-// runs Jacobi-preconditioned CG in FP64 with fixed-order block reductions.
-// Either way the result is bitwise reproducible; every loop is bounded.
+// found through the marker bins in a fixed order).  The solution is FP64:
+// residuals rhs - A~ x and the stopping test are formed in FP64, and only the
+// corrections come from FP32 conjugate gradients, on one CTA (up to 512
+// markers) or one thread-block cluster (up to 16384).  Systems FP32 cannot
+// contract go to a dense FP32 Cholesky refined in FP64 (up to 160 markers)
+// and to Jacobi-preconditioned CG in FP64 on one CTA, which also takes the
+// systems of more than 16384 markers.  Fixed-order sums throughout: the
+// result is bitwise reproducible; every loop is bounded.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
+#include "device_table.h"
 #include "internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace ibmk {
 namespace {
@@ -249,8 +259,469 @@ pcg_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ rh
     }
 }
 
-// Small systems: A~ is copied dense, in FP32, into shared memory from the
-// ELL rows.  FP64 runs at a small fraction of the FP32 rate on this GPU, so
+// sums of a and b over the warp: lanes below 16 return a's, the others b's
+__device__ __forceinline__ float warp_sum2(float a, float b, int lane) {
+    float v = lane & 16 ? b : a;
+    v += __shfl_xor_sync(0xffffffffu, lane & 16 ? a : b, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+// the sums over the CTA's warps of the pairs part[w], part[32 + w] (zeros
+// past the last warp), in every lane
+__device__ __forceinline__ float2 part_sum2(const float *part, int lane) {
+    const float *p = part + (lane & 16 ? 32 : 0) + (lane & 15);
+    float v = p[0] + p[16];
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    const float w = __shfl_xor_sync(0xffffffffu, v, 16);
+    return lane & 16 ? make_float2(w, v) : make_float2(v, w);
+}
+// r.u at which max|r| has fallen far enough: by `inner` from rmax's own r.u,
+// or (the diagonal of A~ is at most one) to a tenth of tol in the mean square
+__device__ __forceinline__ float cg_stop(float ru, float inner, int ns, double tol) {
+    const float t = 0.1f * (float)tol;
+    return fmaxf(ru * inner * inner, (float)ns * t * t);
+}
+
+// BCG_MAX to CL_MAX markers: FP32 conjugate gradients inside FP64 iterative
+// refinement, on one thread-block cluster.
+//
+// The FP64 PCG on one CTA (above) is bound by the FP64 pipe of a single SM
+// (about two operations per cycle; 85 k nonzeros of a 2842-marker sphere take
+// 25 us of it per iteration) and by the L2 latency of the ELL rows: 10.36 ms
+// for that sphere, 3.56 ms for 713 markers.  Here the rows are dealt to the
+// CTAs of a cluster (8, or 16 above CL_WIDE markers), 2^j threads per row,
+// which hold their FP32 entries in registers (past CL_REG in shared memory,
+// past that the ELL rows serve); the correction
+// equation A~ d = r is solved in FP32 (Jacobi preconditioner, the
+// single-reduction form of Chronopoulos and Gear) to CL_INNER of its
+// residual, and r = rhs - A~ x is formed in FP64 from the ELL rows, so the
+// solution and the stopping test max|r| <= tol are those of the FP64 solver.
+// Per iteration: the product from a replicated copy of u, the warps' partial
+// sums sent to every CTA through distributed shared memory, a cluster
+// barrier, the vector updates, u sent to every CTA, a second barrier: what
+// bounds it now are the two exchanges (on a GB300 a cluster barrier behind
+// remote stores takes ~1000 cycles with 8 CTAs and, with all of u travelling,
+// ~2400 with 16).  2842 markers 10.36 -> 0.69 ms, 713 markers 3.56 -> 0.34 ms
+// (one CTA of 1024 threads, whose gathers meet in the banks: 0.55).  Every CTA reduces the same partials in the same order, so all take
+// the same branches and the result is bitwise reproducible.  A system that
+// FP32 cannot contract (near-singular A~: two markers in one cell placed
+// without dedup) goes to the FP64 PCG in the same launch.
+constexpr int CL_CTAS = 8, CL_CTAS_WIDE = 16;
+constexpr int CL_WIDE = 1536;            // above, the product of 8 CTAs outweighs 16's exchange
+constexpr int CL_MAX = 16384;            // 16 CTAs of 1024 rows, 16-bit columns
+constexpr int CL_SM = 16;                // entries of a thread in shared memory
+constexpr float CL_INNER = 1e-5f;
+constexpr int CL_OUTER_MAX = 24;
+template <int NTH> constexpr int CL_REG = NTH <= 512 ? 24 : 12;   // entries in registers
+
+struct ClusterShape {
+    int ctas;       // CTAs of the cluster
+    int rows;       // rows per CTA, a multiple of 4
+    int lpr_log;    // log2 of the threads per row
+};
+
+ClusterShape cluster_shape(int ns) {
+    ClusterShape c;
+    c.ctas = ns > CL_WIDE ? CL_CTAS_WIDE : CL_CTAS;
+    c.rows = ((ns + c.ctas - 1) / c.ctas + 3) / 4 * 4;   // chunks of u move as 16-byte words
+    c.lpr_log = 0;
+    while (c.lpr_log < 4 && (2 << c.lpr_log) * c.rows <= 512) ++c.lpr_log;
+    return c;
+}
+
+// u of every row (16-byte aligned), the CTAs' FP64 maxima and partial sums,
+// the threads' entries past their registers
+template <int NTH>
+size_t cluster_smem(const ClusterShape &c) {
+    return sizeof(float) * (size_t)c.ctas * c.rows + (sizeof(double) + sizeof(float2)) * c.ctas +
+           (sizeof(float) + sizeof(unsigned short)) * (size_t)CL_SM * NTH;
+}
+
+template <int NTH>
+__global__ void __launch_bounds__(NTH, 1)
+cluster_cg_kernel(int ns, const ClusterShape sh, const QuadBuffers q, double *x,
+                  const double *__restrict__ rhs, double tol, int maxit, int warm, int *err) {
+    constexpr int REG = CL_REG<NTH>;
+    extern __shared__ __align__(16) double smem_cl[];
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = sh.ctas, R = sh.rows, LG = sh.lpr_log, LPR = 1 << LG;
+    const int rank = (int)cl.block_rank();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int sub = tid & (LPR - 1), row = tid >> LG, k = rank * R + row;
+    const bool own = row < R && k < ns, on = 32 * warp < (R << LG);
+    float *su = reinterpret_cast<float *>(smem_cl);                    // [C * R]
+    double *smax = reinterpret_cast<double *>(su + C * R);             // [C]
+    float2 *spart = reinterpret_cast<float2 *>(smax + C);              // [C] (r.u, w.u)
+    float *sval = reinterpret_cast<float *>(spart + C);                // [CL_SM][NTH]
+    unsigned short *scol = reinterpret_cast<unsigned short *>(sval + CL_SM * NTH);
+    __shared__ float s_warp[64];
+    __shared__ double s_red[32];
+    if (tid < 64) s_warp[tid] = 0.0f;
+    // entry j of this thread: number sub + j LPR of its row
+    const int cnt = own ? q.cnt[k] : 0;
+    const int mine = cnt > sub ? (cnt - sub + LPR - 1) >> LG : 0;
+    auto entry = [&](int j, float &v, int &l) {
+        v = 0.0f;
+        l = 0;
+        if (j < mine) {
+            const long long at = (long long)(sub + (j << LG)) * q.cap + k;
+            l = q.col[at];
+            v = (float)q.val[at];
+            if (!in_bounds(l, ns, err)) { l = 0; v = 0.0f; }
+        }
+    };
+    float rv[REG];
+    unsigned rc[REG / 2];
+#pragma unroll
+    for (int j = 0; j < REG; j += 2) {
+        int l0, l1;
+        entry(j, rv[j], l0);
+        entry(j + 1, rv[j + 1], l1);
+        rc[j / 2] = (unsigned)l0 | ((unsigned)l1 << 16);
+    }
+    for (int j = REG; j < min(mine, REG + CL_SM); ++j) {
+        float v;
+        int l;
+        entry(j, v, l);
+        sval[(j - REG) * NTH + tid] = v;
+        scol[(j - REG) * NTH + tid] = (unsigned short)l;
+    }
+    const float inv = own ? (float)(1.0 / q.diag[k]) : 0.0f;
+    double xk = own && warm ? x[k] : 0.0;
+    if (own && !warm && sub == 0) x[k] = 0.0;
+    __threadfence();
+    cl.sync();
+
+    // (r.u, w.u) over the cluster: the CTA's own first, one 8-byte store to
+    // every CTA, a cluster barrier; the CTAs' values summed in one order by
+    // every warp
+    auto reduce_all = [&](float a, float b) {
+        if (on) {
+            const float t = warp_sum2(a, b, lane);
+            if ((lane & 15) == 0) s_warp[2 * (lane & 16) + warp] = t;
+        }
+        __syncthreads();
+        if (warp == 0) {
+            const float2 v = part_sum2(s_warp, lane);
+            if (lane < C) cl.map_shared_rank(spart, lane)[rank] = v;
+        }
+        cl.sync();
+        const float2 v = (lane & 15) < C ? spart[lane & 15] : make_float2(0.0f, 0.0f);
+        float s1 = lane & 16 ? v.y : v.x;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        const float s2 = __shfl_xor_sync(0xffffffffu, s1, 16);
+        return lane & 16 ? make_float2(s2, s1) : make_float2(s1, s2);
+    };
+    // this CTA's rows of u to every CTA
+    auto send_u = [&](float u) {
+        if (row < R && sub == 0) su[rank * R + row] = u;
+        __syncthreads();
+        const int n4 = R / 4;
+        float4 *part4 = reinterpret_cast<float4 *>(su + rank * R);
+        for (int i = tid; i < n4 * C; i += NTH) {
+            const int t = i / n4, j = i - t * n4;
+            if (t != rank) cl.map_shared_rank(part4, t)[j] = part4[j];
+        }
+        cl.sync();
+    };
+
+    int it = 0;
+    bool converged = false;
+    double rmax = 0.0, rprev = 0.0;
+    for (int outer = 0;; ++outer) {
+        // r = rhs - A~ x in FP64 from the ELL rows; x was written by its rows'
+        // owners before the last cluster barrier
+        double a = 0.0;
+#pragma unroll 4
+        for (int i = sub; i < cnt; i += LPR) {
+            const int l = __ldg(q.col + (long long)i * q.cap + k);
+            if (in_bounds(l, ns, err)) a += __ldg(q.val + (long long)i * q.cap + k) * __ldcg(x + l);
+        }
+        for (int o = LPR / 2; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        const double r64 = own ? (rhs ? rhs[k] : 1.0) - a : 0.0;
+        rmax = block_max<NTH>(fabs(r64), s_red);
+        if (tid < C) cl.map_shared_rank(smax, tid)[rank] = rmax;
+        cl.sync();
+        rmax = lane < C ? smax[lane] : 0.0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            rmax = dmax_nonneg(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
+        if (rmax <= tol) { converged = true; break; }
+        // no contraction, or a value FP32 cannot hold: the FP64 solver
+        if (!(rmax < 1e15) || rmax < 1e-15 || (outer > 0 && !(rmax < 0.25 * rprev)) ||
+            outer == CL_OUTER_MAX || it >= maxit)
+            break;
+        rprev = rmax;
+        // the correction d, from zero (a row's threads all hold its values)
+        float r = (float)r64, u = r * inv, p = 0.0f, sv = 0.0f, d = 0.0f, gam = 1.0f, alpha = 1.0f,
+              stop = 0.0f;
+        send_u(u);
+        for (bool first = true;; first = false) {
+            float w = 0.0f;
+            if (on) {
+                float w1 = 0.0f;
+#pragma unroll
+                for (int j = 0; j < REG; j += 2) {
+                    if (j >= mine) break;
+                    w += rv[j] * su[rc[j / 2] & 0xffffu];
+                    w1 += rv[j + 1] * su[rc[j / 2] >> 16];
+                }
+                for (int j = REG; j < mine; ++j) {
+                    if (j < REG + CL_SM) {
+                        w += sval[(j - REG) * NTH + tid] * su[scol[(j - REG) * NTH + tid]];
+                    } else {
+                        float v;
+                        int l;
+                        entry(j, v, l);
+                        w += v * su[l];
+                    }
+                }
+                w += w1;
+                for (int o = LPR / 2; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+            }
+            const float2 tot = reduce_all(sub == 0 ? r * u : 0.0f, sub == 0 ? w * u : 0.0f);
+            const float g1 = tot.x, del = tot.y;
+            if (first) stop = cg_stop(g1, CL_INNER, ns, tol);
+            if (g1 <= stop) break;
+            const float beta = first ? 0.0f : __fdividef(g1, gam);
+            const float den = first ? del : del - beta * __fdividef(g1, alpha);
+            if (!(den > 0.0f) || ++it >= maxit) break;   // (a NaN sum ends here too)
+            alpha = __fdividef(g1, den);
+            gam = g1;
+            p = u + beta * p;
+            sv = w + beta * sv;
+            d += alpha * p;
+            r -= alpha * sv;
+            u = r * inv;
+            send_u(u);
+        }
+        // the next residual reads every CTA's rows
+        xk += (double)d;
+        if (own && sub == 0) x[k] = xk;
+        __threadfence();
+        cl.sync();
+    }
+    cl.sync();   // no CTA leaves while another may still write to it
+    if (rank != 0) return;
+    // x holds the refined values: kept if finite with a residual below 1
+    if (!converged)
+        converged = pcg_solve<NTH>(ns, q, x, rhs, tol, maxit, rmax < 1.0, s_red, &it, &rmax, err);
+    if (tid == 0) {
+        *q.iters = it;
+        *q.resid = rmax;
+        if (!converged) record_error(err, ERR_NOCONV);
+    }
+}
+
+template <int NTH>
+cudaError_t launch_cluster_cg(int ns, const ClusterShape &sh, const QuadBuffers &qb, double *x,
+                              const double *rhs, double tol, int maxit, int warm, int *err,
+                              cudaStream_t s) {
+    const void *fn = (const void *)cluster_cg_kernel<NTH>;
+    const size_t smem = cluster_smem<NTH>(sh);
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = func_smem_attr(fn, smem);
+    if (e != cudaSuccess) return e;
+    static DeviceAttrTable wide;   // clusters of 16 are an opt-in of the kernel, per device
+    e = (cudaError_t)wide.ensure(fn, dev, 1, [&]() -> int {
+        return (int)cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    });
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)sh.ctas);
+    cfg.blockDim = dim3(NTH);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)sh.ctas;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, cluster_cg_kernel<NTH>, ns, sh, qb, x, rhs, tol, maxit, warm, err);
+}
+
+// 161 to BCG_MAX markers: the same method on one CTA, one thread per row in
+// bin order (neighbouring lanes gather neighbouring u-values: few bank
+// conflicts), the row's first FP32 entries in its registers.  An iteration is
+// one product, one block reduction (two sums folded into one butterfly, ten
+// shuffles) and two block barriers of ~200 cycles each: 1.2 us at 388
+// markers, where a cluster of eight CTAs took 2.5 us, its two cluster
+// barriers with their remote stores costing more than the wider product
+// saves.  388-marker moving sphere: 1116 us (FP64 PCG) -> 167 us per step;
+// the gathers' bank conflicts bound it (one copy of u: 221 us).
+constexpr int BCG_MAX = 512;
+constexpr int BCG_SM = 24;              // entries of a thread in shared memory
+constexpr int BCG_REP = 8;              // copies of u: lane l gathers from copy l % 8, so only four
+                                        // lanes of a warp can meet in a bank
+constexpr int BCG_OUTER_MAX = 24;
+constexpr float BCG_INNER = 1e-5f;
+template <int NTH> constexpr int BCG_REG = NTH <= 512 ? 32 : 12;   // entries in registers
+
+template <int NTH>
+constexpr size_t block_cg_smem() {
+    return sizeof(double) * NTH + (sizeof(float) + sizeof(unsigned short)) * (size_t)BCG_SM * NTH +
+           sizeof(float) * BCG_REP * NTH + sizeof(unsigned short) * NTH;
+}
+
+template <int NTH>
+__global__ void __launch_bounds__(NTH, 1)
+block_cg_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ rhs, double tol,
+                int maxit, int warm, int *err) {
+    constexpr int REG = BCG_REG<NTH>;
+    extern __shared__ __align__(16) double smem_b[];
+    double *sx = smem_b;                                          // [NTH] solution, marker order
+    float *sval = reinterpret_cast<float *>(sx + NTH);            // [BCG_SM][NTH]
+    float *su = sval + BCG_SM * NTH;                              // [NTH][BCG_REP] u, row order
+    unsigned short *scol = reinterpret_cast<unsigned short *>(su + BCG_REP * NTH);   // [BCG_SM][NTH]
+    unsigned short *srow = scol + BCG_SM * NTH;                   // [NTH] row of a marker
+    __shared__ float s_part[64];
+    __shared__ double s_red[32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool own = tid < ns, on = 32 * warp < ns;               // a row; a warp with rows
+    const int k = own ? (q.order ? q.order[tid] : tid) : 0;
+    const int cnt = own ? q.cnt[k] : 0;
+    if (tid < 64) s_part[tid] = 0.0f;
+    if (own) {
+        srow[k] = (unsigned short)tid;
+        sx[k] = warm ? x[k] : 0.0;
+    }
+    __syncthreads();
+    // the row's entries: FP32 value and row of the column's marker
+    auto entry = [&](int i, float &v, int &l) {
+        v = 0.0f;
+        l = own ? tid : 0;
+        if (i < cnt) {
+            const int c = q.col[(long long)i * q.cap + k];
+            if (in_bounds(c, ns, err)) {
+                v = (float)q.val[(long long)i * q.cap + k];
+                l = srow[c];
+            }
+        }
+    };
+    float rv[REG];
+    unsigned rc[REG / 2];
+#pragma unroll
+    for (int j = 0; j < REG; j += 2) {
+        int l0, l1;
+        entry(j, rv[j], l0);
+        entry(j + 1, rv[j + 1], l1);
+        rc[j / 2] = (unsigned)l0 | ((unsigned)l1 << 16);
+    }
+    for (int j = REG; j < min(cnt, REG + BCG_SM); ++j) {
+        float v;
+        int l;
+        entry(j, v, l);
+        sval[(j - REG) * NTH + tid] = v;
+        scol[(j - REG) * NTH + tid] = (unsigned short)l;
+    }
+    const float inv = own ? (float)(1.0 / q.diag[k]) : 0.0f;
+    const float *const suc = su + (lane & (BCG_REP - 1));   // this lane's copy
+    auto put_u = [&](float u) {
+        if (!own) return;
+        float4 *d4 = reinterpret_cast<float4 *>(su + BCG_REP * tid);
+        d4[0] = d4[1] = make_float4(u, u, u, u);
+    };
+    static_assert(BCG_REP == 8, "put_u writes eight copies");
+    __syncthreads();
+
+    int it = 0;
+    bool converged = false;
+    double rmax = 0.0, rprev = 0.0;
+    for (int outer = 0;; ++outer) {
+        // r = rhs - A~ x in FP64 from the ELL rows
+        double a = 0.0;
+#pragma unroll 4
+        for (int i = 0; i < cnt; ++i) {
+            const int l = __ldg(q.col + (long long)i * q.cap + k);
+            if (in_bounds(l, ns, err)) a += __ldg(q.val + (long long)i * q.cap + k) * sx[l];
+        }
+        const double r64 = own ? (rhs ? rhs[k] : 1.0) - a : 0.0;
+        rmax = block_max<NTH>(fabs(r64), s_red);
+        if (rmax <= tol) { converged = true; break; }
+        if (!(rmax < 1e15) || rmax < 1e-15 || (outer > 0 && !(rmax < 0.25 * rprev)) ||
+            outer == BCG_OUTER_MAX || it >= maxit)
+            break;
+        rprev = rmax;
+        float r = (float)r64, u = r * inv, p = 0.0f, sv = 0.0f, d = 0.0f, gam = 1.0f, alpha = 1.0f,
+              stop = 0.0f;
+        put_u(u);
+        __syncthreads();
+        for (bool first = true;; first = false) {
+            float w = 0.0f;
+            if (on) {
+                float w1 = 0.0f;
+#pragma unroll
+                for (int j = 0; j < REG; j += 2) {
+                    w += rv[j] * suc[BCG_REP * (rc[j / 2] & 0xffffu)];
+                    w1 += rv[j + 1] * suc[BCG_REP * (rc[j / 2] >> 16)];
+                }
+                for (int j = REG; j < cnt; ++j) {
+                    if (j < REG + BCG_SM) {
+                        w += sval[(j - REG) * NTH + tid] * suc[BCG_REP * scol[(j - REG) * NTH + tid]];
+                    } else {
+                        float v;
+                        int l;
+                        entry(j, v, l);
+                        w += v * suc[BCG_REP * l];
+                    }
+                }
+                w += w1;
+                const float t = warp_sum2(r * u, w * u, lane);
+                if ((lane & 15) == 0) s_part[2 * (lane & 16) + warp] = t;
+            }
+            __syncthreads();
+            const float2 tot = part_sum2(s_part, lane);
+            const float g1 = tot.x;
+            if (first) stop = cg_stop(g1, BCG_INNER, ns, tol);
+            if (g1 <= stop) break;
+            const float beta = first ? 0.0f : __fdividef(g1, gam);
+            const float den = first ? tot.y : tot.y - beta * __fdividef(g1, alpha);
+            if (!(den > 0.0f) || ++it >= maxit) break;   // (a NaN sum ends here too)
+            alpha = __fdividef(g1, den);
+            gam = g1;
+            p = u + beta * p;
+            sv = w + beta * sv;
+            d += alpha * p;
+            r -= alpha * sv;
+            u = r * inv;
+            put_u(u);
+            __syncthreads();
+        }
+        if (own) sx[k] += (double)d;
+        __syncthreads();
+    }
+    if (own) x[k] = sx[k];
+    __syncthreads();
+    if (!converged) {
+        // what FP32 cannot contract: the FP64 solver, from the refined values
+        // if they are finite with a residual below 1, else from zero
+        converged = pcg_solve<NTH>(ns, q, x, rhs, tol, maxit, rmax < 1.0, s_red, &it, &rmax, err);
+    }
+    if (tid == 0) {
+        *q.iters = it;
+        *q.resid = rmax;
+        if (!converged) record_error(err, ERR_NOCONV);
+    }
+}
+
+template <int NTH>
+cudaError_t launch_block_cg(int ns, const QuadBuffers &qb, double *x, const double *rhs, double tol,
+                            int maxit, int warm, int *err, cudaStream_t s) {
+    cudaError_t e = func_smem_attr((const void *)block_cg_kernel<NTH>, block_cg_smem<NTH>());
+    if (e != cudaSuccess) return e;
+    block_cg_kernel<NTH><<<1, NTH, block_cg_smem<NTH>(), s>>>(ns, qb, x, rhs, tol, maxit, warm, err);
+    return cudaGetLastError();
+}
+
+// Small systems (up to CHOL_MAX markers) on one CTA: corrections by FP32
+// conjugate gradients first (small_cg); a system they do not contract by ten
+// per pass is factored.  A~ is then copied dense, in FP32, into shared memory
+// from the ELL rows.  FP64 runs at a small fraction of the FP32 rate on this GPU, so
 // the O(ns^3) work is done in FP32: a blocked right-looking Cholesky
 // A~ = L L^T over 32-column panels (one warp factors the panel's diagonal
 // block without block barriers, one thread per row solves the rows below
@@ -438,6 +909,71 @@ __device__ __forceinline__ void chol_diag_inverse(float *__restrict__ F, int ld,
     }
 }
 
+// FP32 conjugate gradients for the correction A~ d = r32 of a small system
+// (the threads of the first ceil(ns / 32) warps, one row each; the other
+// warps wait): Jacobi preconditioner, single-reduction form, until the
+// residual has fallen by SCG_INNER.  The surface systems of one marker per cell are
+// well conditioned (about four iterations per decimal digit), and an
+// iteration costs ~600 cycles against ~118 k for the dense factor of 97
+// markers: 61.5 -> 40.8 us per step of the moving cylinder.  The row's first SCG_REG
+// FP32 entries sit in registers.  d replaces r32 in st; false when it did not
+// get there in SCG_ITS iterations (the caller then factors A~).
+constexpr int SCG_REG = 8, SCG_ITS = 48, SCG_W = (CHOL_MAX + 31) / 32;
+constexpr float SCG_INNER = 1e-5f;
+__device__ __forceinline__ bool small_cg(int ns, const QuadBuffers &q, int k, int cnt,
+                                         const float (&rv)[SCG_REG], const int (&rc)[SCG_REG],
+                                         float inv, const float *__restrict__ ev32,
+                                         const int *__restrict__ ec, float r,
+                                         float *__restrict__ su, float *__restrict__ part,
+                                         float &d, int &it) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nw = (ns + 31) / 32, nth = 32 * nw;
+    auto bar = [&]() { asm volatile("bar.sync 1, %0;" ::"r"(nth) : "memory"); };
+    float stop = 0.0f;
+    float u = r * inv, p = 0.0f, sv = 0.0f, gam = 1.0f, alpha = 1.0f;
+    d = 0.0f;
+    if (k < ns) su[k] = u;
+    bar();
+    for (int n = 0;; ++n) {
+        float w = 0.0f;
+#pragma unroll
+        for (int i = 0; i < SCG_REG; ++i) w += rv[i] * su[rc[i]];
+        for (int i = SCG_REG; i < cnt; ++i) {
+            if (i < CHOL_EC) {
+                w += ev32[i * ns + k] * su[ec[i * ns + k]];
+            } else {
+                const int l = q.col[(long long)i * q.cap + k];
+                w += (float)q.val[(long long)i * q.cap + k] * su[l];
+            }
+        }
+        const float t = warp_sum2(r * u, w * u, lane);
+        if ((lane & 15) == 0) part[2 * warp + (lane >> 4)] = t;
+        bar();
+        float g1 = 0.0f, del = 0.0f;
+#pragma unroll
+        for (int i = 0; i < SCG_W; ++i) {   // the slots past nw hold zeros
+            const float2 v = reinterpret_cast<const float2 *>(part)[i];
+            g1 += v.x;
+            del += v.y;
+        }
+        if (n == 0) stop = g1 * SCG_INNER * SCG_INNER;
+        if (g1 <= stop) return true;
+        const float beta = n == 0 ? 0.0f : __fdividef(g1, gam);
+        const float den = n == 0 ? del : del - beta * __fdividef(g1, alpha);
+        if (!(den > 0.0f) || n == SCG_ITS) return false;   // (a NaN sum too)
+        alpha = __fdividef(g1, den);
+        gam = g1;
+        p = u + beta * p;
+        sv = w + beta * sv;
+        d += alpha * p;
+        r -= alpha * sv;
+        u = r * inv;
+        if (k < ns) su[k] = u;
+        ++it;
+        bar();
+    }
+}
+
 // one CTA per launch: the register file is the CTA's alone, so the
 // registers a thread may take are bounded for one resident block (the
 // diagonal-block factor keeps a 32-float row per lane)
@@ -462,23 +998,21 @@ chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ r
     __shared__ double s_red[CHOL_T / 32];
     __shared__ int s_bad;
     __shared__ __align__(16) float s_col[CHOL_PB];
+    __shared__ __align__(8) float s_part[2 * SCG_W];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int i = tid; i < ns * ld; i += CHOL_T) F[i] = 0.0f;
     if (tid == 0) s_bad = 0;
-    __syncthreads();
-    // lower triangle of A~ (the upper triangle stays zero); the rows' first
-    // CHOL_EC entries and their lengths kept for the residuals
+    if (tid < 2 * SCG_W) s_part[tid] = 0.0f;
+    // the rows' first CHOL_EC entries and their lengths, kept for the
+    // residuals; their FP32 values for the conjugate gradients in F's place
     for (int k = tid; k < ns; k += CHOL_T) {
         const int c = q.cnt[k];
         ecnt[k] = c;
-        for (int i = 0; i < c; ++i) {
-            const int l = q.col[(long long)i * q.cap + k];
-            const double v = q.val[(long long)i * q.cap + k];
-            if (i < CHOL_EC) {
-                ec[(size_t)i * ns + k] = l;
-                ev[(size_t)i * ns + k] = v;
-            }
-            if (in_bounds(l, ns, err) && l <= k) F[(size_t)k * ld + l] = (float)v;
+        for (int i = 0; i < min(c, CHOL_EC); ++i) {
+            int l = q.col[(long long)i * q.cap + k];
+            double v = q.val[(long long)i * q.cap + k];
+            if (!in_bounds(l, ns, err)) { l = k; v = 0.0; }
+            ec[(size_t)i * ns + k] = l;
+            ev[(size_t)i * ns + k] = v;
         }
         sx[k] = warm ? x[k] : 0.0;
     }
@@ -490,26 +1024,9 @@ chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ r
         rscale = block_max<CHOL_T>(lr, s_red);   // synchronizes
     }
     __syncthreads();
-    // blocked Cholesky over 32-column panels, then the diagonal blocks' inverses
-    for (int c0 = 0; c0 < ns; c0 += CHOL_PB) {
-        const int w = min(CHOL_PB, ns - c0);
-        if (warp == 0) chol_diag_block(F, ld, c0, w, dinv, lane, &s_bad, s_col);
-        __syncthreads();
-        if (c0 + w < ns) {
-            chol_panel_rows(F, ld, c0, w, ns, dinv, tid);
-            __syncthreads();
-            chol_trailing(F, ld, c0, w, ns, tid);
-            __syncthreads();
-        }
-    }
-    if (warp * CHOL_PB < ns)
-        chol_diag_inverse(F, ld, warp * CHOL_PB, min(CHOL_PB, ns - warp * CHOL_PB), dinv, lane);
-    __syncthreads();
-    // refinement: r = rhs - A~ x in FP64 from the ELL rows (one thread per
-    // row), x += L^-T L^-1 r in FP32
-    double rmax = 0.0, rprev = 0.0;
-    int it = 0;
-    for (;; ++it) {
+    // r = rhs - A~ x in FP64 from the ELL rows (one thread per row) into r32,
+    // its largest entry returned (synchronizes)
+    auto residual = [&]() {
         double lm = 0.0;
         for (int k = tid; k < ns; k += CHOL_T) {
             const int c = ecnt[k];
@@ -528,7 +1045,7 @@ chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ r
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
-                    if (i0 + u < cc && in_bounds(l[u], ns, err)) sum += v[u] * sx[l[u]];
+                    if (i0 + u < cc) sum += v[u] * sx[l[u]];
             }
             for (int i = CHOL_EC; i < c; ++i) {
                 const int l = q.col[(long long)i * q.cap + k];
@@ -538,7 +1055,81 @@ chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ r
             r32[k] = (float)r;
             lm = dmax_nonneg(lm, fabs(r));
         }
-        rmax = block_max<CHOL_T>(lm, s_red);   // synchronizes
+        return block_max<CHOL_T>(lm, s_red);
+    };
+    double rmax = 0.0, rprev = 0.0;
+    int it = 0;
+    bool done = false;   // the residual is at its floor
+    {
+        // corrections by FP32 conjugate gradients first
+        float rv[SCG_REG], inv = 0.0f;
+        int rc[SCG_REG];
+        float *ev32 = F;
+#pragma unroll
+        for (int i = 0; i < SCG_REG; ++i) { rv[i] = 0.0f; rc[i] = 0; }
+        int cnt = 0;
+        if (tid < ns) {
+            cnt = ecnt[tid];
+            inv = (float)(1.0 / q.diag[tid]);
+            for (int i = 0; i < min(cnt, CHOL_EC); ++i) ev32[(size_t)i * ns + tid] = (float)ev[(size_t)i * ns + tid];
+#pragma unroll
+            for (int i = 0; i < SCG_REG; ++i)
+                if (i < cnt) {
+                    rv[i] = ev32[(size_t)i * ns + tid];
+                    rc[i] = ec[(size_t)i * ns + tid];
+                }
+        }
+        for (int outer = 0;; ++outer) {
+            rmax = residual();
+            if (!(rmax > 0.0) || rmax <= CHOL_FLOOR * rscale ||
+                (outer > 0 && rmax <= 64.0 * CHOL_FLOOR * rscale && !(rmax < 0.5 * rprev))) {
+                done = true;
+                break;
+            }
+            // no contraction by ten, or nothing FP32 can hold: factor A~
+            if (!(rmax < 1e15) || rmax < 1e-16 || (outer > 0 && !(rmax < 0.1 * rprev)) ||
+                outer == CHOL_REFINE_MAX)
+                break;
+            rprev = rmax;
+            float d = 0.0f;
+            bool got = true;
+            if (warp < (ns + 31) / 32) {
+                got = small_cg(ns, q, tid, cnt, rv, rc, inv, ev32, ec, tid < ns ? r32[tid] : 0.0f, st,
+                               s_part, d, it);
+                if (got && tid < ns) sx[tid] += (double)d;
+            }
+            if (__syncthreads_or(!got)) break;
+        }
+    }
+    if (!done) {
+    // the dense factor: the lower triangle of A~ (the upper stays zero)
+    for (int i = tid; i < ns * ld; i += CHOL_T) F[i] = 0.0f;
+    __syncthreads();
+    for (int k = tid; k < ns; k += CHOL_T)
+        for (int i = 0; i < ecnt[k]; ++i) {
+            const int l = q.col[(long long)i * q.cap + k];
+            if (in_bounds(l, ns, err) && l <= k)
+                F[(size_t)k * ld + l] = (float)q.val[(long long)i * q.cap + k];
+        }
+    __syncthreads();
+    // blocked Cholesky over 32-column panels, then the diagonal blocks' inverses
+    for (int c0 = 0; c0 < ns; c0 += CHOL_PB) {
+        const int w = min(CHOL_PB, ns - c0);
+        if (warp == 0) chol_diag_block(F, ld, c0, w, dinv, lane, &s_bad, s_col);
+        __syncthreads();
+        if (c0 + w < ns) {
+            chol_panel_rows(F, ld, c0, w, ns, dinv, tid);
+            __syncthreads();
+            chol_trailing(F, ld, c0, w, ns, tid);
+            __syncthreads();
+        }
+    }
+    if (warp * CHOL_PB < ns)
+        chol_diag_inverse(F, ld, warp * CHOL_PB, min(CHOL_PB, ns - warp * CHOL_PB), dinv, lane);
+    __syncthreads();
+    // refinement: r = rhs - A~ x in FP64, x += L^-T L^-1 r in FP32
+    for (it = 0;; ++it) {
+        rmax = residual();
         if (!(rmax > 0.0) || rmax <= CHOL_FLOOR * rscale || (it > 0 && !(rmax < 0.5 * rprev)) ||
             it == CHOL_REFINE_MAX)
             break;
@@ -623,6 +1214,7 @@ chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ r
         for (int c = tid; c < ns; c += CHOL_T) sx[c] += (double)st[c];
         __syncthreads();
     }
+    }   // !done
     for (int k = tid; k < ns; k += CHOL_T) x[k] = sx[k];
     bool ok = !s_bad && rmax <= tol;
     if (!ok) {
@@ -644,8 +1236,9 @@ chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ r
 
 int quad_row_width(int dim) { return dim == 3 ? 125 * 4 : 25 * 4; }
 
-// A~ x = rhs (rhs == nullptr: all ones): dense Cholesky with refinement up
-// to CHOL_MAX markers, Jacobi-PCG above (either warm-started if asked)
+// A~ x = rhs (rhs == nullptr: all ones), warm-started if asked.  One CTA up
+// to BCG_MAX markers, one cluster to CL_MAX (both sides of each line measured
+// at the kernels), the FP64 PCG above
 static cudaError_t launch_quadrature_solve_w(int ns, const QuadBuffers &qb, const double *rhs,
                                             double *x, double tol, int maxit, int warm, int *err,
                                             cudaStream_t s) {
@@ -654,8 +1247,14 @@ static cudaError_t launch_quadrature_solve_w(int ns, const QuadBuffers &qb, cons
         cudaError_t e = func_smem_attr((const void *)chol_kernel, chol_smem(CHOL_MAX));
         if (e != cudaSuccess) return e;
         chol_kernel<<<1, CHOL_T, chol_smem(ns), s>>>(ns, qb, x, rhs, tol, maxit, warm, err);
-    } else if (ns <= 2048) {
-        pcg_kernel<256><<<1, 256, 0, s>>>(ns, qb, x, rhs, tol, maxit, warm, err);
+    } else if (ns <= BCG_MAX) {
+        return ns <= 512 ? launch_block_cg<512>(ns, qb, x, rhs, tol, maxit, warm, err, s)
+                         : launch_block_cg<1024>(ns, qb, x, rhs, tol, maxit, warm, err, s);
+    } else if (ns <= CL_MAX) {
+        const ClusterShape sh = cluster_shape(ns);
+        return sh.rows <= 512
+                   ? launch_cluster_cg<512>(ns, sh, qb, x, rhs, tol, maxit, warm, err, s)
+                   : launch_cluster_cg<1024>(ns, sh, qb, x, rhs, tol, maxit, warm, err, s);
     } else {
         pcg_kernel<1024><<<1, 1024, 0, s>>>(ns, qb, x, rhs, tol, maxit, warm, err);
     }
@@ -673,7 +1272,9 @@ cudaError_t launch_quadrature(const GridParams &g, const MarkerBuffers &m, const
     else assemble_kernel<2><<<nb, 128, 0, s>>>(g, m, qb, keys, perm);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_quadrature_solve_w(m.ns, qb, nullptr, m.eps, tol, maxit, warm, m.err, s);
+    QuadBuffers q = qb;
+    q.order = perm;   // the solvers may take the rows in bin order
+    return launch_quadrature_solve_w(m.ns, q, nullptr, m.eps, tol, maxit, warm, m.err, s);
 }
 
 // A~ x = rhs with the matrix assembled by the last launch_quadrature (the

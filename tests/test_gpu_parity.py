@@ -621,3 +621,41 @@ def test_quadrature_two_markers_in_one_cell(oracle, sep):
     A = oracle.assemble_A_dense(g, X[idx])
     assert np.max(np.abs(1.0 - A @ eps)) < 1e-9
     grid.close()
+
+
+@pytest.mark.parametrize("n", [31, 512, 513, 1024, 1537, 8200, 16385])
+def test_quadrature_solvers_at_their_limits(oracle, n):
+    """The one-CTA and cluster solvers on both sides of the marker counts at
+    which they change, and the FP64 PCG above 16384, against the oracle's CG.
+    Both stop at max|1 - A~ eps~| <= 1e-12; for one marker per cell the
+    smallest eigenvalue of A~ is above 1e-2 and the largest weight above 6, so the weights agree to 1e-9."""
+    rng = np.random.default_rng(n)
+    g = C.small_grid(3, (n + 8, 8, 8), h=0.1, fp_bytes=4)
+    cells = np.zeros((n, 3))
+    cells[:, 0] = 4 + rng.permutation(n)     # input order unlike bin order
+    cells[:, 1:] = 4 if n < 1000 else 3 + rng.integers(0, 2, (n, 2))
+    X = np.array(g.lo[:3]) + (cells + 0.5 + rng.uniform(-0.3, 0.3, (n, 3))) * g.h
+    grid = ibm.Grid(g, max_markers=n)
+    assert grid.set_markers(X, np.ones(n), dedup=False) == n
+    _, eps, idx = grid.markers()
+    rc, eo, it, res = oracle.quadrature(g, X[idx])
+    assert rc == 0
+    assert np.max(np.abs(eps - eo) / np.abs(eo).max()) < 1e-9
+    grid.close()
+
+
+@pytest.mark.parametrize("n", [200, 700])
+def test_near_singular_quadrature_beyond_the_dense_solver(oracle, n):
+    """Two markers 0.1 cells apart in one cell of a longer line: A~ is too
+    ill-conditioned for FP32 corrections and the same launch hands over to
+    the FP64 PCG, which meets the solver's residual bound."""
+    g = C.small_grid(2, (n + 16, 24), h=0.1, fp_bytes=8)
+    lo = np.array(g.lo[:2])
+    base = lo + (np.stack([8 + np.arange(n - 1), np.full(n - 1, 10)], 1) + 0.5) * g.h
+    X = np.vstack([base, base[5] + np.array([0.1 * g.h, 0.0])])
+    grid = ibm.Grid(g, max_markers=n)
+    assert grid.set_markers(X, np.ones(n), dedup=False) == n
+    _, eps, idx = grid.markers()
+    A = oracle.assemble_A_dense(g, X[idx])
+    assert np.max(np.abs(1.0 - A @ eps)) < 1e-9
+    grid.close()
