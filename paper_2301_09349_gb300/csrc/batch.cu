@@ -121,7 +121,7 @@ ibm_status fail(ibm_batch *b, ibm_status st, const std::string &msg) {
 
 int tiles_of_shape(const ibm_grid_desc &d, int shape) {
     int bx = 0, by = 0;
-    batch_tile_shape(shape, &bx, &by);
+    batch_tile_shape(shape, d.fp_bytes, &bx, &by);
     return ((d.n[0] + bx - 1) / bx) * ((d.n[1] + by - 1) / by);
 }
 

@@ -6,6 +6,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 namespace ibmk {
@@ -36,6 +37,11 @@ constexpr double kHeatSourceCap = 0.9;
 struct FloatConsts {
     float gamma, inv_gm1, gm1, invR, mu_inf, S, onepS, lam_fac, inv_h, qinv_h, kvisc, E_inf;
     int viscous;
+    // the 2D march's folded constants (flux_ym.cu): 2/(gamma-1),
+    // 2 + 2/(gamma-1), 2 S r, 2 mu_inf (1+S) sqrt(8)/4 r^(-1/2) / h with
+    // mu = (..) T^2 rsqrt(T (T + 2 S r)^2) of the two cells' summed T = p/rho,
+    // and 2 c_p / (Pr r)
+    float ym_e1, ym_h1, ym_s2, ym_km, ym_kl;
 };
 
 struct GridParams {
@@ -74,6 +80,11 @@ inline FloatConsts float_consts(const GridParams &g) {
     c.kvisc = (float)g.kvisc;
     c.E_inf = (float)(g.p_inf / (g.gamma - 1.0) + 0.5);
     c.viscous = g.mu_inf > 0.0;
+    c.ym_e1 = (float)(2.0 / (g.gamma - 1.0));
+    c.ym_h1 = (float)(2.0 + 2.0 / (g.gamma - 1.0));
+    c.ym_s2 = (float)(2.0 * g.S * g.R);
+    c.ym_km = (float)(2.0 * g.mu_inf * (1.0 + g.S) * sqrt(8.0) / 4.0 / sqrt(g.R) * g.inv_h);
+    c.ym_kl = (float)(2.0 * g.cp / (g.Pr * g.R));
     return c;
 }
 
@@ -165,6 +176,14 @@ __device__ __forceinline__ float2 fsub2_ftz(float2 a, float2 b) {
         "mov.b64 {%0, %1}, pd; }"
         : "=f"(r.x), "=f"(r.y)
         : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+
+// 1/a by the hardware approximation alone (1 ulp; subnormals flushed), one
+// instruction where a division by the fast intrinsic adds a product
+__device__ __forceinline__ float rcp_ftz(float a) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
     return r;
 }
 

@@ -52,6 +52,10 @@ cudaError_t launch_dt_init(const GridParams &g, int fp_bytes, const void *U,
 cudaError_t launch_zmarch(int mode, const GridParams &g, const void *Uin, const void *Un,
                           void *out, const FluidBuffers &fb, double dt_fixed, cudaStream_t s);
 size_t zmarch_blocks(const GridParams &g);
+// the y-marching form used for 2D FP32 grids (flux_ym.cu)
+cudaError_t launch_ymarch(int mode, const GridParams &g, const void *Uin, const void *Un, void *out,
+                          const FluidBuffers &fb, double dt_fixed, cudaStream_t s);
+size_t ymarch_blocks(const GridParams &g);
 
 // Step-size rate of one cell from its conserved state (DIM+2 values):
 // s = sum_d (|u_d| + c)/h + 2 DIM nu / h^2, nu = max(4/3, gamma/Pr) mu(T)/rho.
@@ -241,8 +245,11 @@ struct BatchCase {
     int band0, nband;            // its (case, band tile) spread items
 };
 
-constexpr int kBatchShapes = 4;   // 2D tile shapes of the batched stage kernel
-void batch_tile_shape(int shape, int *bx, int *by);
+constexpr int kBatchShapes = 4;   // 2D tile shapes of the batched stage kernels
+void batch_tile_shape(int shape, int fp_bytes, int *bx, int *by);
+void ymarch_tile_shape(int shape, int *bx, int *by);   // FP32: strips, by rows high
+cudaError_t launch_batch_ymarch(int mode, int shape, const BatchCase *cases, const int2 *items,
+                                int n_items, double *item_max, double dt_fixed, cudaStream_t s);
 // mode 1 or 2 as launch_stage1/2; items are (case, tile) pairs in the
 // shape's tile numbering; mode 2 writes item_max[item]
 cudaError_t launch_batch_stage(int mode, int shape, int fp_bytes, const BatchCase *cases,

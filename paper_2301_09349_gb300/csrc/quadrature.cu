@@ -916,8 +916,13 @@ __device__ __forceinline__ void chol_diag_inverse(float *__restrict__ F, int ld,
 // well conditioned (about four iterations per decimal digit), and an
 // iteration costs ~600 cycles against ~118 k for the dense factor of 97
 // markers: 61.5 -> 40.8 us per step of the moving cylinder.  The row's first SCG_REG
-// FP32 entries sit in registers.  d replaces r32 in st; false when it did not
-// get there in SCG_ITS iterations (the caller then factors A~).
+// FP32 entries sit in registers.  Curves have five to nine entries per row;
+// surfaces have over twenty and a condition number four times theirs, where
+// the dense factor is the faster (62 iterations per pass at 120 markers), so
+// systems with a row of more than SCG_ROW entries are factored at once.
+// false when it did not get there in SCG_ITS iterations (the caller then
+// factors A~).
+constexpr int SCG_ROW = 12;   // longest row for which it is tried: see above
 constexpr int SCG_REG = 8, SCG_ITS = 48, SCG_W = (CHOL_MAX + 31) / 32;
 constexpr float SCG_INNER = 1e-5f;
 __device__ __forceinline__ bool small_cg(int ns, const QuadBuffers &q, int k, int cnt,
@@ -1079,7 +1084,8 @@ chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ r
                     rc[i] = ec[(size_t)i * ns + tid];
                 }
         }
-        for (int outer = 0;; ++outer) {
+        const bool wide = __syncthreads_or(cnt > SCG_ROW) != 0;
+        for (int outer = 0; !wide; ++outer) {
             rmax = residual();
             if (!(rmax > 0.0) || rmax <= CHOL_FLOOR * rscale ||
                 (outer > 0 && rmax <= 64.0 * CHOL_FLOOR * rscale && !(rmax < 0.5 * rprev))) {

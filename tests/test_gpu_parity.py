@@ -659,3 +659,29 @@ def test_near_singular_quadrature_beyond_the_dense_solver(oracle, n):
     A = oracle.assemble_A_dense(g, X[idx])
     assert np.max(np.abs(1.0 - A @ eps)) < 1e-9
     grid.close()
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("bc", [(0, 1, 2, 2), (3, 3, 3, 3), (1, 0, 1, 2), (2, 2, 3, 3)])
+@pytest.mark.parametrize("n", [(4, 4), (5, 7), (58, 9), (59, 33), (60, 5), (61, 64), (122, 130),
+                               (181, 17), (600, 401)])
+def test_2d_fp32_march_equals_the_box_kernel(n, bc, offset):
+    """L(U) of the 2D FP32 march (strips of 60 columns, pairs of cells, chunks
+    of rows) against the FP64 tile kernel on the same FP32 values: sizes
+    around a strip, odd and smallest ones, every boundary condition, a state
+    that is only 4-byte aligned.  FP32 rounding of L with 5 % perturbations is
+    at most 1e-4 of its norm (see the module's tolerances)."""
+    g4 = C.small_grid(2, n, h=0.1, fp_bytes=4, bc=bc + (2, 2))
+    g8 = C.small_grid(2, n, h=0.1, fp_bytes=8, bc=bc + (2, 2))
+    U = torch.from_numpy(C.random_state(g4, 5).astype(np.float32)).cuda()
+    buf = torch.empty(2 * U.numel() + 8, dtype=torch.float32, device="cuda")
+    Ua = buf[offset:offset + U.numel()].view(U.shape)
+    La = buf[U.numel() + 4 + offset:2 * U.numel() + 4 + offset].view(U.shape)
+    Ua.copy_(U)
+    a, b = ibm.Grid(g4), ibm.Grid(g8)
+    ibm.ibm_rhs(a.h, Ua.data_ptr(), La.data_ptr())
+    L8 = b.rhs(U.double())
+    torch.cuda.synchronize()
+    assert float((La.double() - L8).norm() / L8.norm()) < 1e-4
+    a.close()
+    b.close()
