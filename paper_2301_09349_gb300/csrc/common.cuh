@@ -35,13 +35,13 @@ constexpr double kHeatSourceCap = 0.9;
 // (double arithmetic runs at a small fraction of the FP32 rate on this GPU,
 // so no FP32 kernel converts or divides doubles per cell or per face).
 struct FloatConsts {
-    float gamma, inv_gm1, gm1, invR, mu_inf, S, onepS, lam_fac, inv_h, qinv_h, kvisc, E_inf;
+    float gamma, inv_gm1, gm1, invR, mu_inf, S, onepS, lam_fac, inv_h, hinv_h, qinv_h, kvisc, E_inf;
     int viscous;
-    // the 2D march's folded constants (flux_ym.cu): 2/(gamma-1),
+    // the marches' folded constants (flux_pair.cuh): 2/(gamma-1),
     // 2 + 2/(gamma-1), 2 S r, 2 mu_inf (1+S) sqrt(8)/4 r^(-1/2) / h with
     // mu = (..) T^2 rsqrt(T (T + 2 S r)^2) of the two cells' summed T = p/rho,
     // and 2 c_p / (Pr r)
-    float ym_e1, ym_h1, ym_s2, ym_km, ym_kl;
+    float e1, h1, s2, km, kl;
 };
 
 struct GridParams {
@@ -76,15 +76,16 @@ inline FloatConsts float_consts(const GridParams &g) {
     c.onepS = (float)(1.0 + g.S);
     c.lam_fac = (float)(g.cp / g.Pr);
     c.inv_h = (float)g.inv_h;
+    c.hinv_h = (float)(0.5 * g.inv_h);
     c.qinv_h = (float)(0.25 * g.inv_h);
     c.kvisc = (float)g.kvisc;
     c.E_inf = (float)(g.p_inf / (g.gamma - 1.0) + 0.5);
     c.viscous = g.mu_inf > 0.0;
-    c.ym_e1 = (float)(2.0 / (g.gamma - 1.0));
-    c.ym_h1 = (float)(2.0 + 2.0 / (g.gamma - 1.0));
-    c.ym_s2 = (float)(2.0 * g.S * g.R);
-    c.ym_km = (float)(2.0 * g.mu_inf * (1.0 + g.S) * sqrt(8.0) / 4.0 / sqrt(g.R) * g.inv_h);
-    c.ym_kl = (float)(2.0 * g.cp / (g.Pr * g.R));
+    c.e1 = (float)(2.0 / (g.gamma - 1.0));
+    c.h1 = (float)(2.0 + 2.0 / (g.gamma - 1.0));
+    c.s2 = (float)(2.0 * g.S * g.R);
+    c.km = (float)(2.0 * g.mu_inf * (1.0 + g.S) * sqrt(8.0) / 4.0 / sqrt(g.R) * g.inv_h);
+    c.kl = (float)(2.0 * g.cp / (g.Pr * g.R));
     return c;
 }
 

@@ -1,0 +1,47 @@
+// Packed FP32x2 arithmetic of the marching fluid stages (flux_ym.cu,
+// flux_zm.cu): a float2 holds the same quantity of two faces or cells, and
+// every operation is one explicit rounding (nothing is left to contraction).
+#pragma once
+
+#include "common.cuh"
+
+namespace ibmk {
+namespace {
+
+__device__ __forceinline__ float2 operator+(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 operator-(float2 a, float2 b) { return fsub2_ftz(a, b); }
+__device__ __forceinline__ float2 operator*(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 sp(float s) { return make_float2(s, s); }
+__device__ __forceinline__ float2 rcp2(float2 a) { return make_float2(rcp_ftz(a.x), rcp_ftz(a.y)); }
+__device__ __forceinline__ float2 rsqrt2(float2 a) { return make_float2(rsqrtf(a.x), rsqrtf(a.y)); }
+__device__ __forceinline__ float2 abs2(float2 a) { return make_float2(fabsf(a.x), fabsf(a.y)); }
+__device__ __forceinline__ float2 max2(float2 a, float2 b) {
+    return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y));
+}
+// products with a constant, lane by lane: a packed one would need the constant
+// twice in a register pair, which costs moves
+__device__ __forceinline__ float2 cmul(float c, float2 a) {
+    return make_float2(__fmul_rn(c, a.x), __fmul_rn(c, a.y));
+}
+__device__ __forceinline__ float2 cfma(float c, float2 a, float2 b) {
+    return make_float2(__fmaf_rn(c, a.x, b.x), __fmaf_rn(c, a.y, b.y));
+}
+__device__ __forceinline__ float2 fabs_fma(float2 a, float2 b, float2 u) {   // a b + |u|
+    return make_float2(__fmaf_rn(a.x, b.x, fabsf(u.x)), __fmaf_rn(a.y, b.y, fabsf(u.y)));
+}
+__device__ __forceinline__ float vlh1(float a, float b) {
+    const float ab = __fmul_rn(a, b);
+    const float q = __fmul_rn(ab, rcp_ftz(__fadd_rn(a, b)));
+    return ab > 0.0f ? q : 0.0f;
+}
+// half the van Leer slope, ab / (a + b) where ab > 0: the face states are
+// w +- psi/2, and the factor 2 of psi = 2ab/(a+b) and the 1/2 cancel exactly
+__device__ __forceinline__ float2 vlh2(float2 a, float2 b) {
+    const float2 ab = a * b;
+    const float2 q = ab * rcp2(a + b);
+    return make_float2(ab.x > 0.0f ? q.x : 0.0f, ab.y > 0.0f ? q.y : 0.0f);
+}
+
+}  // namespace
+}  // namespace ibmk

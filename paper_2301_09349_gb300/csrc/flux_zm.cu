@@ -23,12 +23,26 @@
 // 32-bit words of the ring, so most stencil loads are 8-byte (two cells).
 // All constants are single precision: the kernel issues no FP64 work except
 // the per-CTA step-size maximum.
+//
+// Bound: instruction issue and latency (16 warps per SM at 56 % issue; the
+// plane barriers and fixed-latency waits are the rest).  Folding the halves
+// and 1/h out of the fluxes, one special-function operation for the sound
+// speed and one for Sutherland's law, plain reciprocals, and scalar arithmetic
+// where a one-cell shift breaks the register pairs took 777 -> 710 and 892 ->
+// 838 thread instructions per cell (192^3): 256^3 533 -> 487 us (stage 1) and
+// 616 -> 575 us (stage 2).  Measured and not kept: converting pairs of cells
+// (18 x 20 of them do not divide among 256 threads: 532 us), and per-pair
+// source tables with asynchronous copies in place of the mapped loads (510
+// and 679 us, stage 2 spilling).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <float.h>
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
+
+#include "flux_pair.cuh"
 #include "internal.h"
 
 namespace ibmk {
@@ -75,96 +89,70 @@ __device__ __forceinline__ float rate_f(const FC &c, const float *u, bool &ok) {
 
 FC make_fc(const GridParams &g) { return float_consts(g); }
 
-// ---- packed pairs: two faces evaluated by one FP32x2 instruction stream ----
-__device__ __forceinline__ float2 operator+(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 operator-(float2 a, float2 b) { return fsub2_ftz(a, b); }
-__device__ __forceinline__ float2 operator*(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 sp(float s) { return make_float2(s, s); }
-__device__ __forceinline__ float2 rcp2(float2 a) {
-    return make_float2(__fdividef(1.0f, a.x), __fdividef(1.0f, a.y));
-}
-__device__ __forceinline__ float2 rsqrt2(float2 a) { return make_float2(rsqrtf(a.x), rsqrtf(a.y)); }
-__device__ __forceinline__ float2 abs2(float2 a) { return make_float2(fabsf(a.x), fabsf(a.y)); }
-__device__ __forceinline__ float2 max2(float2 a, float2 b) {
-    return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y));
-}
-// half the van Leer slope, ab / (a + b) where ab > 0: the face states are
-// w +- psi/2, and the factor 2 of psi = 2ab/(a+b) and the 1/2 cancel exactly
-__device__ __forceinline__ float2 vlh2(float2 a, float2 b) {
-    const float2 ab = a * b;
-    const float2 q = ab * rcp2(a + b);
-    return make_float2(ab.x > 0.0f ? q.x : 0.0f, ab.y > 0.0f ? q.y : 0.0f);
-}
-__device__ __forceinline__ float vlh1(float a, float b) {
-    const float ab = a * b;
-    const float q = ab * __fdividef(1.0f, a + b);
-    return ab > 0.0f ? q : 0.0f;
-}
 // two neighbouring ring cells (the first at an even index)
 __device__ __forceinline__ float2 ld2(const float *p) { return *reinterpret_cast<const float2 *>(p); }
 __device__ __forceinline__ void st2(float *p, float2 v) { *reinterpret_cast<float2 *>(p) = v; }
 
+// Fluxes are evaluated doubled (mass, momentum) and four-fold (energy), so no
+// half remains in them: the output scales by 1/(2h) and 1/(4h).
+
 // Rusanov flux of two faces from their reconstructed states in the face
-// frame (rho, u_n, u_t1, u_t2, p): F = (mass, normal momentum, t1 momentum,
-// t2 momentum, energy).
+// frame (rho, u_n, u_t1, u_t2, p): F = 2 (mass, normal momentum, t1 momentum,
+// t2 momentum), 4 energy.  The speed of sound is gamma p rsqrt(gamma p rho):
+// one special-function operation per side.
 __device__ __forceinline__ void euler_pair(const FC &c, const float2 (&wl)[NC],
                                            const float2 (&wr)[NC], float2 (&F)[NC]) {
-    const float2 keL = fma2(wl[1], wl[1], fma2(wl[2], wl[2], wl[3] * wl[3]));
-    const float2 keR = fma2(wr[1], wr[1], fma2(wr[2], wr[2], wr[3] * wr[3]));
-    const float2 EL = fma2(wl[4], sp(c.inv_gm1), sp(0.5f) * wl[0] * keL);
-    const float2 ER = fma2(wr[4], sp(c.inv_gm1), sp(0.5f) * wr[0] * keR);
     const float2 unL = wl[1], unR = wr[1];
-    const float2 c2L = sp(c.gamma) * wl[4] * rcp2(wl[0]);
-    const float2 c2R = sp(c.gamma) * wr[4] * rcp2(wr[0]);
-    const float2 sL = fma2(c2L, rsqrt2(c2L), abs2(unL));
-    const float2 sR = fma2(c2R, rsqrt2(c2R), abs2(unR));
-    const float2 hs = sp(-0.5f) * max2(sL, sR);      // -smax/2
     const float2 mLn = wl[0] * unL, mRn = wr[0] * unR;
     const float2 mL1 = wl[0] * wl[2], mR1 = wr[0] * wr[2];
     const float2 mL2 = wl[0] * wl[3], mR2 = wr[0] * wr[3];
-    F[0] = fma2(hs, wr[0] - wl[0], sp(0.5f) * (mLn + mRn));
-    F[1] = fma2(hs, mRn - mLn, sp(0.5f) * (fma2(mLn, unL, wl[4]) + fma2(mRn, unR, wr[4])));
-    F[2] = fma2(hs, mR1 - mL1, sp(0.5f) * fma2(mL1, unL, mR1 * unR));
-    F[3] = fma2(hs, mR2 - mL2, sp(0.5f) * fma2(mL2, unL, mR2 * unR));
-    F[4] = fma2(hs, ER - EL, sp(0.5f) * fma2(EL + wl[4], unL, (ER + wr[4]) * unR));
+    const float2 rkL = fma2(mLn, unL, fma2(mL1, wl[2], mL2 * wl[3]));   // rho |u|^2
+    const float2 rkR = fma2(mRn, unR, fma2(mR1, wr[2], mR2 * wr[3]));
+    const float2 gpL = cmul(c.gamma, wl[4]), gpR = cmul(c.gamma, wr[4]);
+    const float2 sL = fabs_fma(gpL, rsqrt2(gpL * wl[0]), unL);
+    const float2 sR = fabs_fma(gpR, rsqrt2(gpR * wr[0]), unR);
+    const float2 sm = max2(sL, sR);
+    F[0] = fma2(sm, wl[0] - wr[0], mLn + mRn);
+    F[1] = fma2(sm, mLn - mRn, fma2(mLn, unL, wl[4]) + fma2(mRn, unR, wr[4]));
+    F[2] = fma2(sm, mL1 - mR1, fma2(mL1, unL, mR1 * unR));
+    F[3] = fma2(sm, mL2 - mR2, fma2(mL2, unL, mR2 * unR));
+    const float2 HL = cfma(c.h1, wl[4], rkL), HR = cfma(c.h1, wr[4], rkR);   // 2 rho H
+    const float2 EL = cfma(c.e1, wl[4], rkL), ER = cfma(c.e1, wr[4], rkR);   // 2 rho E
+    F[4] = fma2(sm, EL - ER, fma2(HL, unL, HR * unR));
 }
 
 // Viscous stress and heat flux of two faces, subtracted from F (face frame).
-// Cell values of the velocity components (n, t1, t2) and T on the two sides
-// a and b; d1n, d11: the sums over the two cells of the central differences
-// (w[+1] - w[-1], unscaled) of u_n and u_t1 along t1; d2n, d22: of u_n and
-// u_t2 along t2.  Tangential derivatives are those sums / (4h) (reading 11).
-__device__ __forceinline__ void visc_pair(const FC &c, float2 na, float2 nb, float2 t1a,
-                                          float2 t1b, float2 t2a, float2 t2b, float2 Ta,
-                                          float2 Tb, float2 d1n, float2 d11, float2 d2n,
-                                          float2 d22, float2 (&F)[NC]) {
-    const float2 Tf = sp(0.5f) * (Ta + Tb);
-    const float2 mu = sp(c.mu_inf * c.onepS) * Tf * (Tf * rsqrt2(Tf)) * rcp2(Tf + sp(c.S));
-    const float2 lam = mu * sp(c.lam_fac);
-    const float2 ih = sp(c.inv_h), qh = sp(c.qinv_h);
-    const float2 dn_n = (nb - na) * ih;
-    const float2 dn_1 = (t1b - t1a) * ih;
-    const float2 dn_2 = (t2b - t2a) * ih;
-    const float2 dn_T = (Tb - Ta) * ih;
-    const float2 div = fma2(d11 + d22, qh, dn_n);
-    const float2 tNN = mu * fma2(sp(2.0f), dn_n, sp(-2.0f / 3.0f) * div);
-    const float2 tN1 = mu * fma2(d1n, qh, dn_1);
-    const float2 tN2 = mu * fma2(d2n, qh, dn_2);
-    const float2 ufn = sp(0.5f) * (na + nb);
-    const float2 uf1 = sp(0.5f) * (t1a + t1b);
-    const float2 uf2 = sp(0.5f) * (t2a + t2b);
+// dn, d1, d2, dT: differences (upper - lower cell) and sn, s1, s2, sT sums of
+// u_n, u_t1, u_t2 and T = p / rho over the two cells; d1n, d11: the sums over
+// the two cells of the central differences (w[+1] - w[-1], unscaled) of u_n
+// and u_t1 along t1; d2n, d22: of u_n and u_t2 along t2.  Tangential
+// derivatives are those sums / (4h) (reading 11).  T^(3/2) / (T + S) is
+// T^2 rsqrt(T (T + S)^2).
+__device__ __forceinline__ void visc_pair(const FC &c, float2 dn, float2 d1, float2 d2, float2 dT,
+                                          float2 sn, float2 s1, float2 s2, float2 sT, float2 d1n,
+                                          float2 d11, float2 d2n, float2 d22, float2 (&F)[NC]) {
+    const float2 y = make_float2(__fadd_rn(sT.x, c.s2), __fadd_rn(sT.y, c.s2));
+    const float2 m = cmul(c.km, sT) * (sT * rsqrt2(sT * y * y));   // 2 mu / h
+    const float2 tNN = m * cfma(4.0f / 3.0f, dn, cmul(-1.0f / 6.0f, d11 + d22));
+    const float2 tN1 = m * cfma(0.25f, d1n, d1);
+    const float2 tN2 = m * cfma(0.25f, d2n, d2);
     F[1] = F[1] - tNN;
     F[2] = F[2] - tN1;
     F[3] = F[3] - tN2;
-    F[4] = F[4] - fma2(ufn, tNN, fma2(uf1, tN1, fma2(uf2, tN2, lam * dn_T)));
+    F[4] = F[4] - fma2(sn, tNN, fma2(s1, tN1, fma2(s2, tN2, cmul(c.kl, m) * dT)));
+}
+// from the cell values a (lower) and b (upper) of (n, t1, t2) and T
+__device__ __forceinline__ void visc_cells(const FC &c, const float2 (&ca)[NC],
+                                           const float2 (&cb)[NC], float2 Ta, float2 Tb, float2 d1n,
+                                           float2 d11, float2 d2n, float2 d22, float2 (&F)[NC]) {
+    visc_pair(c, cb[1] - ca[1], cb[2] - ca[2], cb[3] - ca[3], Tb - Ta, ca[1] + cb[1], ca[2] + cb[2],
+              ca[3] + cb[3], Ta + Tb, d1n, d11, d2n, d22, F);
 }
 
 // central differences (unscaled) along x of a field at cells 2t, 2t+1 of one
-// row: w[x+1] - w[x-1] from the pairs at x-2, x (given) and x+2
+// row: w[x+1] - w[x-1] from the pair (given) and its neighbours
 __device__ __forceinline__ float2 cdx2(const float *f, float2 mid) {
-    const float2 lo = ld2(f - 2), hi = ld2(f + 2);
-    return make_float2(mid.y, hi.x) - make_float2(lo.y, mid.x);
+    return make_float2(__fsub_rn(mid.y, f[-1]), __fsub_rn(f[2], mid.x));
 }
 
 // x-faces 2t-1/2 (.x) and 2t+1/2 (.y) of one row; b: ring index of cell 2t
@@ -173,45 +161,43 @@ __device__ __forceinline__ float2 cdx2(const float *f, float2 mid) {
 __device__ __forceinline__ void x_pair(const FC &c, const float *__restrict__ R, int b, int up,
                                        int dn, float2 (&F)[NC]) {
     float2 wl[NC], wr[NC];
-    float2 va[3], vb[3];     // u, v, w on the a side (cells 2t-1, 2t) and b side (2t, 2t+1)
+    float2 df[3], sm[3];     // differences and sums of u, v, w over each face's cells
+    // The five cells 2t-2 .. 2t+2 and their three slopes; formed lane by lane,
+    // since values shifted by one cell do not line up with register pairs
 #pragma unroll
     for (int m = 0; m < NC; ++m) {
         const float *f = R + m * PP + b;
         const float2 lo = ld2(f - 2), mid = ld2(f);
         const float w2 = f[2];
-        const float2 dA = make_float2(lo.y, mid.y) - make_float2(lo.x, mid.x);   // d(-3/2), d(1/2)
-        const float2 dB = make_float2(mid.x, w2) - make_float2(lo.y, mid.y);     // d(-1/2), d(3/2)
-        const float2 so = vlh2(dA, dB);                                          // slopes of 2t-1, 2t+1
-        const float s0 = vlh1(dB.x, dA.y);                                       // slope of 2t
-        wl[m] = make_float2(lo.y, mid.x) + make_float2(so.x, s0);
-        wr[m] = mid - make_float2(s0, so.y);
+        const float d0 = __fsub_rn(lo.y, lo.x), d1 = __fsub_rn(mid.x, lo.y),
+                    d2 = __fsub_rn(mid.y, mid.x), d3 = __fsub_rn(w2, mid.y);
+        const float sa = vlh1(d0, d1), sb = vlh1(d1, d2), sc = vlh1(d2, d3);
+        wl[m] = make_float2(__fadd_rn(lo.y, sa), __fadd_rn(mid.x, sb));
+        wr[m] = make_float2(__fsub_rn(mid.x, sb), __fsub_rn(mid.y, sc));
         if (m >= 1 && m <= 3) {
-            va[m - 1] = make_float2(lo.y, mid.x);
-            vb[m - 1] = mid;
+            df[m - 1] = make_float2(d1, d2);
+            sm[m - 1] = make_float2(__fadd_rn(lo.y, mid.x), __fadd_rn(mid.x, mid.y));
         }
     }
     euler_pair(c, wl, wr, F);
     if (!c.viscous) return;
     const float *T = R + 5 * PP + b;
-    const float2 Tmid = ld2(T);
-    const float2 Ta = make_float2(T[-1], Tmid.x), Tb = Tmid;
-    // central differences of cells 2t-1, 2t, 2t+1 along an axis of stride o
-    // (o = PX: y) summed pairwise per face
-    auto cd = [&](const float *f, int o) {
-        const float cm = f[o - 1] - f[-o - 1];
-        const float2 c01 = ld2(f + o) - ld2(f - o);
-        return make_float2(cm, c01.x) + c01;
+    const float2 Tm = ld2(T);
+    const float tl = T[-1];
+    const float2 dT = make_float2(__fsub_rn(Tm.x, tl), __fsub_rn(Tm.y, Tm.x));
+    const float2 sT = make_float2(__fadd_rn(tl, Tm.x), __fadd_rn(Tm.x, Tm.y));
+    // central differences of cells 2t-1, 2t, 2t+1 between the offsets hi and
+    // lo, summed pairwise per face
+    auto cd = [&](const float *f, int hi, int lo) {
+        const float cm = __fsub_rn(f[hi - 1], f[lo - 1]);
+        const float2 c01 = ld2(f + hi) - ld2(f + lo);
+        return make_float2(__fadd_rn(cm, c01.x), __fadd_rn(c01.x, c01.y));
     };
     const float *U = R + PP + b, *V = R + 2 * PP + b, *W = R + 3 * PP + b;
-    const float2 d1n = cd(U, PX), d11 = cd(V, PX);   // along y: u (normal), v (t1)
-    // along z (planes above and below): u (normal) and w (t2)
-    const float um = U[up - 1] - U[dn - 1];
-    const float2 u01 = ld2(U + up) - ld2(U + dn);
-    const float wm = W[up - 1] - W[dn - 1];
-    const float2 w01 = ld2(W + up) - ld2(W + dn);
-    const float2 d2n = make_float2(um, u01.x) + u01;
-    const float2 d22 = make_float2(wm, w01.x) + w01;
-    visc_pair(c, va[0], vb[0], va[1], vb[1], va[2], vb[2], Ta, Tb, d1n, d11, d2n, d22, F);
+    // along y: u (normal), v (t1); along z: u (normal) and w (t2)
+    const float2 d1n = cd(U, PX, -PX), d11 = cd(V, PX, -PX);
+    const float2 d2n = cd(U, up, dn), d22 = cd(W, up, dn);
+    visc_pair(c, df[0], df[1], df[2], dT, sm[0], sm[1], sm[2], sT, d1n, d11, d2n, d22, F);
 }
 
 // y-faces at row r-1/2 of cells 2t (.x) and 2t+1 (.y); b: ring index of cell
@@ -242,7 +228,7 @@ __device__ __forceinline__ void y_pair(const FC &c, const float *__restrict__ R,
         // along z: v (normal) and w (t2)
         const float2 d2n = (ld2(V - PX + up) - ld2(V - PX + dn)) + (ld2(V + up) - ld2(V + dn));
         const float2 d22 = (ld2(W - PX + up) - ld2(W - PX + dn)) + (ld2(W + up) - ld2(W + dn));
-        visc_pair(c, ca[1], cb[1], ca[2], cb[2], ca[3], cb[3], Ta, Tb, d1n, d11, d2n, d22, F);
+        visc_cells(c, ca, cb, Ta, Tb, d1n, d11, d2n, d22, F);
     }
     Fo[0] = F[0]; Fo[1] = F[2]; Fo[2] = F[1]; Fo[3] = F[3]; Fo[4] = F[4];
 }
@@ -288,7 +274,7 @@ __device__ __forceinline__ void z_pair(const FC &c, const float *__restrict__ ri
                            (ld2(B + 3 * PP + PX) - ld2(B + 3 * PP - PX));
         const float2 d22 = (ld2(A + 2 * PP + PX) - ld2(A + 2 * PP - PX)) +
                            (ld2(B + 2 * PP + PX) - ld2(B + 2 * PP - PX));
-        visc_pair(c, ca[1], cb[1], ca[2], cb[2], ca[3], cb[3], Ta, Tb, d1n, d11, d2n, d22, F);
+        visc_cells(c, ca, cb, Ta, Tb, d1n, d11, d2n, d22, F);
     }
     Fo[0] = F[0]; Fo[1] = F[2]; Fo[2] = F[3]; Fo[3] = F[1]; Fo[4] = F[4];
 }
@@ -332,7 +318,7 @@ __device__ __forceinline__ void edge_pair(const FC &c, const float *__restrict__
         };
         const float2 d1n = cd(NA, NB, st, -st), d11 = cd(PA, PB, st, -st);
         const float2 d2n = cd(NA, NB, up, dn), d22 = cd(WA, WB, up, dn);
-        visc_pair(c, ca[1], cb[1], ca[2], cb[2], ca[3], cb[3], Ta, Tb, d1n, d11, d2n, d22, F);
+        visc_cells(c, ca, cb, Ta, Tb, d1n, d11, d2n, d22, F);
     }
     // back to lab order: the normal momentum goes to u (x-face) or v (y-face)
     const bool xf = nf == 1;
@@ -378,11 +364,11 @@ __device__ __forceinline__ bool tma_wait(unsigned mbar, unsigned parity, int *er
     return false;
 }
 
-// primitives (rho, u, v, w, p, T) of one conserved cell into ring cell q
+// primitives (rho, u, v, w, p, T = p / rho) of one conserved cell into ring cell q
 __device__ __forceinline__ void to_primitive(const FC &c, const float (&u)[NC],
                                              float *__restrict__ slot, int q) {
     const float rho = u[0];
-    const float inv = __fdividef(1.0f, rho);
+    const float inv = rcp_ftz(rho);
     const float vx = u[1] * inv, vy = u[2] * inv, vz = u[3] * inv;
     const float p = c.gm1 * (u[4] - 0.5f * rho * (vx * vx + vy * vy + vz * vz));
     slot[q] = rho;
@@ -390,7 +376,7 @@ __device__ __forceinline__ void to_primitive(const FC &c, const float (&u)[NC],
     slot[2 * PP + q] = vy;
     slot[3 * PP + q] = vz;
     slot[4 * PP + q] = p;
-    slot[5 * PP + q] = p * inv * c.invR;
+    slot[5 * PP + q] = p * inv;
 }
 
 // conserved state of a ghost or interior cell through the boundary maps
@@ -643,8 +629,9 @@ zmarch_kernel(const __grid_constant__ CUtensorMap tmap, const GridParams g, cons
             // x-face right of cell 2t+1: the neighbour's first face, or the edge
             float fr = __shfl_down_sync(0xffffffffu, Fx[m].x, 1);
             if (t == 15) fr = FXe[m * TY + r];
+            const float2 dx = make_float2(__fsub_rn(Fx[m].x, Fx[m].y), __fsub_rn(Fx[m].y, fr));
             const float2 Fyu = ld2(FY + (m * (TY + 1) + r + 1) * TX + 2 * t);
-            acc[m] = ((Fx[m] - make_float2(Fx[m].y, fr)) + (Fy[m] - Fyu)) + (Fzl[m] - Fzh[m]);
+            acc[m] = cmul(m == NC - 1 ? c.qinv_h : c.hinv_h, (dx + (Fy[m] - Fyu)) + (Fzl[m] - Fzh[m]));
             Fzl[m] = Fzh[m];
         }
         // output operands of the two cells: U^n (stage 2) is issued now and
@@ -674,7 +661,6 @@ zmarch_kernel(const __grid_constant__ CUtensorMap tmap, const GridParams g, cons
         }
 
         if (in0 && in_bounds(j + (vec ? 1 : 0), N, err)) {
-            const float2 ih = sp(c.inv_h), dt2 = sp(dt);
             // the input state at the two cells, rebuilt from the primitives
             // of plane z in the ring (a few FP32 roundings from the stored
             // values; saves holding them in registers across the conversion).
@@ -688,22 +674,22 @@ zmarch_kernel(const __grid_constant__ CUtensorMap tmap, const GridParams g, cons
                 u[1] = rh * vu;
                 u[2] = rh * vv;
                 u[3] = rh * vw;
-                u[4] = fma2(pr, sp(c.inv_gm1), sp(0.5f) * rh * ke);
+                u[4] = cfma(c.inv_gm1, pr, cmul(0.5f, rh) * ke);
             };
             if (vec) {
                 if (MODE != 0) u_from_ring(o1);
                 if (MODE == 0) {
 #pragma unroll
-                    for (int m = 0; m < NC; ++m) st2(out + m * N + j, acc[m] * ih);
+                    for (int m = 0; m < NC; ++m) st2(out + m * N + j, acc[m]);
                 } else if (MODE == 1) {
 #pragma unroll
-                    for (int m = 0; m < NC; ++m) st2(out + m * N + j, fma2(dt2, acc[m] * ih, o1[m]));
+                    for (int m = 0; m < NC; ++m) st2(out + m * N + j, cfma(dt, acc[m], o1[m]));
                 } else {
                     float ua[NC], ub[NC];
 #pragma unroll
                     for (int m = 0; m < NC; ++m) {
                         const float2 us =
-                            fma2(sp(0.5f), o2[m], sp(0.5f) * fma2(dt2, acc[m] * ih, o1[m]));
+                            cfma(0.5f, o2[m], cmul(0.5f, cfma(dt, acc[m], o1[m])));
                         st2(out + m * N + j, us);
                         ua[m] = us.x;
                         ub[m] = us.y;
@@ -719,7 +705,7 @@ zmarch_kernel(const __grid_constant__ CUtensorMap tmap, const GridParams g, cons
                     float us[NC];
 #pragma unroll
                     for (int m = 0; m < NC; ++m) {
-                        const float a = (k == 0 ? acc[m].x : acc[m].y) * c.inv_h;
+                        const float a = k == 0 ? acc[m].x : acc[m].y;
                         if (MODE == 0) {
                             out[m * N + jk] = a;
                         } else if (MODE == 1) {
@@ -764,23 +750,36 @@ zmarch_kernel(const __grid_constant__ CUtensorMap tmap, const GridParams g, cons
 
 }  // namespace
 
-#ifndef IBM_ZM_WAVES
-#define IBM_ZM_WAVES 3
-#endif
-#ifndef IBM_ZM_CHUNK
-#define IBM_ZM_CHUNK 19
-#endif
-
+// Planes per CTA.  A chunk of zc planes costs about zc + 2.5 plane times (its
+// four-plane prologue, the z-faces below it), and the grid runs in waves of
+// two CTAs per SM, so the chunk count k is the one with the least
+// waves(k) * (zc + 2.5); a grid of at most one CTA per SM runs each of them
+// in ~0.6 of the time.  At most ZM_CHUNK_MAX planes: the tiles at the domain's
+// edge take longer, and short chunks even that out (256^3, both stages: 19
+// planes 1062 us, 37 planes, three full waves, 1080).  The former rule halved
+// 19-plane chunks until there were three waves, which left four planes per
+// chunk below ~150^3 and doubled the work: 131 x 97 x 113 237 -> 202 us for
+// both stages, 96^3 118 -> 88, 48^3 (L alone) 26 -> 18, 128^3 (L alone) 101 ->
+// 82.
+constexpr int ZM_CHUNK_MAX = 24;
 int zmarch_chunk(const GridParams &g) {
-    // planes per CTA: enough CTAs to fill the GPU several times over (two
-    // resident per SM).  At 256^3 (bench, ms per step): 16: 1.236, 19:
-    // 1.220, 21: 1.251, 24: 1.227, 32: 1.27 - the wave count of the grid
-    // (128 columns x 14 chunks = 5.9 waves at 19) matters as much as the
-    // four-plane prologue of each chunk
     const long long cols = (long long)((g.n[0] + TX - 1) / TX) * ((g.n[1] + TY - 1) / TY);
-    int zc = IBM_ZM_CHUNK;
-    while (zc > 4 && cols * ((g.n[2] + zc - 1) / zc) < IBM_ZM_WAVES * 2 * 152) zc /= 2;
-    return zc;
+    const long long slots = 2 * 152;
+    const int kmin = (g.n[2] + ZM_CHUNK_MAX - 1) / ZM_CHUNK_MAX;
+    const long long most = std::max<long long>(kmin, 8 * slots / cols + 1);
+    const int kmax = (int)std::min<long long>(most, g.n[2]);
+    int best = 1;
+    double cost = 1e300;
+    for (int k = kmin; k <= kmax; ++k) {
+        const int zc = (g.n[2] + k - 1) / k;
+        const long long ctas = cols * ((g.n[2] + zc - 1) / zc);
+        const double c = (double)((ctas + slots - 1) / slots) * (zc + 2.5) * (2 * ctas <= slots ? 0.6 : 1.0);
+        if (c < cost) {
+            cost = c;
+            best = zc;
+        }
+    }
+    return best;
 }
 
 size_t zmarch_blocks(const GridParams &g) {
