@@ -103,6 +103,7 @@ GridParams make_params(const ibm_grid_desc &d) {
     g.energy_reading = d.energy_reading;
     g.forcing_per_stage = d.forcing_per_stage;
     g.f = float_consts(g);
+    g.d = double_consts(g);
     return g;
 }
 

@@ -44,6 +44,17 @@ struct FloatConsts {
     float e1, h1, s2, km, kl;
 };
 
+// The same folded constants for the FP64 kernels: a division costs an FP64
+// kernel ten operations of a pipe that retires two per SM cycle, so none is
+// left to the device.
+struct DoubleConsts {
+    double e1, h1, s2, km, kl;     // as in FloatConsts
+    double hinv_h, qinv_h;         // 1/(2h), 1/(4h)
+    double E_inf;                  // free-stream rho E
+    double ks, kn;                 // step-size rate: (2 dim) kvisc / h^2 and mu_inf (1 + S) r^(-1/2)
+                                   // with mu = kn T^2 rsqrt(T (T + S r)^2), T = p / rho
+};
+
 struct GridParams {
     int dim;
     int n[3];
@@ -63,6 +74,7 @@ struct GridParams {
     int energy_reading;
     int forcing_per_stage;
     FloatConsts f;        // FP32 copies of the constants above
+    DoubleConsts d;
 };
 
 inline FloatConsts float_consts(const GridParams &g) {
@@ -87,6 +99,46 @@ inline FloatConsts float_consts(const GridParams &g) {
     c.km = (float)(2.0 * g.mu_inf * (1.0 + g.S) * sqrt(8.0) / 4.0 / sqrt(g.R) * g.inv_h);
     c.kl = (float)(2.0 * g.cp / (g.Pr * g.R));
     return c;
+}
+
+inline DoubleConsts double_consts(const GridParams &g) {
+    DoubleConsts c;
+    c.e1 = 2.0 / (g.gamma - 1.0);
+    c.h1 = 2.0 + 2.0 / (g.gamma - 1.0);
+    c.s2 = 2.0 * g.S * g.R;
+    c.km = 2.0 * g.mu_inf * (1.0 + g.S) * sqrt(8.0) / 4.0 / sqrt(g.R) * g.inv_h;
+    c.kl = 2.0 * g.cp / (g.Pr * g.R);
+    c.hinv_h = 0.5 * g.inv_h;
+    c.qinv_h = 0.25 * g.inv_h;
+    c.E_inf = g.p_inf / (g.gamma - 1.0) + 0.5;
+    c.ks = 2.0 * g.dim * g.kvisc * g.inv_h * g.inv_h;
+    c.kn = g.mu_inf * (1.0 + g.S) / sqrt(g.R);
+    return c;
+}
+
+// 1/x and 1/sqrt(x) in FP64 from the hardware seeds (a relative error e below
+// 2^-18) by one step of the third-order Householder iteration, whose error is
+// e^3 plus rounding: r (1 + e + e^2) with e = 1 - x r, and y (1 + e/2 + 3 e^2/8)
+// with e = 1 - x y^2.  Within 2 ulp for positive normal x (the kernels divide
+// by densities, pressures and sums of their differences); four and six
+// operations against ten and more of an IEEE division or square root, on a
+// pipe of two operations per SM cycle.
+__device__ __forceinline__ double drcp(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(fma(e, e, e), r, r);
+}
+__device__ __forceinline__ double drsqrt(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-__dmul_rn(x, y), y, 1.0);
+    return fma(__dmul_rn(y, e), fma(0.375, e, 0.5), y);
+}
+// x > 0 by the sign and magnitude bits (integer instructions; NaN counts as
+// positive and propagates through what is computed for it)
+__device__ __forceinline__ bool dpos(double x) {
+    return (unsigned)(__double2hiint(x) - 1) < 0x7fffffffu - 1u;
 }
 
 // The 1D regularised 3-point delta of Sec. 2.2 (Pinelli et al.); r in cells.

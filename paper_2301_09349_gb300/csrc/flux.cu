@@ -10,20 +10,24 @@
 // with dt = cfl / max_j s_j(U^n), formed at the end of the previous step (or
 // by dt_init after a new state) so that stage 1 can write U^1 directly.
 //
-// Each CTA owns a BX x BY x BZ tile of cells.  It loads the tile plus a
-// two-cell halo once (ghost cells mapped through the boundary conditions on
-// the fly), converts to primitives in shared memory, then evaluates every
-// face of the tile exactly once per direction into a shared face buffer and
+// Here: FP64 grids (FP32 grids march: flux_zm.cu, flux_ym.cu).  Each CTA owns
+// a BX x BY x BZ tile of cells.  It loads the tile plus a two-cell halo once
+// (ghost cells mapped through the boundary conditions on the fly), converts
+// to primitives in shared memory, then per direction evaluates every limited
+// slope once and every face of the tile once into shared buffers and
 // accumulates the flux differences in registers.
+//
+// Bound: the FP64 pipe (two operations per SM cycle).  What is kept small is
+// their number: no division or IEEE square root (drcp, drsqrt), slopes once
+// per cell, constants folded on the host, signs and maxima by integer
+// instructions.  Stages 1 / 2: 128 x 64 24.0 -> 13.1 and 29.0 -> 15.2 us, 64^3
+// 629 -> 346 and 710 -> 373 us.
 #include <atomic>
 #include <float.h>
 
 #include <type_traits>
 
 #include "internal.h"
-
-// the pair tiles leave some of BoxT's stride constants unused
-#pragma nv_diag_suppress 177
 
 namespace ibmk {
 namespace {
@@ -33,14 +37,14 @@ constexpr int NT = 256;
 constexpr int cmax(int a, int b) { return a > b ? a : b; }
 
 // A BX x BY x BZ tile of cells with its two-cell halo, 256 threads.
-template <int DIM_, typename T, int BX_, int BY_, int BZ_>
+template <int DIM_, int BX_, int BY_, int BZ_>
 struct BoxT {
     static constexpr int DIM = DIM_;
     static constexpr int BX = BX_, BY = BY_, BZ = DIM_ == 3 ? BZ_ : 1;
     static constexpr int PX = BX + 4, PY = BY + 4, PZ = DIM == 3 ? BZ + 4 : 1;
     static constexpr int PN = PX * PY * PZ;          // cells in tile + halo
     static constexpr int NC = DIM + 2;               // conserved components
-    static constexpr int NW = DIM + 3;               // rho, u.., p, T
+    static constexpr int NW = DIM + 3;               // rho, u.., p, T = p / rho
     static constexpr int SX = 1, SY = PX, SZ = PX * PY;
     static constexpr int NCELL = BX * BY * BZ;
     static constexpr int CPT = (NCELL + NT - 1) / NT;
@@ -48,171 +52,156 @@ struct BoxT {
     static constexpr int NF1 = BX * (BY + 1) * BZ;
     static constexpr int NF2 = DIM == 3 ? BX * BY * (BZ + 1) : 0;
     static constexpr int NFMAX = cmax(NF0, cmax(NF1, NF2));
-    static constexpr size_t SMEM = sizeof(T) * (size_t)(NW * PN + NC * NFMAX);
+    // cells whose slope along an axis is needed: one more at either end
+    static constexpr int NS0 = (BX + 2) * BY * BZ;
+    static constexpr int NS1 = BX * (BY + 2) * BZ;
+    static constexpr int NS2 = DIM == 3 ? BX * BY * (BZ + 2) : 0;
+    static constexpr int NSMAX = cmax(NS0, cmax(NS1, NS2));
+    static constexpr size_t SMEM = sizeof(double) * (size_t)(NW * PN + NC * (NFMAX + NSMAX));
 };
 
 // Tile of the single-grid kernels.
-template <int DIM, typename T> struct DefaultBox;
-template <> struct DefaultBox<3, double> { using type = BoxT<3, double, 8, 8, 4>; };
-template <> struct DefaultBox<2, double> { using type = BoxT<2, double, 16, 16, 1>; };
-template <int DIM, typename T> using Box = typename DefaultBox<DIM, T>::type;
+template <int DIM> struct DefaultBox;
+template <> struct DefaultBox<3> { using type = BoxT<3, 8, 8, 4>; };
+template <> struct DefaultBox<2> { using type = BoxT<2, 16, 16, 1>; };
 
 // Small 2D FP64 grids: FP64 arithmetic runs at a small fraction of the FP32
 // rate on this GPU, so the stage time of a grid with few 16 x 16 tiles is set
 // by how many SMs take part; 8 x 8 tiles spread it over four times as many.
-using SmallBox2D = BoxT<2, double, 8, 8, 1>;
+using SmallBox2D = BoxT<2, 8, 8, 1>;
 inline bool small_2d_fp64(const GridParams &g) {
     return g.dim == 2 && (long long)((g.n[0] + 15) / 16) * ((g.n[1] + 15) / 16) < 256;
 }
-template <int DIM, typename T, bool SMALL>
-using StageBox = typename std::conditional<SMALL, SmallBox2D, Box<DIM, T>>::type;
+template <int DIM, bool SMALL>
+using StageBox = typename std::conditional<SMALL, SmallBox2D, typename DefaultBox<DIM>::type>::type;
 
 // 2D tile shapes of the batched kernel (all 256 cells): the autotuner's
 // choices.  Every face is evaluated by the same arithmetic whatever the
 // tile, so the shape changes the speed, never the result.
-template <typename T, int S> struct Shape2;
-template <typename T> struct Shape2<T, 0> { using type = BoxT<2, T, 16, 16, 1>; };
-template <typename T> struct Shape2<T, 1> { using type = BoxT<2, T, 32, 8, 1>; };
-template <typename T> struct Shape2<T, 2> { using type = BoxT<2, T, 64, 4, 1>; };
-template <typename T> struct Shape2<T, 3> { using type = BoxT<2, T, 8, 32, 1>; };
+template <int S> struct Shape2;
+template <> struct Shape2<0> { using type = BoxT<2, 16, 16, 1>; };
+template <> struct Shape2<1> { using type = BoxT<2, 32, 8, 1>; };
+template <> struct Shape2<2> { using type = BoxT<2, 64, 4, 1>; };
+template <> struct Shape2<3> { using type = BoxT<2, 8, 32, 1>; };
 
-// Arithmetic helpers.  FP32 uses the hardware approximations (MUFU
-// reciprocal / reciprocal square root, ~2 ulp), which are far inside the
-// FP32 parity tolerance; FP64 keeps correctly rounded division and sqrt.
-template <typename T> __device__ __forceinline__ T fdiv(T a, T b);
-template <> __device__ __forceinline__ float fdiv<float>(float a, float b) { return __fdividef(a, b); }
-template <> __device__ __forceinline__ double fdiv<double>(double a, double b) { return a / b; }
+// explicit roundings: no kernel's bits depend on what the compiler contracts
+__device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double sub(double a, double b) { return __dsub_rn(a, b); }
 
-// sqrt of a positive argument
-template <typename T> __device__ __forceinline__ T psqrt(T x);
-template <> __device__ __forceinline__ float psqrt<float>(float x) { return x * rsqrtf(x); }
-template <> __device__ __forceinline__ double psqrt<double>(double x) { return sqrt(x); }
-
-template <typename T>
-__device__ __forceinline__ T van_leer(T a, T b) {
-    T ab = a * b;
-    return ab > T(0) ? fdiv<T>(T(2) * ab, a + b) : T(0);
+// Half the limited slopes along axis D, ab / (a + b) where ab > 0 (the states
+// are w +- psi/2, psi = 2ab/(a+b)), of (rho, u.., p) of the tile's cells and
+// one more at either end: one work item per value, so that even a small tile
+// keeps every scheduler's FP64 pipe busy.  Each slope serves the two faces of
+// its cell.
+template <typename B, int D>
+__device__ __forceinline__ void slope_pass(const double *__restrict__ sW, double *__restrict__ sS) {
+    constexpr int DIM = B::DIM;
+    constexpr int EX = B::BX + 2 * (D == 0), EY = B::BY + 2 * (D == 1),
+                  EZ = B::BZ + 2 * (D == 2 && DIM == 3);
+    constexpr int NS = EX * EY * EZ;
+    constexpr int s = D == 0 ? B::SX : (D == 1 ? B::SY : B::SZ);
+    for (int i = threadIdx.x; i < NS * B::NC; i += NT) {
+        const int m = i / NS, q = i - m * NS;
+        const int x = q % EX, r = q / EX, y = r % EY, z = r / EY;
+        const int a = (x + 2 - (D == 0)) + B::PX * (y + 2 - (D == 1)) +
+                      (DIM == 3 ? B::PX * B::PY * (z + 2 - (D == 2)) : 0);
+        const double *w = sW + m * B::PN + a;
+        const double d0 = sub(w[0], w[-s]), d1 = sub(w[s], w[0]);
+        const double ab = mul(d0, d1);
+        const double h = mul(ab, drcp(add(d0, d1)));
+        sS[i] = dpos(ab) ? h : 0.0;
+    }
 }
 
-// The constants of the face flux in the compute type: FP32 kernels read the
-// host-rounded copies, FP64 kernels the doubles (same values either way as
-// converting in the kernel).
-template <typename T> struct FluxK;
-template <> struct FluxK<float> {
-    float gam, inv_gm1, inv_h, S, mu_inf, lam_fac, gm1, invR, E_inf;
-    bool viscous;
-    __device__ __forceinline__ explicit FluxK(const GridParams &g)
-        : gam(g.f.gamma), inv_gm1(g.f.inv_gm1), inv_h(g.f.inv_h), S(g.f.S), mu_inf(g.f.mu_inf),
-          lam_fac(g.f.lam_fac), gm1(g.f.gm1), invR(g.f.invR), E_inf(g.f.E_inf),
-          viscous(g.f.viscous != 0) {}
-};
-template <> struct FluxK<double> {
-    double gam, inv_gm1, inv_h, S, mu_inf, lam_fac, gm1, invR, E_inf;
-    bool viscous;
-    __device__ __forceinline__ explicit FluxK(const GridParams &g)
-        : gam(g.gamma), inv_gm1(1.0 / (g.gamma - 1.0)), inv_h(g.inv_h), S(g.S), mu_inf(g.mu_inf),
-          lam_fac(g.cp / g.Pr), gm1(g.gamma - 1.0), invR(1.0 / g.R),
-          E_inf(g.p_inf / (g.gamma - 1.0) + 0.5), viscous(g.mu_inf > 0.0) {}
-};
-
-// Numerical flux through the face between box cells a and a + s_D.
-template <typename B, typename T, int D>
-__device__ __forceinline__ void face_flux(const FluxK<T> &k, const T *__restrict__ sW, int a,
-                                          T (&F)[B::DIM + 2]) {
+// Numerical flux through the face between box cells a and a + s_D, doubled
+// (mass, momentum) and four-fold (energy); h0, h1: its cells' entries in the
+// slope buffer.  ~110 FP64 operations in 3D where the form with divisions,
+// both slopes per face and IEEE square roots took ~340.
+template <typename B, int D>
+__device__ __forceinline__ void face_flux(const GridParams &g, const double *__restrict__ sW, int a,
+                                          const double *__restrict__ h, int hs, int ns,
+                                          double (&F)[B::DIM + 2]) {
     constexpr int DIM = B::DIM;
-    constexpr int s = D == 0 ? B::SX : (D == 1 ? B::SY : B::SZ);
     constexpr int NC = DIM + 2;
+    constexpr int s = D == 0 ? B::SX : (D == 1 ? B::SY : B::SZ);
+    const DoubleConsts &k = g.d;
     const int b = a + s;
-    const T gam = k.gam;
-    const T inv_gm1 = k.inv_gm1;
-
-    // MUSCL reconstruction of (rho, u.., p) with the van Leer limiter
-    T wl[NC], wr[NC];
+    double wl[NC], wr[NC];
 #pragma unroll
     for (int m = 0; m < NC; ++m) {
-        const T *w = sW + m * B::PN;
-        T wam = w[a - s], wa = w[a], wb = w[b], wbp = w[b + s];
-        T d0 = wa - wam, d1 = wb - wa, d2 = wbp - wb;
-        wl[m] = wa + T(0.5) * van_leer(d0, d1);
-        wr[m] = wb - T(0.5) * van_leer(d1, d2);
+        wl[m] = add(sW[m * B::PN + a], h[m * ns]);
+        wr[m] = sub(sW[m * B::PN + b], h[m * ns + hs]);
     }
-
-    // Rusanov flux: (F_L + F_R)/2 - s_max (U_R - U_L)/2
-    T keL = 0, keR = 0;
+    // Rusanov; the speed of sound is gamma p / sqrt(gamma p rho)
+    const double unL = wl[1 + D], unR = wr[1 + D], pL = wl[NC - 1], pR = wr[NC - 1];
+    double mL[DIM], mR[DIM], rkL = 0.0, rkR = 0.0;
 #pragma unroll
     for (int m = 0; m < DIM; ++m) {
-        keL += wl[1 + m] * wl[1 + m];
-        keR += wr[1 + m] * wr[1 + m];
+        mL[m] = mul(wl[0], wl[1 + m]);
+        mR[m] = mul(wr[0], wr[1 + m]);
+        rkL = fma(mL[m], wl[1 + m], rkL);
+        rkR = fma(mR[m], wr[1 + m], rkR);
     }
-    const T EL = wl[NC - 1] * inv_gm1 + T(0.5) * wl[0] * keL;
-    const T ER = wr[NC - 1] * inv_gm1 + T(0.5) * wr[0] * keR;
-    const T unL = wl[1 + D], unR = wr[1 + D];
-    const T cL = psqrt<T>(fdiv<T>(gam * wl[NC - 1], wl[0]));
-    const T cR = psqrt<T>(fdiv<T>(gam * wr[NC - 1], wr[0]));
-    const T sL = fabs(unL) + cL, sR = fabs(unR) + cR;
-    const T smax = sL > sR ? sL : sR;
-    F[0] = T(0.5) * (wl[0] * unL + wr[0] * unR) - T(0.5) * smax * (wr[0] - wl[0]);
+    const double gpL = mul(g.gamma, pL), gpR = mul(g.gamma, pR);
+    const double sL = fma(gpL, drsqrt(mul(gpL, wl[0])), fabs(unL));
+    const double sR = fma(gpR, drsqrt(mul(gpR, wr[0])), fabs(unR));
+    const double sm = dmax_nonneg(sL, sR);
+    F[0] = fma(sm, sub(wl[0], wr[0]), add(mL[D], mR[D]));
 #pragma unroll
     for (int m = 0; m < DIM; ++m) {
-        T mL = wl[0] * wl[1 + m], mR = wr[0] * wr[1 + m];
-        T fL = mL * unL + (m == D ? wl[NC - 1] : T(0));
-        T fR = mR * unR + (m == D ? wr[NC - 1] : T(0));
-        F[1 + m] = T(0.5) * (fL + fR) - T(0.5) * smax * (mR - mL);
+        const double f = m == D ? add(fma(mL[m], unL, pL), fma(mR[m], unR, pR))
+                                : fma(mL[m], unL, mul(mR[m], unR));
+        F[1 + m] = fma(sm, sub(mL[m], mR[m]), f);
     }
-    F[NC - 1] = T(0.5) * ((EL + wl[NC - 1]) * unL + (ER + wr[NC - 1]) * unR) -
-                T(0.5) * smax * (ER - EL);
-
-    if (!k.viscous) return;
+    const double HL = fma(pL, k.h1, rkL), HR = fma(pR, k.h1, rkR);   // 2 rho H
+    const double EL = fma(pL, k.e1, rkL), ER = fma(pR, k.e1, rkR);   // 2 rho E
+    F[NC - 1] = fma(sm, sub(EL, ER), fma(HL, unL, mul(HR, unR)));
+    if (!(g.mu_inf > 0.0)) return;
 
     // viscous stress and heat flux; face values from the two adjacent cells,
     // tangential derivatives from the average of the two cells' central
-    // differences
-    const T inv_h = k.inv_h;
-    const T *Tc = sW + (DIM + 2) * B::PN;
-    const T Tf = T(0.5) * (Tc[a] + Tc[b]);
-    const T Sv = k.S;
-    const T mu = fdiv<T>(k.mu_inf * Tf * psqrt<T>(Tf) * (T(1) + Sv), Tf + Sv);
-    const T lam = mu * k.lam_fac;
-    T grad[DIM][DIM];
+    // differences; T^(3/2) / (T + S) is T^2 / sqrt(T (T + S)^2)
+    const double *T = sW + (DIM + 2) * B::PN;
+    const double sT = add(T[a], T[b]), y = add(sT, k.s2);
+    const double mm = mul(mul(k.km, sT), mul(sT, drsqrt(mul(mul(sT, y), y))));   // 2 mu / h
+    const double *un = sW + (1 + D) * B::PN;
+    double dt = 0.0, work = 0.0;     // tangential part of the divergence; 2 u . tau
 #pragma unroll
     for (int m = 0; m < DIM; ++m) {
-        const T *um = sW + (1 + m) * B::PN;
-#pragma unroll
-        for (int e = 0; e < DIM; ++e) {
-            if (e == D) {
-                grad[m][e] = (um[b] - um[a]) * inv_h;
-            } else {
-                const int t = e == 0 ? B::SX : (e == 1 ? B::SY : B::SZ);
-                grad[m][e] = (um[a + t] - um[a - t] + um[b + t] - um[b - t]) * (T(0.25) * inv_h);
-            }
-        }
+        if (m == D) continue;
+        const int t = m == 0 ? B::SX : (m == 1 ? B::SY : B::SZ);
+        const double *um = sW + (1 + m) * B::PN;
+        // along axis m: the normal and the m-th velocity
+        const double d1n = add(sub(un[a + t], un[a - t]), sub(un[b + t], un[b - t]));
+        const double d1m = add(sub(um[a + t], um[a - t]), sub(um[b + t], um[b - t]));
+        dt = add(dt, d1m);
+        const double tau = mul(mm, fma(0.25, d1n, sub(um[b], um[a])));
+        F[1 + m] = sub(F[1 + m], tau);
+        work = fma(add(um[a], um[b]), tau, work);
     }
-    T div = 0;
-#pragma unroll
-    for (int m = 0; m < DIM; ++m) div += grad[m][m];
-    T work = 0;
-#pragma unroll
-    for (int m = 0; m < DIM; ++m) {
-        T tau = mu * (grad[D][m] + grad[m][D]);
-        if (m == D) tau -= T(2.0 / 3.0) * mu * div;
-        const T *um = sW + (1 + m) * B::PN;
-        const T uf = T(0.5) * (um[a] + um[b]);
-        F[1 + m] -= tau;
-        work += uf * tau;
-    }
-    F[NC - 1] -= work + lam * (Tc[b] - Tc[a]) * inv_h;
+    const double tnn = mul(mm, fma(4.0 / 3.0, sub(un[b], un[a]), mul(-1.0 / 6.0, dt)));
+    F[1 + D] = sub(F[1 + D], tnn);
+    work = fma(add(un[a], un[b]), tnn, work);
+    F[NC - 1] = sub(F[NC - 1], fma(mul(k.kl, mm), sub(T[b], T[a]), work));
 }
 
-// One direction: evaluate all faces of the tile normal to axis D, then add
-// each cell's flux difference to its accumulator.
-template <typename B, typename T, int D>
-__device__ __forceinline__ void direction_pass(const FluxK<T> &k, const T *__restrict__ sW,
-                                               T *__restrict__ sF, T (&acc)[B::CPT][B::DIM + 2]) {
+// One direction: the limited slopes, all faces of the tile normal to axis D,
+// then each cell's flux difference added to its accumulator.
+template <typename B, int D>
+__device__ __forceinline__ void direction_pass(const GridParams &g, const double *__restrict__ sW,
+                                               double *__restrict__ sF, double *__restrict__ sS,
+                                               double (&acc)[B::CPT][B::DIM + 2]) {
     constexpr int DIM = B::DIM;
     constexpr int NC = DIM + 2;
     constexpr int dx = D == 0, dy = D == 1, dz = (D == 2 && DIM == 3);
     constexpr int FX = B::BX + dx, FY = B::BY + dy, FZ = B::BZ + dz;
     constexpr int NF = FX * FY * FZ;
+    // the slope buffer's extents and its stride along D
+    constexpr int EX = B::BX + 2 * dx, EY = B::BY + 2 * dy, EZ = B::BZ + 2 * dz, NS = EX * EY * EZ;
+    constexpr int HS = D == 0 ? 1 : (D == 1 ? EX : EX * EY);
+    slope_pass<B, D>(sW, sS);
+    __syncthreads();
     for (int f = threadIdx.x; f < NF; f += NT) {
         const int fx = f % FX;
         const int r = f / FX;
@@ -220,8 +209,8 @@ __device__ __forceinline__ void direction_pass(const FluxK<T> &k, const T *__res
         const int fz = r / FY;
         const int a = (fx - dx + 2) + B::PX * (fy - dy + 2) +
                       (DIM == 3 ? B::PX * B::PY * (fz - dz + 2) : 0);
-        T F[NC];
-        face_flux<B, T, D>(k, sW, a, F);
+        double F[NC];
+        face_flux<B, D>(g, sW, a, sS + fx + EX * (fy + EY * fz), HS, NS, F);
 #pragma unroll
         for (int c = 0; c < NC; ++c) sF[c * B::NFMAX + f] = F[c];
     }
@@ -236,10 +225,12 @@ __device__ __forceinline__ void direction_pass(const FluxK<T> &k, const T *__res
             const int flo = cx + FX * (cy + FY * cz);
             const int fhi = (cx + dx) + FX * ((cy + dy) + FY * (cz + dz));
 #pragma unroll
-            for (int c = 0; c < NC; ++c) acc[i][c] += sF[c * B::NFMAX + flo] - sF[c * B::NFMAX + fhi];
+            for (int c = 0; c < NC; ++c)
+                acc[i][c] = add(acc[i][c], sub(sF[c * B::NFMAX + flo], sF[c * B::NFMAX + fhi]));
         }
     }
-    __syncthreads();
+    // (no barrier: the next pass writes the slopes, read before the barrier
+    // above, and its faces only after its own)
 }
 
 __device__ __forceinline__ double warp_max(double v) {
@@ -253,93 +244,96 @@ __device__ __forceinline__ double warp_max(double v) {
 // and the maximum of s_j(U*) over the tile's cells outside the band is
 // returned to thread 0 (every thread must call; the function synchronises;
 // a later call may reuse s_red only after its own first barrier).
-template <typename B, typename T, int MODE>
+template <typename B, int MODE>
 __device__ __forceinline__ double stage_tile(const GridParams &g, int ox, int oy, int oz,
-                                             const T *__restrict__ Uin, const T *__restrict__ Un,
-                                             T *__restrict__ out, const T dt,
+                                             const double *__restrict__ Uin,
+                                             const double *__restrict__ Un,
+                                             double *__restrict__ out, const double dt,
                                              const unsigned *__restrict__ band_bits,
                                              unsigned char *smem_raw, double *s_red, bool &bad,
                                              int *err) {
     constexpr int DIM = B::DIM;
     constexpr int NC = DIM + 2;
-    T *sW = reinterpret_cast<T *>(smem_raw);
-    T *sF = sW + B::NW * B::PN;
+    double *sW = reinterpret_cast<double *>(smem_raw);
+    double *sF = sW + B::NW * B::PN;
+    double *sS = sF + NC * B::NFMAX;
 
     const int tid = threadIdx.x;
     const long long N = g.N;
-    const FluxK<T> k(g);
-    const T gm1 = k.gm1;
-    const T invR = k.invR;
+    const double gm1 = g.gamma - 1.0;
 
     // ---- load tile + halo, to primitives
     // Tiles whose halo lies inside the domain index directly; the others map
-    // every halo index through the boundary conditions.
+    // every halo index through the boundary conditions.  The halo's corners
+    // (outside the tile along two axes, by two cells along one of them, or
+    // along three) are read by no face.
     const bool interior = ox >= 2 && oy >= 2 && ox + B::BX + 2 <= g.n[0] &&
                           oy + B::BY + 2 <= g.n[1] &&
                           (DIM == 2 || (oz >= 2 && oz + B::BZ + 2 <= g.n[2]));
-    const T p_inf_E = k.E_inf;
     for (int q = tid; q < B::PN; q += NT) {
         const int lx = q % B::PX;
         const int r = q / B::PX;
         const int ly = r % B::PY;
         const int lz = r / B::PY;
-        T u[NC];
+        auto outside = [](int l, int n) { return l < 2 ? 2 - l : l > n + 1 ? l - n - 1 : 0; };
+        const int ex = outside(lx, B::BX), ey = outside(ly, B::BY),
+                  ez = DIM == 3 ? outside(lz, B::BZ) : 0;
+        if (ex + ey + ez > 2 || (ex && ey && ez)) continue;
+        double u[NC];
         if (interior) {
             const long long j = (ox + lx - 2) +
                                 (long long)g.n[0] * ((oy + ly - 2) + (long long)g.n[1] * (oz + lz - 2 * (DIM == 3)));
             const bool okj = in_bounds(j, N, err);
 #pragma unroll
-            for (int c = 0; c < NC; ++c) u[c] = okj ? __ldg(Uin + c * N + j) : T(0);
+            for (int c = 0; c < NC; ++c) u[c] = okj ? __ldg(Uin + c * N + j) : 0.0;
         } else {
             int flip = 0, fs = 0;
             const int sx = map_axis(ox + lx - 2, g.n[0], g.bc[0], g.bc[1], 0, flip, fs);
             const int sy = map_axis(oy + ly - 2, g.n[1], g.bc[2], g.bc[3], 1, flip, fs);
             const int sz = DIM == 3 ? map_axis(oz + lz - 2, g.n[2], g.bc[4], g.bc[5], 2, flip, fs) : 0;
             if (fs) {
-                u[0] = T(1);
-                u[1] = T(1);
+                u[0] = 1.0;
+                u[1] = 1.0;
 #pragma unroll
-                for (int d = 1; d < DIM; ++d) u[1 + d] = T(0);
-                u[NC - 1] = p_inf_E;
+                for (int d = 1; d < DIM; ++d) u[1 + d] = 0.0;
+                u[NC - 1] = g.d.E_inf;
             } else {
                 const long long j = sx + (long long)g.n[0] * (sy + (long long)g.n[1] * sz);
                 const bool okj = in_bounds(j, N, err);
 #pragma unroll
-                for (int c = 0; c < NC; ++c) u[c] = okj ? __ldg(Uin + c * N + j) : T(0);
+                for (int c = 0; c < NC; ++c) u[c] = okj ? __ldg(Uin + c * N + j) : 0.0;
 #pragma unroll
                 for (int d = 0; d < DIM; ++d)
                     if ((flip >> d) & 1) u[1 + d] = -u[1 + d];
             }
         }
-        const T rho = u[0];
-        const T inv = fdiv<T>(T(1), rho);
-        T ke = 0;
+        const double inv = drcp(u[0]);
+        double rk = 0.0;
 #pragma unroll
         for (int d = 0; d < DIM; ++d) {
-            const T v = u[1 + d] * inv;
+            const double v = mul(u[1 + d], inv);
             sW[(1 + d) * B::PN + q] = v;
-            ke += v * v;
+            rk = fma(u[1 + d], v, rk);
         }
-        const T p = gm1 * (u[NC - 1] - T(0.5) * rho * ke);
-        sW[q] = rho;
+        const double p = mul(gm1, fma(-0.5, rk, u[NC - 1]));
+        sW[q] = u[0];
         sW[(DIM + 1) * B::PN + q] = p;
-        sW[(DIM + 2) * B::PN + q] = p * inv * invR;
+        sW[(DIM + 2) * B::PN + q] = mul(p, inv);
     }
     __syncthreads();
 
     // ---- faces, one direction at a time
-    T acc[B::CPT][NC];
+    double acc[B::CPT][NC];
 #pragma unroll
     for (int i = 0; i < B::CPT; ++i)
 #pragma unroll
-        for (int c = 0; c < NC; ++c) acc[i][c] = T(0);
-    direction_pass<B, T, 0>(k, sW, sF, acc);
-    direction_pass<B, T, 1>(k, sW, sF, acc);
-    if constexpr (DIM == 3) direction_pass<B, T, 2>(k, sW, sF, acc);
+        for (int c = 0; c < NC; ++c) acc[i][c] = 0.0;
+    direction_pass<B, 0>(g, sW, sF, sS, acc);
+    direction_pass<B, 1>(g, sW, sF, sS, acc);
+    if constexpr (DIM == 3) direction_pass<B, 2>(g, sW, sF, sS, acc);
 
     // ---- outputs
-    const T inv_h = k.inv_h;
-    T smax_t = T(0);   // in the compute type: one conversion per tile, not per cell
+    double smax_t = 0.0;
     bool ok = true;
 #pragma unroll
     for (int i = 0; i < B::CPT; ++i) {
@@ -352,57 +346,49 @@ __device__ __forceinline__ double stage_tile(const GridParams &g, int ox, int oy
         if (gx >= g.n[0] || gy >= g.n[1] || (DIM == 3 && gz >= g.n[2])) continue;
         const long long j = gx + (long long)g.n[0] * (gy + (long long)g.n[1] * gz);
         if (!in_bounds(j, N, err)) continue;
-        if (MODE == 0) {
+        double us[NC];
 #pragma unroll
-            for (int c = 0; c < NC; ++c) out[c * N + j] = acc[i][c] * inv_h;
-        } else if (MODE == 1) {
-#pragma unroll
-            for (int c = 0; c < NC; ++c) out[c * N + j] = __ldg(Uin + c * N + j) + dt * (acc[i][c] * inv_h);
-        } else {
-            T us[NC];
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                const T un = __ldg(Un + c * N + j);
-                const T u1 = __ldg(Uin + c * N + j);
-                us[c] = T(0.5) * un + T(0.5) * (u1 + dt * (acc[i][c] * inv_h));
-                out[c * N + j] = us[c];
-            }
-            if (!band_bit(band_bits, j)) {
-                const T sj = step_rate<DIM, T>(g, us, ok);
-                smax_t = fmax(smax_t, sj);
-            }
+        for (int c = 0; c < NC; ++c) {
+            const double L = mul(c == NC - 1 ? g.d.qinv_h : g.d.hinv_h, acc[i][c]);
+            if (MODE == 0) us[c] = L;
+            else us[c] = fma(dt, L, __ldg(Uin + c * N + j));
+            if (MODE == 2) us[c] = fma(0.5, __ldg(Un + c * N + j), mul(0.5, us[c]));
+            out[c * N + j] = us[c];
         }
+        if (MODE == 2 && !band_bit(band_bits, j))
+            smax_t = fmax(smax_t, step_rate<DIM, double>(g, us, ok));
     }
 
     if (MODE == 2) {
-        // the tile's maximum in the compute type (exact), widened once
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) smax_t = fmax(smax_t, __shfl_xor_sync(0xffffffffu, smax_t, o));
+        for (int o = 16; o > 0; o >>= 1)
+            smax_t = dmax_nonneg(smax_t, __shfl_xor_sync(0xffffffffu, smax_t, o));
         bad = __syncthreads_or(!ok) != 0;
-        if ((tid & 31) == 0) s_red[tid >> 5] = (double)smax_t;
+        if ((tid & 31) == 0) s_red[tid >> 5] = smax_t;
         __syncthreads();
         if (tid != 0) return 0.0;
         double m = s_red[0];
-        for (int w = 1; w < NT / 32; ++w) m = fmax(m, s_red[w]);
+        for (int w = 1; w < NT / 32; ++w) m = dmax_nonneg(m, s_red[w]);
         return m;
     }
     return 0.0;
 }
 
-template <int DIM, typename T, int MODE, bool SMALL>
-__global__ void __launch_bounds__(NT)
-stage_kernel(const GridParams g, const T *__restrict__ Uin, const T *__restrict__ Un,
-             T *__restrict__ out, double *__restrict__ blockmax, const double *__restrict__ dt_ptr,
-             int *__restrict__ err, const unsigned *__restrict__ band_bits, double dt_fixed) {
-    using B = StageBox<DIM, T, SMALL>;
+template <int DIM, int MODE, bool SMALL>
+__global__ void __launch_bounds__(NT, 2)
+stage_kernel(const GridParams g, const double *__restrict__ Uin, const double *__restrict__ Un,
+             double *__restrict__ out, double *__restrict__ blockmax,
+             const double *__restrict__ dt_ptr, int *__restrict__ err,
+             const unsigned *__restrict__ band_bits, double dt_fixed) {
+    using B = StageBox<DIM, SMALL>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double s_red[NT / 32];
     const int ox = blockIdx.x * B::BX, oy = blockIdx.y * B::BY;
     const int oz = DIM == 3 ? blockIdx.z * B::BZ : 0;
-    const T dt = MODE == 0 ? T(0) : (T)(dt_fixed > 0.0 ? dt_fixed : *dt_ptr);
+    const double dt = MODE == 0 ? 0.0 : (dt_fixed > 0.0 ? dt_fixed : *dt_ptr);
     bool bad = false;
-    const double m = stage_tile<B, T, MODE>(g, ox, oy, oz, Uin, Un, out, dt, band_bits, smem_raw,
-                                            s_red, bad, err);
+    const double m = stage_tile<B, MODE>(g, ox, oy, oz, Uin, Un, out, dt, band_bits, smem_raw, s_red,
+                                         bad, err);
     if (MODE == 2 && threadIdx.x == 0) {
         blockmax[blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)] = m;
         if (bad) record_error(err, ERR_NONFINITE);
@@ -412,16 +398,11 @@ stage_kernel(const GridParams g, const T *__restrict__ Uin, const T *__restrict_
 // The same stages over a batch of 2D grids: one persistent launch walks a
 // list of (case, tile) work items; every case keeps its own parameters,
 // state, step size and error word.  MODE 2 writes one maximum per item.
-// FP32: five CTAs per SM (48 registers, a few bytes of spill): measured
-// faster on the 64-case batch than four (64 registers) or three
-#ifndef IBM_BATCH_MIN_BLOCKS
-#define IBM_BATCH_MIN_BLOCKS 5
-#endif
-template <typename T, int S, int MODE>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? IBM_BATCH_MIN_BLOCKS : 1)
+template <int S, int MODE>
+__global__ void __launch_bounds__(NT, 2)
 batch_stage_kernel(const BatchCase *__restrict__ cases, const int2 *__restrict__ items,
                    int n_items, double *__restrict__ item_max, double dt_fixed) {
-    using B = typename Shape2<T, S>::type;
+    using B = typename Shape2<S>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double s_red[NT / 32];
     for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
@@ -430,16 +411,17 @@ batch_stage_kernel(const BatchCase *__restrict__ cases, const int2 *__restrict__
         const GridParams g = bc.g;
         const int ntx = (g.n[0] + B::BX - 1) / B::BX;
         const int ox = (w.y % ntx) * B::BX, oy = (w.y / ntx) * B::BY;
-        const T dt = MODE == 0 ? T(0) : (T)(dt_fixed > 0.0 ? dt_fixed : *bc.dt);
-        const T *Uin = (const T *)(MODE == 2 ? bc.U1 : bc.Un);
-        T *out = (T *)(MODE == 2 ? bc.Us : bc.U1);
+        const double dt = dt_fixed > 0.0 ? dt_fixed : *bc.dt;
+        const double *Uin = (const double *)(MODE == 2 ? bc.U1 : bc.Un);
+        double *out = (double *)(MODE == 2 ? bc.Us : bc.U1);
         bool bad = false;
-        const double m = stage_tile<B, T, MODE>(g, ox, oy, 0, Uin, (const T *)bc.Un, out, dt,
-                                                bc.band_bits, smem_raw, s_red, bad, bc.err);
+        const double m = stage_tile<B, MODE>(g, ox, oy, 0, Uin, (const double *)bc.Un, out, dt,
+                                             bc.band_bits, smem_raw, s_red, bad, bc.err);
         if (MODE == 2 && threadIdx.x == 0) {
             item_max[it] = m;
             if (bad) record_error(bc.err, ERR_NONFINITE);
         }
+        __syncthreads();   // the next item rewrites the tile's shared memory
     }
 }
 
@@ -448,13 +430,14 @@ batch_stage_kernel(const BatchCase *__restrict__ cases, const int2 *__restrict__
 template <int DIM, typename T>
 __global__ void __launch_bounds__(NT)
 dt_init_kernel(const GridParams g, const T *__restrict__ U, double *__restrict__ blockmax,
-               unsigned *__restrict__ counter, double *__restrict__ dt, int *__restrict__ err) {
+               unsigned *__restrict__ counter, double *__restrict__ dt, int *__restrict__ err,
+               int cells) {
     constexpr int NC = DIM + 2;
     __shared__ double s_red[NT / 32];
     __shared__ int s_last;
     const long long N = g.N;
-    const long long j0 = (long long)blockIdx.x * DT_CELLS_PER_CTA;
-    const long long j1 = j0 + DT_CELLS_PER_CTA < N ? j0 + DT_CELLS_PER_CTA : N;
+    const long long j0 = (long long)blockIdx.x * cells;
+    const long long j1 = j0 + cells < N ? j0 + cells : N;
     double smax = 0.0;
     bool ok = true;
     for (long long j = j0 + threadIdx.x; j < j1; j += NT) {
@@ -493,58 +476,50 @@ dt_init_kernel(const GridParams g, const T *__restrict__ U, double *__restrict__
     }
 }
 
-template <int DIM, typename T, bool SMALL = false>
+template <int DIM, bool SMALL = false>
 dim3 stage_grid(const GridParams &g) {
-    using B = StageBox<DIM, T, SMALL>;
+    using B = StageBox<DIM, SMALL>;
     return dim3((g.n[0] + B::BX - 1) / B::BX, (g.n[1] + B::BY - 1) / B::BY,
                 DIM == 3 ? (g.n[2] + B::BZ - 1) / B::BZ : 1);
 }
 
-template <int DIM, typename T, int MODE, bool SMALL>
+template <int DIM, int MODE, bool SMALL>
 cudaError_t launch_box(const GridParams &g, const void *Uin, const void *Un, void *out,
                        const FluidBuffers &fb, double dt_fixed, cudaStream_t s) {
-    using B = StageBox<DIM, T, SMALL>;
-    cudaError_t e = func_smem_attr((const void *)stage_kernel<DIM, T, MODE, SMALL>, B::SMEM);
+    using B = StageBox<DIM, SMALL>;
+    cudaError_t e = func_smem_attr((const void *)stage_kernel<DIM, MODE, SMALL>, B::SMEM);
     if (e != cudaSuccess) return e;
-    stage_kernel<DIM, T, MODE, SMALL><<<stage_grid<DIM, T, SMALL>(g), NT, B::SMEM, s>>>(
-        g, (const T *)Uin, (const T *)Un, (T *)out, fb.blockmax, fb.dt, fb.err, fb.band_bits,
-        dt_fixed);
+    stage_kernel<DIM, MODE, SMALL><<<stage_grid<DIM, SMALL>(g), NT, B::SMEM, s>>>(
+        g, (const double *)Uin, (const double *)Un, (double *)out, fb.blockmax, fb.dt, fb.err,
+        fb.band_bits, dt_fixed);
     return cudaGetLastError();
-}
-
-template <int DIM, typename T, int MODE>
-cudaError_t launch_one(const GridParams &g, const void *Uin, const void *Un, void *out,
-                       const FluidBuffers &fb, double dt_fixed, cudaStream_t s) {
-    if (DIM == 2 && sizeof(T) == 8 && small_2d_fp64(g))
-        return launch_box<DIM, T, MODE, DIM == 2 && sizeof(T) == 8>(g, Uin, Un, out, fb, dt_fixed, s);
-    return launch_box<DIM, T, MODE, false>(g, Uin, Un, out, fb, dt_fixed, s);
 }
 
 template <int MODE>
 cudaError_t dispatch(const GridParams &g, int fp_bytes, const void *Uin, const void *Un, void *out,
                      const FluidBuffers &fb, double dt_fixed, cudaStream_t s) {
-    if (g.dim == 3) {
-        if (fp_bytes == 4) return launch_zmarch(MODE, g, Uin, Un, out, fb, dt_fixed, s);
-        return launch_one<3, double, MODE>(g, Uin, Un, out, fb, dt_fixed, s);
-    }
-    if (fp_bytes == 4) return launch_ymarch(MODE, g, Uin, Un, out, fb, dt_fixed, s);
-    return launch_one<2, double, MODE>(g, Uin, Un, out, fb, dt_fixed, s);
+    if (fp_bytes == 4)
+        return g.dim == 3 ? launch_zmarch(MODE, g, Uin, Un, out, fb, dt_fixed, s)
+                          : launch_ymarch(MODE, g, Uin, Un, out, fb, dt_fixed, s);
+    if (g.dim == 3) return launch_box<3, MODE, false>(g, Uin, Un, out, fb, dt_fixed, s);
+    return small_2d_fp64(g) ? launch_box<2, MODE, true>(g, Uin, Un, out, fb, dt_fixed, s)
+                            : launch_box<2, MODE, false>(g, Uin, Un, out, fb, dt_fixed, s);
 }
 
-template <typename T, int S, int MODE>
+template <int S, int MODE>
 cudaError_t batch_stage_t(const BatchCase *cases, const int2 *items, int n_items,
                           double *item_max, double dt_fixed, int n_sm, cudaStream_t s) {
-    using B = typename Shape2<T, S>::type;
+    using B = typename Shape2<S>::type;
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = func_smem_attr((const void *)batch_stage_kernel<T, S, MODE>, B::SMEM);
+    if (e == cudaSuccess) e = func_smem_attr((const void *)batch_stage_kernel<S, MODE>, B::SMEM);
     if (e != cudaSuccess) return e;
     // resident blocks per SM, per device ordinal (0: not yet asked)
     static std::atomic<int> per_sm_of[64];
     int per_sm = dev < 64 ? per_sm_of[dev].load() : 0;
     if (per_sm == 0) {
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_stage_kernel<T, S, MODE>,
-                                                          NT, B::SMEM);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_stage_kernel<S, MODE>, NT,
+                                                          B::SMEM);
         if (e != cudaSuccess) return e;
         if (per_sm < 1) per_sm = 1;
         if (dev < 64) per_sm_of[dev].store(per_sm);
@@ -552,19 +527,19 @@ cudaError_t batch_stage_t(const BatchCase *cases, const int2 *items, int n_items
     long long ctas = (long long)per_sm * (n_sm > 0 ? n_sm : 1);
     if (ctas > n_items) ctas = n_items;
     if (ctas < 1) return cudaSuccess;
-    batch_stage_kernel<T, S, MODE><<<(unsigned)ctas, NT, B::SMEM, s>>>(cases, items, n_items,
-                                                                        item_max, dt_fixed);
+    batch_stage_kernel<S, MODE><<<(unsigned)ctas, NT, B::SMEM, s>>>(cases, items, n_items, item_max,
+                                                                     dt_fixed);
     return cudaGetLastError();
 }
 
-template <typename T, int MODE>
+template <int MODE>
 cudaError_t batch_stage_shape(int shape, const BatchCase *cases, const int2 *items, int n_items,
                               double *item_max, double dt_fixed, int n_sm, cudaStream_t s) {
     switch (shape) {
-    case 0: return batch_stage_t<T, 0, MODE>(cases, items, n_items, item_max, dt_fixed, n_sm, s);
-    case 1: return batch_stage_t<T, 1, MODE>(cases, items, n_items, item_max, dt_fixed, n_sm, s);
-    case 2: return batch_stage_t<T, 2, MODE>(cases, items, n_items, item_max, dt_fixed, n_sm, s);
-    case 3: return batch_stage_t<T, 3, MODE>(cases, items, n_items, item_max, dt_fixed, n_sm, s);
+    case 0: return batch_stage_t<0, MODE>(cases, items, n_items, item_max, dt_fixed, n_sm, s);
+    case 1: return batch_stage_t<1, MODE>(cases, items, n_items, item_max, dt_fixed, n_sm, s);
+    case 2: return batch_stage_t<2, MODE>(cases, items, n_items, item_max, dt_fixed, n_sm, s);
+    case 3: return batch_stage_t<3, MODE>(cases, items, n_items, item_max, dt_fixed, n_sm, s);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -585,23 +560,22 @@ cudaError_t launch_batch_stage(int mode, int shape, int fp_bytes, const BatchCas
     if (fp_bytes == 4)
         return launch_batch_ymarch(mode, shape, cases, items, n_items, item_max, dt_fixed, s);
     if (mode == 1)
-        return batch_stage_shape<double, 1>(shape, cases, items, n_items, item_max, dt_fixed, n_sm, s);
+        return batch_stage_shape<1>(shape, cases, items, n_items, item_max, dt_fixed, n_sm, s);
     if (mode == 2)
-        return batch_stage_shape<double, 2>(shape, cases, items, n_items, item_max, dt_fixed, n_sm, s);
+        return batch_stage_shape<2>(shape, cases, items, n_items, item_max, dt_fixed, n_sm, s);
     return cudaErrorInvalidValue;
 }
 
 size_t fluid_stage_blocks(const GridParams &g, int fp_bytes) {
-    dim3 d;
-    if (g.dim == 3 && fp_bytes == 4) return zmarch_blocks(g);
-    if (g.dim == 3) d = stage_grid<3, double>(g);
-    else if (fp_bytes == 4) return ymarch_blocks(g);
-    else d = small_2d_fp64(g) ? stage_grid<2, double, true>(g) : stage_grid<2, double>(g);
+    if (fp_bytes == 4) return g.dim == 3 ? zmarch_blocks(g) : ymarch_blocks(g);
+    const dim3 d = g.dim == 3 ? stage_grid<3>(g)
+                   : small_2d_fp64(g) ? stage_grid<2, true>(g) : stage_grid<2>(g);
     return (size_t)d.x * d.y * d.z;
 }
 
 size_t dt_init_blocks(const GridParams &g) {
-    return (size_t)((g.N + DT_CELLS_PER_CTA - 1) / DT_CELLS_PER_CTA);
+    const int c = dt_cells_per_cta(g.N);
+    return (size_t)((g.N + c - 1) / c);
 }
 
 size_t fluid_blockmax_count(const GridParams &g, int fp_bytes) {
@@ -627,12 +601,13 @@ cudaError_t launch_rhs(const GridParams &g, int fp_bytes, const void *U, void *L
 cudaError_t launch_dt_init(const GridParams &g, int fp_bytes, const void *U,
                            const FluidBuffers &fb, cudaStream_t s) {
     const unsigned nb = (unsigned)dt_init_blocks(g);
+    const int c = dt_cells_per_cta(g.N);
     if (g.dim == 3) {
-        if (fp_bytes == 4) dt_init_kernel<3, float><<<nb, NT, 0, s>>>(g, (const float *)U, fb.blockmax, fb.counter, fb.dt, fb.err);
-        else dt_init_kernel<3, double><<<nb, NT, 0, s>>>(g, (const double *)U, fb.blockmax, fb.counter, fb.dt, fb.err);
+        if (fp_bytes == 4) dt_init_kernel<3, float><<<nb, NT, 0, s>>>(g, (const float *)U, fb.blockmax, fb.counter, fb.dt, fb.err, c);
+        else dt_init_kernel<3, double><<<nb, NT, 0, s>>>(g, (const double *)U, fb.blockmax, fb.counter, fb.dt, fb.err, c);
     } else {
-        if (fp_bytes == 4) dt_init_kernel<2, float><<<nb, NT, 0, s>>>(g, (const float *)U, fb.blockmax, fb.counter, fb.dt, fb.err);
-        else dt_init_kernel<2, double><<<nb, NT, 0, s>>>(g, (const double *)U, fb.blockmax, fb.counter, fb.dt, fb.err);
+        if (fp_bytes == 4) dt_init_kernel<2, float><<<nb, NT, 0, s>>>(g, (const float *)U, fb.blockmax, fb.counter, fb.dt, fb.err, c);
+        else dt_init_kernel<2, double><<<nb, NT, 0, s>>>(g, (const double *)U, fb.blockmax, fb.counter, fb.dt, fb.err, c);
     }
     return cudaGetLastError();
 }

@@ -34,7 +34,10 @@ struct FluidBuffers {
     const unsigned *band_bits;   // one bit per cell changed by the forcing
 };
 
-constexpr int DT_CELLS_PER_CTA = 2048;   // dt_init: 256 threads x 8 cells
+// dt_init: cells per 256-thread CTA.  One cell per thread until that fills the
+// GPU (an FP64 rate is a chain of ~40 operations of 64 cycles: 8192 cells took
+// 59 us in four CTAs), eight beyond.
+constexpr int dt_cells_per_cta(long long N) { return N >= (1ll << 21) ? 2048 : 256; }
 
 size_t fluid_stage_blocks(const GridParams &g, int fp_bytes);
 size_t dt_init_blocks(const GridParams &g);
@@ -93,34 +96,40 @@ __device__ __forceinline__ float step_rate<3, float>(const GridParams &g, const 
     return step_rate_f<3>(g, u, ok);
 }
 
-template <int DIM, typename T>
-__device__ __forceinline__ T step_rate_generic(const GridParams &g, const T *u, bool &ok) {
-    const T rho = u[0];
-    T ke = T(0), sabs = T(0);
+// FP64 grids, without divisions (explicit roundings: every kernel that forms a
+// rate gives the same bits)
+template <int DIM>
+__device__ __forceinline__ double step_rate_d(const GridParams &g, const double *u, bool &ok) {
+    const DoubleConsts &c = g.d;
+    const double rho = u[0], inv = drcp(rho);
+    double rk = 0.0, sabs = 0.0;
+#pragma unroll
     for (int d = 0; d < DIM; ++d) {
-        const T v = u[1 + d] / rho;
-        ke += v * v;
-        sabs += v < T(0) ? -v : v;
+        const double v = __dmul_rn(u[1 + d], inv);
+        rk = fma(u[1 + d], v, rk);
+        sabs = __dadd_rn(sabs, fabs(v));
     }
-    const T p = (T)(g.gamma - 1.0) * (u[DIM + 1] - T(0.5) * rho * ke);
-    const T c = sqrt((T)g.gamma * p / rho);
-    T mu = T(0);
+    const double p = __dmul_rn(g.gamma - 1.0, fma(-0.5, rk, u[DIM + 1]));
+    const double gp = __dmul_rn(g.gamma, p);
+    const double snd = __dmul_rn(gp, drsqrt(__dmul_rn(gp, rho)));
+    double nu = 0.0;
     if (g.mu_inf > 0.0) {
-        const T Tt = p / (rho * (T)g.R), S = (T)g.S;
-        mu = (T)g.mu_inf * Tt * sqrt(Tt) * (T(1) + S) / (Tt + S);
+        const double T = __dmul_rn(p, inv), y = fma(0.5, c.s2, T);
+        const double mu = __dmul_rn(__dmul_rn(c.kn, T),
+                                    __dmul_rn(T, drsqrt(__dmul_rn(__dmul_rn(T, y), y))));
+        nu = __dmul_rn(mu, inv);
     }
-    const T nu = (T)g.kvisc * mu / rho;
-    const T s = (sabs + T(DIM) * c) * (T)g.inv_h + T(2 * DIM) * nu * (T)(g.inv_h * g.inv_h);
-    if (!(rho > T(0) && p > T(0) && (double)s <= 1.0e300)) ok = false;
+    const double s = fma(fma((double)DIM, snd, sabs), g.inv_h, __dmul_rn(c.ks, nu));
+    if (!(rho > 0.0 && p > 0.0 && s <= 1.0e300)) ok = false;
     return s;
 }
 template <>
 __device__ __forceinline__ double step_rate<3, double>(const GridParams &g, const double *u, bool &ok) {
-    return step_rate_generic<3, double>(g, u, ok);
+    return step_rate_d<3>(g, u, ok);
 }
 template <>
 __device__ __forceinline__ double step_rate<2, double>(const GridParams &g, const double *u, bool &ok) {
-    return step_rate_generic<2, double>(g, u, ok);
+    return step_rate_d<2>(g, u, ok);
 }
 template <>
 __device__ __forceinline__ float step_rate<2, float>(const GridParams &g, const float *u, bool &ok) {

@@ -923,6 +923,8 @@ __device__ __forceinline__ void chol_diag_inverse(float *__restrict__ F, int ld,
 // false when it did not get there in SCG_ITS iterations (the caller then
 // factors A~).
 constexpr int SCG_ROW = 12;   // longest row for which it is tried: see above
+constexpr int SCG_MIN = 64;   // one or two panels factor sooner (61 markers, cold: 171 us for a
+                              // whole set_markers against 176)
 constexpr int SCG_REG = 8, SCG_ITS = 48, SCG_W = (CHOL_MAX + 31) / 32;
 constexpr float SCG_INNER = 1e-5f;
 __device__ __forceinline__ bool small_cg(int ns, const QuadBuffers &q, int k, int cnt,
@@ -1065,7 +1067,7 @@ chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ r
     double rmax = 0.0, rprev = 0.0;
     int it = 0;
     bool done = false;   // the residual is at its floor
-    {
+    if (ns > SCG_MIN && !__syncthreads_or(tid < ns && ecnt[tid] > SCG_ROW)) {
         // corrections by FP32 conjugate gradients first
         float rv[SCG_REG], inv = 0.0f;
         int rc[SCG_REG];
@@ -1084,8 +1086,7 @@ chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ r
                     rc[i] = ec[(size_t)i * ns + tid];
                 }
         }
-        const bool wide = __syncthreads_or(cnt > SCG_ROW) != 0;
-        for (int outer = 0; !wide; ++outer) {
+        for (int outer = 0;; ++outer) {
             rmax = residual();
             if (!(rmax > 0.0) || rmax <= CHOL_FLOOR * rscale ||
                 (outer > 0 && rmax <= 64.0 * CHOL_FLOOR * rscale && !(rmax < 0.5 * rprev))) {
@@ -1111,12 +1112,18 @@ chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ r
     // the dense factor: the lower triangle of A~ (the upper stays zero)
     for (int i = tid; i < ns * ld; i += CHOL_T) F[i] = 0.0f;
     __syncthreads();
-    for (int k = tid; k < ns; k += CHOL_T)
-        for (int i = 0; i < ecnt[k]; ++i) {
+    for (int k = tid; k < ns; k += CHOL_T) {
+        const int c = ecnt[k], cc = min(c, CHOL_EC);
+        for (int i = 0; i < cc; ++i) {
+            const int l = ec[(size_t)i * ns + k];
+            if (l <= k) F[(size_t)k * ld + l] = (float)ev[(size_t)i * ns + k];
+        }
+        for (int i = CHOL_EC; i < c; ++i) {
             const int l = q.col[(long long)i * q.cap + k];
             if (in_bounds(l, ns, err) && l <= k)
                 F[(size_t)k * ld + l] = (float)q.val[(long long)i * q.cap + k];
         }
+    }
     __syncthreads();
     // blocked Cholesky over 32-column panels, then the diagonal blocks' inverses
     for (int c0 = 0; c0 < ns; c0 += CHOL_PB) {

@@ -685,3 +685,19 @@ def test_2d_fp32_march_equals_the_box_kernel(n, bc, offset):
     assert float((La.double() - L8).norm() / L8.norm()) < 1e-4
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("bc", [MIXED_BC, (C.BC_PERIODIC,) * 6, (C.BC_SLIP,) * 6])
+@pytest.mark.parametrize("n", [(4, 4), (5, 7), (8, 17), (33, 9), (257, 255),
+                               (4, 4, 4), (5, 6, 7), (9, 8, 4), (17, 9, 5)])
+def test_fp64_tiles_match_oracle(oracle, n, bc):
+    """L(U) of the FP64 tile kernels around their 8 x 8, 16 x 16 and 8 x 8 x 4
+    tiles, smallest grids and every boundary condition, with the tolerance of
+    test_rhs_matches_oracle"""
+    g = C.small_grid(len(n), n, h=0.1, fp_bytes=8, bc=bc, Re=80.0, Mach=0.4)
+    U = C.random_state(g, seed=43, amp=0.05)
+    grid = ibm.Grid(g)
+    L = grid.rhs(torch.from_numpy(U)).cpu().numpy()
+    grid.close()
+    err = rel_l2(L, oracle.rhs(g, U).reshape(L.shape))
+    assert np.all(err < 1e-12), err
