@@ -326,7 +326,8 @@ ibm_status ibm_rhs_dt_noalloc(const ibm_grid_desc *desc, const void *U, void *L,
 typedef struct ibm_batch ibm_batch;
 
 typedef struct {
-    int tile_shape;        /* fluid-stage tile: 0 = 16x16, 1 = 32x8, 2 = 64x4, 3 = 8x32 cells */
+    int tile_shape;        /* fluid-stage tile, FP64: 0 = 16x16, 1 = 32x8, 2 = 64x4, 3 = 8x32
+                            * cells; FP32: chunks of at most 16, 8, 32 or 64 rows */
     int markers_per_block; /* interpolation: warps (one marker each) per CTA, 1..16 */
     int use_graph;         /* != 0: replay each step from a captured CUDA graph */
 } ibm_batch_tuning;

@@ -20,8 +20,8 @@ LIB = os.path.join(LIBDIR, "libibm_gb300.so")
 # (IBM_ERR_BOUNDS) and the access skipped; for tests, not for timing
 LIB_CHECKED = os.path.join(LIBDIR, "libibm_gb300_checked.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
-UNITS = ["flux.cu", "flux_zm.cu", "flux_ym.cu", "markers.cu", "quadrature.cu", "api.cu", "noalloc.cu", "adjoint.cu",
-         "batch.cu"]
+UNITS = ["flux.cu", "flux_zm.cu", "markers.cu", "quadrature.cu", "api.cu", "noalloc.cu",
+         "adjoint.cu", "batch.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + INCLUDE]
 # The FP32 fluid-stage units flush subnormals to zero: no value of the flow
@@ -31,7 +31,6 @@ FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I" + INCLUDE
 # approximations (FP64 code is unaffected): its FP32 reverse sweep is 23 %
 # faster and stays within the FP32 gradient tolerance.
 UNIT_FLAGS = {"flux.cu": ["-ftz=true"], "flux_zm.cu": ["-ftz=true"],
-              "flux_ym.cu": ["-ftz=true"],
               "adjoint.cu": ["-ftz=true", "-prec-div=false", "-prec-sqrt=false"]}
 # extra nvcc flags (e.g. -DIBM_ZM_MIN_BLOCKS=2) for build variants
 EXTRA = os.environ.get("IBM_NVCC_FLAGS", "").split()

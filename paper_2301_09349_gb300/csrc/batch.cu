@@ -61,6 +61,7 @@ struct ibm_batch {
     int n_stage = 0, n_band = 0, n_mk = 0;
     size_t spread_smem = 0;
     bool spread_op = false;   // spreading through the cases' operators
+    int rows[kBatchShapes] = {0};   // FP32 stages: rows per chunk by shape
     ibm_batch_tuning tune{0, 4, 1};
 
     // kernel timing (ibm_batch_profile): event pairs around each group;
@@ -119,9 +120,11 @@ ibm_status fail(ibm_batch *b, ibm_status st, const std::string &msg) {
             return fail(b, IBM_ERR_CUDA, std::string(where) + ": " + cudaGetErrorString(_e)); \
     } while (0)
 
-int tiles_of_shape(const ibm_grid_desc &d, int shape) {
+// work items of a case: FP64 tiles of the shape, FP32 strip chunks of `rows`
+int tiles_of_shape(const ibm_grid_desc &d, int shape, int rows) {
+    if (d.fp_bytes == 4) return (int)ymarch_batch_items(d, rows);
     int bx = 0, by = 0;
-    batch_tile_shape(shape, d.fp_bytes, &bx, &by);
+    batch_tile_shape(shape, &bx, &by);
     return ((d.n[0] + bx - 1) / bx) * ((d.n[1] + by - 1) / by);
 }
 
@@ -134,6 +137,7 @@ struct BatchLayout {
     size_t tbl = 0, stage_items = 0, item_max = 0, band_items = 0, band_max = 0, mk_items = 0,
            save = 0, gather = 0, tw = 0, total = 0;
     size_t stage_cap = 0, band_cap = 0, mk_cap = 0;
+    int rows[kBatchShapes] = {0};   // FP32: rows per chunk of every shape
 };
 
 // Why the batch description is invalid, or nullptr.
@@ -165,6 +169,8 @@ const char *check_batch(int ncases, const ibm_grid_desc *descs, const int *max_m
 BatchLayout batch_layout(int ncases, const ibm_grid_desc *descs, const int *max_markers) {
     BatchLayout L;
     size_t off = 0;
+    if (descs[0].fp_bytes == 4)
+        for (int s = 0; s < kBatchShapes; ++s) L.rows[s] = ymarch_batch_rows(s, ncases, descs);
     for (int c = 0; c < ncases; ++c) {
         const int mm = max_markers ? max_markers[c] : 0;
         const size_t wb = ibm_workspace_bytes(&descs[c], mm);
@@ -172,7 +178,7 @@ BatchLayout batch_layout(int ncases, const ibm_grid_desc *descs, const int *max_
         L.case_bytes.push_back(wb);
         off = align_up(off + wb, 256);
         int most = 0;
-        for (int s = 0; s < kBatchShapes; ++s) most = std::max(most, tiles_of_shape(descs[c], s));
+        for (int s = 0; s < kBatchShapes; ++s) most = std::max(most, tiles_of_shape(descs[c], s, L.rows[s]));
         L.stage_cap += most;
         // band items: band tiles, or runs of 32 forced cells (at most 3^2 per marker)
         L.band_cap += std::max(marker_tiles(descs[c]), (9 * mm + 31) / 32);
@@ -227,7 +233,7 @@ ibm_status build_tables(ibm_batch *b) {
         bc.band_bits = g->mb.band_bits;
         bc.m = g->mb;
         bc.item0 = (int)st.size();
-        bc.nitems = tiles_of_shape(g->desc, shape);
+        bc.nitems = tiles_of_shape(g->desc, shape, b->rows[shape]);
         for (int t = 0; t < bc.nitems; ++t) st.push_back(make_int2(c, t));
         const int ns = g->mb.ns;
         const int ncell = ns > 0 ? counts[(size_t)c * 4 + 2] : 0;
@@ -310,10 +316,10 @@ cudaError_t launch_group(ibm_batch *b, int p, int group, double dt_fixed, cudaSt
     const int sh = b->tune.tile_shape, fp = b->fp_bytes;
     switch (group) {
     case IBM_PROF_STAGE1:
-        return launch_batch_stage(1, sh, fp, t, b->stage_items, b->n_stage, b->item_max, dt_fixed,
+        return launch_batch_stage(1, sh, b->rows[sh], fp, t, b->stage_items, b->n_stage, b->item_max, dt_fixed,
                                   b->n_sm, s);
     case IBM_PROF_STAGE2:
-        return launch_batch_stage(2, sh, fp, t, b->stage_items, b->n_stage, b->item_max, dt_fixed,
+        return launch_batch_stage(2, sh, b->rows[sh], fp, t, b->stage_items, b->n_stage, b->item_max, dt_fixed,
                                   b->n_sm, s);
     case IBM_PROF_INTERP:
         return launch_batch_interp(fp, t, b->mk_items, b->n_mk, b->tune.markers_per_block, s);
@@ -464,6 +470,7 @@ ibm_status ibm_create_batch(int ncases, const ibm_grid_desc *descs, const int *m
     b->tw_slots = (BatchTwSlot *)(base + L.tw);
     b->tw_vals = (double *)(b->tw_slots + ncases);
     b->stage_cap = L.stage_cap;
+    std::copy(L.rows, L.rows + kBatchShapes, b->rows);
     b->band_cap = L.band_cap;
     b->mk_cap = L.mk_cap;
     int dev = 0;

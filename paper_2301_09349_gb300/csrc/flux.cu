@@ -10,7 +10,7 @@
 // with dt = cfl / max_j s_j(U^n), formed at the end of the previous step (or
 // by dt_init after a new state) so that stage 1 can write U^1 directly.
 //
-// Here: FP64 grids (FP32 grids march: flux_zm.cu, flux_ym.cu).  Each CTA owns
+// Here: FP64 grids (FP32 grids march: flux_zm.cu, flux_ym.cuh).  Each CTA owns
 // a BX x BY x BZ tile of cells.  It loads the tile plus a two-cell halo once
 // (ghost cells mapped through the boundary conditions on the fly), converts
 // to primitives in shared memory, then per direction evaluates every limited
@@ -546,19 +546,18 @@ cudaError_t batch_stage_shape(int shape, const BatchCase *cases, const int2 *ite
 
 }  // namespace
 
-void batch_tile_shape(int shape, int fp_bytes, int *bx, int *by) {
-    if (fp_bytes == 4) return ymarch_tile_shape(shape, bx, by);
+void batch_tile_shape(int shape, int *bx, int *by) {
     static const int X[kBatchShapes] = {16, 32, 64, 8}, Y[kBatchShapes] = {16, 8, 4, 32};
     *bx = X[shape];
     *by = Y[shape];
 }
 
-cudaError_t launch_batch_stage(int mode, int shape, int fp_bytes, const BatchCase *cases,
+cudaError_t launch_batch_stage(int mode, int shape, int rows, int fp_bytes, const BatchCase *cases,
                                const int2 *items, int n_items, double *item_max, double dt_fixed,
                                int n_sm, cudaStream_t s) {
     if (n_items <= 0) return cudaSuccess;
     if (fp_bytes == 4)
-        return launch_batch_ymarch(mode, shape, cases, items, n_items, item_max, dt_fixed, s);
+        return launch_batch_ymarch(mode, rows, cases, items, n_items, item_max, dt_fixed, s);
     if (mode == 1)
         return batch_stage_shape<1>(shape, cases, items, n_items, item_max, dt_fixed, n_sm, s);
     if (mode == 2)
@@ -613,3 +612,5 @@ cudaError_t launch_dt_init(const GridParams &g, int fp_bytes, const void *U,
 }
 
 }  // namespace ibmk
+
+#include "flux_ym.cuh"

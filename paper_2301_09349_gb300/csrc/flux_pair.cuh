@@ -1,4 +1,4 @@
-// Packed FP32x2 arithmetic of the marching fluid stages (flux_ym.cu,
+// Packed FP32x2 arithmetic of the marching fluid stages (flux_ym.cuh,
 // flux_zm.cu): a float2 holds the same quantity of two faces or cells, and
 // every operation is one explicit rounding (nothing is left to contraction).
 #pragma once
@@ -42,6 +42,28 @@ __device__ __forceinline__ float2 vlh2(float2 a, float2 b) {
     const float2 q = ab * rcp2(a + b);
     return make_float2(ab.x > 0.0f ? q.x : 0.0f, ab.y > 0.0f ? q.y : 0.0f);
 }
+
+__device__ __forceinline__ float2 cadd(float c, float2 a) {
+    return make_float2(__fadd_rn(a.x, c), __fadd_rn(a.y, c));
+}
+
+// The same operations on one face or cell.
+struct F1 {
+    float x;
+};
+__device__ __forceinline__ F1 operator+(F1 a, F1 b) { return {__fadd_rn(a.x, b.x)}; }
+__device__ __forceinline__ F1 operator-(F1 a, F1 b) { return {__fsub_rn(a.x, b.x)}; }
+__device__ __forceinline__ F1 operator*(F1 a, F1 b) { return {__fmul_rn(a.x, b.x)}; }
+__device__ __forceinline__ F1 fma2(F1 a, F1 b, F1 c) { return {__fmaf_rn(a.x, b.x, c.x)}; }
+__device__ __forceinline__ F1 rcp2(F1 a) { return {rcp_ftz(a.x)}; }
+__device__ __forceinline__ F1 rsqrt2(F1 a) { return {rsqrtf(a.x)}; }
+__device__ __forceinline__ F1 abs2(F1 a) { return {fabsf(a.x)}; }
+__device__ __forceinline__ F1 max2(F1 a, F1 b) { return {fmaxf(a.x, b.x)}; }
+__device__ __forceinline__ F1 cadd(float c, F1 a) { return {__fadd_rn(a.x, c)}; }
+__device__ __forceinline__ F1 cmul(float c, F1 a) { return {__fmul_rn(c, a.x)}; }
+__device__ __forceinline__ F1 cfma(float c, F1 a, F1 b) { return {__fmaf_rn(c, a.x, b.x)}; }
+__device__ __forceinline__ F1 fabs_fma(F1 a, F1 b, F1 u) { return {__fmaf_rn(a.x, b.x, fabsf(u.x))}; }
+__device__ __forceinline__ F1 vlh2(F1 a, F1 b) { return {vlh1(a.x, b.x)}; }
 
 }  // namespace
 }  // namespace ibmk

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "../../include/ibm.h"
 #include "common.cuh"
 
 namespace ibmk {
@@ -55,7 +56,7 @@ cudaError_t launch_dt_init(const GridParams &g, int fp_bytes, const void *U,
 cudaError_t launch_zmarch(int mode, const GridParams &g, const void *Uin, const void *Un,
                           void *out, const FluidBuffers &fb, double dt_fixed, cudaStream_t s);
 size_t zmarch_blocks(const GridParams &g);
-// the y-marching form used for 2D FP32 grids (flux_ym.cu)
+// the y-marching form used for 2D FP32 grids (flux_ym.cuh)
 cudaError_t launch_ymarch(int mode, const GridParams &g, const void *Uin, const void *Un, void *out,
                           const FluidBuffers &fb, double dt_fixed, cudaStream_t s);
 size_t ymarch_blocks(const GridParams &g);
@@ -255,13 +256,15 @@ struct BatchCase {
 };
 
 constexpr int kBatchShapes = 4;   // 2D tile shapes of the batched stage kernels
-void batch_tile_shape(int shape, int fp_bytes, int *bx, int *by);
-void ymarch_tile_shape(int shape, int *bx, int *by);   // FP32: strips, by rows high
-cudaError_t launch_batch_ymarch(int mode, int shape, const BatchCase *cases, const int2 *items,
+void batch_tile_shape(int shape, int *bx, int *by);   // FP64
+// FP32: strips in chunks of rows; a shape's rows for these cases, a case's chunks
+int ymarch_batch_rows(int shape, int ncases, const ibm_grid_desc *descs);
+long long ymarch_batch_items(const ibm_grid_desc &d, int rows);
+cudaError_t launch_batch_ymarch(int mode, int rows, const BatchCase *cases, const int2 *items,
                                 int n_items, double *item_max, double dt_fixed, cudaStream_t s);
 // mode 1 or 2 as launch_stage1/2; items are (case, tile) pairs in the
-// shape's tile numbering; mode 2 writes item_max[item]
-cudaError_t launch_batch_stage(int mode, int shape, int fp_bytes, const BatchCase *cases,
+// shape's tile numbering (FP32: chunks of `rows`); mode 2 writes item_max[item]
+cudaError_t launch_batch_stage(int mode, int shape, int rows, int fp_bytes, const BatchCase *cases,
                                const int2 *items, int n_items, double *item_max, double dt_fixed,
                                int n_sm, cudaStream_t s);
 // interpolation + forcing: items are (case, marker); warps = markers per CTA

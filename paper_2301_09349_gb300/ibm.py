@@ -110,6 +110,7 @@ SIGNATURES = [
     ("ibm_batch_last_error", ctypes.c_char_p, [_vp]),
 ]
 
+# FP64 stages; FP32 stages: chunks of at most 16, 8, 32, 64 rows
 BATCH_TILE_SHAPES = [(16, 16), (32, 8), (64, 4), (8, 32)]
 BATCH_WARPS = [1, 2, 4, 8, 16]
 BATCH_FORCE_FIELDS = ["Fx", "Fy", "heat_rate", "Cd", "Cl", "Nu", "dt", "t"]

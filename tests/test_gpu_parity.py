@@ -701,3 +701,25 @@ def test_fp64_tiles_match_oracle(oracle, n, bc):
     grid.close()
     err = rel_l2(L, oracle.rhs(g, U).reshape(L.shape))
     assert np.all(err < 1e-12), err
+
+
+@pytest.mark.parametrize("bc", [(0, 1), (3, 3), (2, 2)])
+@pytest.mark.parametrize("nx", [4, 27, 28, 29, 61, 131])
+def test_2d_fp32_single_rows_equal_the_march(nx, bc):
+    """A grid small enough for the single-row form, and the same flow repeated
+    52 times along a periodic y, which marches: the same bits."""
+    small = C.small_grid(2, (nx, 60), h=0.1, fp_bytes=4, bc=bc + (3, 3, 2, 2))
+    tall = C.small_grid(2, (nx, 60 * 52), h=0.1, fp_bytes=4, bc=bc + (3, 3, 2, 2))
+    U = C.random_state(small, 7).astype(np.float32).reshape(4, 60, nx)
+    a, b = ibm.Grid(small), ibm.Grid(tall)
+    La = a.rhs(torch.from_numpy(U).cuda())
+    Lb = b.rhs(torch.from_numpy(np.tile(U, (1, 52, 1))).cuda())
+    assert torch.equal(La.repeat(1, 52, 1), Lb)
+    a.set_state(U)
+    b.set_state(np.tile(U, (1, 52, 1)))
+    a.step(3)
+    b.step(3)
+    assert torch.equal(a.get_state().repeat(1, 52, 1), b.get_state())
+    assert a.time()[0] == b.time()[0]
+    a.close()
+    b.close()
