@@ -53,9 +53,9 @@ template <> struct AdjK<double> {
     double gam, inv_gm1, gm1, invR, mu_inf, S, lam_fac, inv_h, E_inf;
     bool viscous;
     __device__ __forceinline__ explicit AdjK(const GridParams &g)
-        : gam(g.gamma), inv_gm1(1.0 / (g.gamma - 1.0)), gm1(g.gamma - 1.0), invR(1.0 / g.R),
-          mu_inf(g.mu_inf), S(g.S), lam_fac(g.cp / g.Pr), inv_h(g.inv_h),
-          E_inf(g.p_inf / (g.gamma - 1.0) + 0.5), viscous(g.mu_inf > 0.0) {}
+        : gam(g.gamma), inv_gm1(0.5 * g.d.e1), gm1(g.gamma - 1.0), invR(g.d.invR),
+          mu_inf(g.mu_inf), S(g.S), lam_fac(g.d.lam_fac), inv_h(g.inv_h),
+          E_inf(g.d.E_inf), viscous(g.mu_inf > 0.0) {}
 };
 template <> struct AdjK<float> {
     float gam, inv_gm1, gm1, invR, mu_inf, S, lam_fac, inv_h, E_inf;
@@ -69,6 +69,13 @@ template <> struct AdjK<float> {
 template <typename R> __device__ __forceinline__ R sgn(R x) {
     return x > R(0) ? R(1) : (x < R(0) ? R(-1) : R(0));
 }
+
+// reciprocal and reciprocal square root in the compute type: one hardware
+// operation in FP32, a seed with one third-order step in FP64
+__device__ __forceinline__ float rcp_of(float x) { return rcp_ftz(x); }
+__device__ __forceinline__ double rcp_of(double x) { return drcp(x); }
+__device__ __forceinline__ float rsq_of(float x) { return rsqrtf(x); }
+__device__ __forceinline__ double rsq_of(double x) { return drsqrt(x); }
 
 // primitives (rho, u.., p) of the (ghost-mapped) cell (x, y, z); its source
 // cell, slip flips and free-stream flag are returned for the scatter
@@ -97,32 +104,28 @@ __device__ __forceinline__ void load_prim(const GridParams &g, const AdjK<R> &k,
         for (int d = 0; d < DIM; ++d)
             if ((flip >> d) & 1) u[1 + d] = -u[1 + d];
     }
-    const R rho = u[0];
+    const R rho = u[0], inv = rcp_of(rho);
     R ke = R(0);
     w[0] = rho;
 #pragma unroll
     for (int d = 0; d < DIM; ++d) {
-        w[1 + d] = u[1 + d] / rho;
+        w[1 + d] = u[1 + d] * inv;
         ke += w[1 + d] * w[1 + d];
     }
     w[NC - 1] = k.gm1 * (u[NC - 1] - R(0.5) * rho * ke);
 }
 
+// half the limited slope h = ab / (a + b) and its derivatives b^2 / (a + b)^2
+// and a^2 / (a + b)^2 where ab > 0 (all zero off that branch), from one
+// reciprocal
 template <typename R>
-__device__ __forceinline__ R vl(R a, R b) {
-    const R ab = a * b;
-    return ab > R(0) ? R(2) * ab / (a + b) : R(0);
-}
-// partial derivatives of vl(a, b) (zero off the branch taken)
-template <typename R>
-__device__ __forceinline__ void vl_grad(R a, R b, R &da, R &db) {
-    if (a * b > R(0)) {
-        const R s = a + b, s2 = s * s;
-        da = R(2) * b * b / s2;
-        db = R(2) * a * a / s2;
-    } else {
-        da = db = R(0);
-    }
+__device__ __forceinline__ R half_slope(R a, R b, R &da, R &db) {
+    const bool up = a * b > R(0);
+    const R r = rcp_of(up ? a + b : R(1));
+    const R ar = a * r, br = b * r;
+    da = up ? br * br : R(0);
+    db = up ? ar * ar : R(0);
+    return up ? a * br : R(0);
 }
 
 // Reverse of one side's Euler flux and conserved vector: Fx = dJ/dF_side,
@@ -170,15 +173,14 @@ __device__ __forceinline__ void face_vjp(const AdjK<R> &k, const R (&w)[4][DIM +
                                          const R (&Fb)[DIM + 2], R (&wb)[4][DIM + 2],
                                          R (&utb)[ntan(DIM)][4][DIM]) {
     constexpr int NC = DIM + 2;
-    // ---- forward: MUSCL states
-    R wl[NC], wr[NC], d0[NC], d1[NC], d2[NC];
+    // ---- forward: MUSCL states; the half slopes' derivatives are kept for
+    // the reverse pass
+    R wl[NC], wr[NC], a01[NC], b01[NC], a12[NC], b12[NC];
 #pragma unroll
     for (int m = 0; m < NC; ++m) {
-        d0[m] = w[1][m] - w[0][m];
-        d1[m] = w[2][m] - w[1][m];
-        d2[m] = w[3][m] - w[2][m];
-        wl[m] = w[1][m] + R(0.5) * vl(d0[m], d1[m]);
-        wr[m] = w[2][m] - R(0.5) * vl(d1[m], d2[m]);
+        const R d0 = w[1][m] - w[0][m], d1 = w[2][m] - w[1][m], d2 = w[3][m] - w[2][m];
+        wl[m] = w[1][m] + half_slope(d0, d1, a01[m], b01[m]);
+        wr[m] = w[2][m] - half_slope(d1, d2, a12[m], b12[m]);
     }
     // ---- forward: Rusanov
     R UL[NC], UR[NC];
@@ -197,7 +199,11 @@ __device__ __forceinline__ void face_vjp(const AdjK<R> &k, const R (&w)[4][DIM +
     }
     UL[NC - 1] = wl[NC - 1] * k.inv_gm1 + R(0.5) * wl[0] * keL;
     UR[NC - 1] = wr[NC - 1] * k.inv_gm1 + R(0.5) * wr[0] * keR;
-    const R cL = sqrt(k.gam * wl[NC - 1] / wl[0]), cR = sqrt(k.gam * wr[NC - 1] / wr[0]);
+    // c = gamma p y, y = 1 / sqrt(gamma p rho); 1/(2 rho c) gamma = gamma y / 2
+    // and c / (2 rho) = c^2 y / 2 serve the reverse pass
+    const R gpL = k.gam * wl[NC - 1], gpR = k.gam * wr[NC - 1];
+    const R yL = rsq_of(gpL * wl[0]), yR = rsq_of(gpR * wr[0]);
+    const R cL = gpL * yL, cR = gpR * yR;
     const R unL = wl[1 + D], unR = wr[1 + D];
     const R sL = fabs(unL) + cL, sR = fabs(unR) + cR;
     const bool left = sL > sR;
@@ -209,9 +215,11 @@ __device__ __forceinline__ void face_vjp(const AdjK<R> &k, const R (&w)[4][DIM +
 
     // ---- reverse: viscous stress and heat flux
     if (k.viscous) {
-        const R Ta = w[1][NC - 1] * k.invR / w[1][0], Tb = w[2][NC - 1] * k.invR / w[2][0];
+        const R ia = rcp_of(w[1][0]), ib = rcp_of(w[2][0]);
+        const R Ta = w[1][NC - 1] * k.invR * ia, Tb = w[2][NC - 1] * k.invR * ib;
         const R Tf = R(0.5) * (Ta + Tb);
-        const R mu = k.mu_inf * Tf * sqrt(Tf) * (R(1) + k.S) / (Tf + k.S);
+        const R qT = rsq_of(Tf), qS = rcp_of(Tf + k.S);   // 1/sqrt(T), 1/(T + S)
+        const R mu = k.mu_inf * Tf * (Tf * qT) * (R(1) + k.S) * qS;
         const R lam = mu * k.lam_fac;
         const R q = R(0.25) * k.inv_h;
         R grad[DIM][DIM];
@@ -262,7 +270,7 @@ __device__ __forceinline__ void face_vjp(const AdjK<R> &k, const R (&w)[4][DIM +
         }
 #pragma unroll
         for (int m = 0; m < DIM; ++m) gb[m][m] += divb;
-        const R Tfb = mub * mu * (R(1.5) / Tf - R(1) / (Tf + k.S));
+        const R Tfb = mub * mu * (R(1.5) * qT * qT - qS);
         Tab += R(0.5) * Tfb;
         Tbb += R(0.5) * Tfb;
 #pragma unroll
@@ -283,10 +291,10 @@ __device__ __forceinline__ void face_vjp(const AdjK<R> &k, const R (&w)[4][DIM +
             }
         }
         // T = p r^-1 / rho at a and b
-        wb[1][NC - 1] += Tab * k.invR / w[1][0];
-        wb[1][0] -= Tab * Ta / w[1][0];
-        wb[2][NC - 1] += Tbb * k.invR / w[2][0];
-        wb[2][0] -= Tbb * Tb / w[2][0];
+        wb[1][NC - 1] += Tab * k.invR * ia;
+        wb[1][0] -= Tab * Ta * ia;
+        wb[2][NC - 1] += Tbb * k.invR * ib;
+        wb[2][0] -= Tbb * Tb * ib;
     }
 
     // ---- reverse: Rusanov, F = (F_L + F_R)/2 - smax (U_R - U_L)/2
@@ -306,10 +314,10 @@ __device__ __forceinline__ void face_vjp(const AdjK<R> &k, const R (&w)[4][DIM +
     const R sLb = left ? sb : R(0), sRb = left ? R(0) : sb;
     unLb += sgn(unL) * sLb;
     unRb += sgn(unR) * sRb;
-    wlb[NC - 1] += sLb * k.gam / (R(2) * wl[0] * cL);
-    wlb[0] -= sLb * cL / (R(2) * wl[0]);
-    wrb[NC - 1] += sRb * k.gam / (R(2) * wr[0] * cR);
-    wrb[0] -= sRb * cR / (R(2) * wr[0]);
+    wlb[NC - 1] += R(0.5) * sLb * k.gam * yL;
+    wlb[0] -= R(0.5) * sLb * cL * cL * yL;
+    wrb[NC - 1] += R(0.5) * sRb * k.gam * yR;
+    wrb[0] -= R(0.5) * sRb * cR * cR * yR;
     wlb[1 + D] += unLb;
     wrb[1 + D] += unRb;
 
@@ -318,11 +326,8 @@ __device__ __forceinline__ void face_vjp(const AdjK<R> &k, const R (&w)[4][DIM +
     for (int m = 0; m < NC; ++m) {
         wb[1][m] += wlb[m];
         wb[2][m] += wrb[m];
-        R a01, b01, a12, b12;
-        vl_grad(d0[m], d1[m], a01, b01);
-        vl_grad(d1[m], d2[m], a12, b12);
-        const R g01 = R(0.5) * wlb[m], g12 = -R(0.5) * wrb[m];
-        const R d0b = g01 * a01, d1b = g01 * b01 + g12 * a12, d2b = g12 * b12;
+        const R d0b = wlb[m] * a01[m], d1b = wlb[m] * b01[m] - wrb[m] * a12[m],
+                d2b = -(wrb[m] * b12[m]);
         wb[1][m] += d0b - d1b;
         wb[0][m] -= d0b;
         wb[2][m] += d1b - d2b;
@@ -348,34 +353,47 @@ constexpr int FT = IBM_ADJ_FT;
 // axis also the domain face b = n - accumulating the stencil adjoints in
 // shared memory, then adds the tile-plus-halo accumulators to the source
 // cells in global memory (slip flips applied, free-stream ghosts dropped).
-template <int DIM, typename T> struct AdjTile;
-template <> struct AdjTile<3, float> { static constexpr int BX = 8, BY = 8, BZ = 8; };
-template <> struct AdjTile<3, double> { static constexpr int BX = 8, BY = 8, BZ = 4; };
-template <> struct AdjTile<2, float> { static constexpr int BX = 16, BY = 16, BZ = 1; };
-template <> struct AdjTile<2, double> { static constexpr int BX = 16, BY = 16, BZ = 1; };
+// Bound: FP64 grids by the FP64 pipe (two operations per SM cycle; no division
+// or square root is left to it), FP32 grids by instruction issue and latency.
+// SMALL: 2D FP64 grids of fewer than 256 16 x 16 tiles take 8 x 8 ones, four
+// times as many SMs, and reverse their x- and y-faces side by side: 128 x 64
+// (32 of the large tiles) 105 -> 26.5 us; the line is where large tiles fill
+// the SMs (that of the forward stages).
+template <int DIM, typename T, bool SMALL> struct AdjTile;
+template <> struct AdjTile<3, float, false> { static constexpr int BX = 8, BY = 8, BZ = 8; };
+template <> struct AdjTile<3, double, false> { static constexpr int BX = 8, BY = 8, BZ = 4; };
+template <> struct AdjTile<2, float, false> { static constexpr int BX = 16, BY = 16, BZ = 1; };
+template <> struct AdjTile<2, double, false> { static constexpr int BX = 16, BY = 16, BZ = 1; };
+template <> struct AdjTile<2, double, true> { static constexpr int BX = 8, BY = 8, BZ = 1; };
+__host__ __device__ inline bool adj_small(int dim, int fp_bytes, const int *n) {
+    return dim == 2 && fp_bytes == 8 && (long long)((n[0] + 15) / 16) * ((n[1] + 15) / 16) < 256;
+}
 
-template <int DIM, typename T>
+template <int DIM, typename T, bool SMALL>
 struct AdjBox {
-    static constexpr int BX = AdjTile<DIM, T>::BX, BY = AdjTile<DIM, T>::BY,
-                         BZ = AdjTile<DIM, T>::BZ;
+    using Tile = AdjTile<DIM, T, SMALL>;
+    static constexpr int BX = Tile::BX, BY = Tile::BY, BZ = Tile::BZ;
     static constexpr int PX = BX + 4, PY = BY + 4, PZ = DIM == 3 ? BZ + 4 : 1;
     static constexpr int PN = PX * PY * PZ;
     static constexpr size_t SMEM = 2 * sizeof(T) * (size_t)(DIM + 2) * PN;
 };
 
-template <int DIM, int D, typename T>
-__device__ __forceinline__ void tile_faces(const GridParams &g, const AdjK<T> &k,
-                                           const T *__restrict__ V, const T *__restrict__ Wsm,
-                                           T *__restrict__ Acc, int ox, int oy, int oz) {
-    using B = AdjBox<DIM, T>;
-    using R = T;
-    constexpr int NC = DIM + 2;
-    constexpr int NT2 = ntan(DIM);
-    constexpr int PN = B::PN;
-    const int o[3] = {ox, oy, oz};
+// What the reverse of one face adds: to the 4 cells qs along its normal and
+// the 4 cells qt per tangent.
+template <int DIM, typename R>
+struct FaceAdj {
+    static constexpr int NC = DIM + 2, NT2 = ntan(DIM);
+    bool act;
+    int qs[4];
+    int qt[NT2][4];
+    R wb[4][NC];
+    R utb[NT2][4][DIM];
+};
+
+// faces of a tile normal to axis D
+template <typename B, int DIM, int D>
+__device__ __forceinline__ int face_counts(const GridParams &g, const int (&o)[3], int (&cnt)[3]) {
     const int bsz[3] = {B::BX, B::BY, B::BZ};
-    const int str[3] = {1, B::PX, B::PX * B::PY};
-    int cnt[3];
 #pragma unroll
     for (int e = 0; e < 3; ++e) {
         const int n = e < DIM ? g.n[e] : 1;
@@ -383,107 +401,154 @@ __device__ __forceinline__ void tile_faces(const GridParams &g, const AdjK<T> &k
         cnt[e] = min(b, n - o[e]);
     }
     if (o[D] + bsz[D] >= g.n[D]) cnt[D] += 1;   // the last tile owns the domain face b = n
-    const int nf = cnt[0] * cnt[1] * cnt[2];
+    return cnt[0] * cnt[1] * cnt[2];
+}
+
+// reverse of face f (of the cnt faces normal to axis D)
+template <typename B, int DIM, int D, typename T>
+__device__ __forceinline__ void reverse_face(const GridParams &g, const AdjK<T> &k,
+                                             const T *__restrict__ V, const T *__restrict__ Wsm,
+                                             const int (&o)[3], const int (&cnt)[3], int f,
+                                             FaceAdj<DIM, T> &r) {
+    using R = T;
+    constexpr int NC = DIM + 2;
+    constexpr int NT2 = ntan(DIM);
+    constexpr int PN = B::PN;
+    const int str[3] = {1, B::PX, B::PX * B::PY};
     const long long N = g.N;
-    // Faces go in batches of one per thread.  Each face adds to 4 cells along
-    // its normal and 4 cells per tangent; for one such stencil slot the map
-    // face -> cell is one-to-one, so the slots are added in a fixed order
-    // with a barrier between them and no two faces of a batch ever touch the
-    // same accumulator at once: the sums are bitwise reproducible.
-    for (int base = 0; base < nf; base += FT) {
-        const int f = base + threadIdx.x;
-        bool act = false;
-        int qs[4];
-        int qt[NT2][4];
-        R wb[4][NC];
-        R utb[NT2][4][DIM];
-        if (f < nf) {
-            int l[3];
-            l[0] = f % cnt[0];
-            l[1] = (f / cnt[0]) % cnt[1];
-            l[2] = f / (cnt[0] * cnt[1]);
-            const int gb = o[D] + l[D];
-            const bool b_in = gb < g.n[D], a_in = gb >= 1;
-            long long jb = 0, ja = 0;
-            {
-                int c[3] = {o[0] + l[0], o[1] + l[1], o[2] + l[2]};
-                jb = c[0] + (long long)g.n[0] * (c[1] + (long long)g.n[1] * c[2]);
-                c[D] -= 1;
-                ja = c[0] + (long long)g.n[0] * (c[1] + (long long)g.n[1] * c[2]);
-            }
-            R Fb[NC];
-            bool any = false;
+    int l[3];
+    l[0] = f % cnt[0];
+    l[1] = (f / cnt[0]) % cnt[1];
+    l[2] = f / (cnt[0] * cnt[1]);
+    const int gb = o[D] + l[D];
+    const bool b_in = gb < g.n[D], a_in = gb >= 1;
+    long long jb = 0, ja = 0;
+    {
+        int c[3] = {o[0] + l[0], o[1] + l[1], o[2] + l[2]};
+        jb = c[0] + (long long)g.n[0] * (c[1] + (long long)g.n[1] * c[2]);
+        c[D] -= 1;
+        ja = c[0] + (long long)g.n[0] * (c[1] + (long long)g.n[1] * c[2]);
+    }
+    R Fb[NC];
+    bool any = false;
 #pragma unroll
-            for (int q = 0; q < NC; ++q) {
-                const R vb = b_in ? V[q * N + jb] : R(0);
-                const R va = a_in ? V[q * N + ja] : R(0);
-                Fb[q] = (vb - va) * k.inv_h;
-                any |= Fb[q] != R(0);
-            }
-            if (any) {
-                act = true;
-                const int qb =
-                    (l[0] + 2) + B::PX * ((l[1] + 2) + B::PY * (DIM == 3 ? l[2] + 2 : 0));
-                const int sD = str[D];
-                R w[4][NC];
+    for (int q = 0; q < NC; ++q) {
+        const R vb = b_in ? V[q * N + jb] : R(0);
+        const R va = a_in ? V[q * N + ja] : R(0);
+        Fb[q] = (vb - va) * k.inv_h;
+        any |= Fb[q] != R(0);
+    }
+    r.act = any;
+    if (!any) return;
+    const int qb = (l[0] + 2) + B::PX * ((l[1] + 2) + B::PY * (DIM == 3 ? l[2] + 2 : 0));
+    const int sD = str[D];
+    R w[4][NC];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    qs[i] = qb + (i - 2) * sD;
+    for (int i = 0; i < 4; ++i) {
+        r.qs[i] = qb + (i - 2) * sD;
 #pragma unroll
-                    for (int c = 0; c < NC; ++c) {
-                        w[i][c] = Wsm[c * PN + qs[i]];
-                        wb[i][c] = R(0);
-                    }
-                }
-                R ut[NT2][4][DIM];
-                {
-                    int ti = 0;
-#pragma unroll
-                    for (int e = 0; e < DIM; ++e) {
-                        if (e == D) continue;
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            qt[ti][i] = (i < 2 ? qb - sD : qb) + ((i & 1) ? str[e] : -str[e]);
-#pragma unroll
-                            for (int m = 0; m < DIM; ++m) {
-                                ut[ti][i][m] = Wsm[(1 + m) * PN + qt[ti][i]];
-                                utb[ti][i][m] = R(0);
-                            }
-                        }
-                        ++ti;
-                    }
-                }
-                face_vjp<DIM, D, R>(k, w, ut, Fb, wb, utb);
-            }
+        for (int c = 0; c < NC; ++c) {
+            w[i][c] = Wsm[c * PN + r.qs[i]];
+            r.wb[i][c] = R(0);
         }
+    }
+    R ut[NT2][4][DIM];
+    {
+        int ti = 0;
+#pragma unroll
+        for (int e = 0; e < DIM; ++e) {
+            if (e == D) continue;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                r.qt[ti][i] = (i < 2 ? qb - sD : qb) + ((i & 1) ? str[e] : -str[e]);
+#pragma unroll
+                for (int m = 0; m < DIM; ++m) {
+                    ut[ti][i][m] = Wsm[(1 + m) * PN + r.qt[ti][i]];
+                    r.utb[ti][i][m] = R(0);
+                }
+            }
+            ++ti;
+        }
+    }
+    face_vjp<DIM, D, R>(k, w, ut, Fb, r.wb, r.utb);
+}
+
+// Each face adds to 4 cells along its normal and 4 cells per tangent; for one
+// such stencil slot the map face -> cell is one-to-one over the faces of one
+// axis, so the slots are added in a fixed order with a barrier between them
+// and no two faces of a batch ever touch the same accumulator at once: the
+// sums are bitwise reproducible.
+template <int DIM, typename R>
+__device__ __forceinline__ void add_slots(const FaceAdj<DIM, R> &r, bool act, R *__restrict__ Acc,
+                                          int PN) {
+    constexpr int NC = DIM + 2;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        if (act) {
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+                if (r.wb[i][c] != R(0)) Acc[c * PN + r.qs[i]] += r.wb[i][c];
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int ti = 0; ti < (DIM > 1 ? DIM - 1 : 0); ++ti)
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             if (act) {
 #pragma unroll
-                for (int c = 0; c < NC; ++c)
-                    if (wb[i][c] != R(0)) Acc[c * PN + qs[i]] += wb[i][c];
+                for (int m = 0; m < DIM; ++m)
+                    if (r.utb[ti][i][m] != R(0)) Acc[(1 + m) * PN + r.qt[ti][i]] += r.utb[ti][i][m];
             }
             __syncthreads();
         }
-#pragma unroll
-        for (int ti = 0; ti < (DIM > 1 ? DIM - 1 : 0); ++ti)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                if (act) {
-#pragma unroll
-                    for (int m = 0; m < DIM; ++m)
-                        if (utb[ti][i][m] != R(0)) Acc[(1 + m) * PN + qt[ti][i]] += utb[ti][i][m];
-                }
-                __syncthreads();
-            }
+}
+
+// all faces normal to axis D, in batches of one per thread
+template <typename B, int DIM, int D, typename T>
+__device__ __forceinline__ void tile_faces(const GridParams &g, const AdjK<T> &k,
+                                           const T *__restrict__ V, const T *__restrict__ Wsm,
+                                           T *__restrict__ Acc, int ox, int oy, int oz) {
+    const int o[3] = {ox, oy, oz};
+    int cnt[3];
+    const int nf = face_counts<B, DIM, D>(g, o, cnt);
+    for (int base = 0; base < nf; base += FT) {
+        FaceAdj<DIM, T> r;
+        r.act = false;
+        if (base + (int)threadIdx.x < nf)
+            reverse_face<B, DIM, D, T>(g, k, V, Wsm, o, cnt, base + threadIdx.x, r);
+        add_slots<DIM, T>(r, r.act, Acc, B::PN);
     }
 }
 
-template <int DIM, typename T>
-__global__ void __launch_bounds__(FT, IBM_ADJ_FT_MIN)
+// x-faces by the first half of the CTA and y-faces by the second, at once
+// (tiles of at most FT / 2 faces per axis)
+template <typename B, typename T>
+__device__ __forceinline__ void tile_faces_xy(const GridParams &g, const AdjK<T> &k,
+                                              const T *__restrict__ V, const T *__restrict__ Wsm,
+                                              T *__restrict__ Acc, int ox, int oy) {
+    static_assert((B::BX + 1) * B::BY <= FT / 2 && B::BX * (B::BY + 1) <= FT / 2, "one face per thread");
+    const int o[3] = {ox, oy, 0};
+    const bool second = threadIdx.x >= FT / 2;
+    const int f = threadIdx.x - (second ? FT / 2 : 0);
+    FaceAdj<2, T> r;
+    r.act = false;
+    int cnt[3];
+    if (!second) {
+        if (f < face_counts<B, 2, 0>(g, o, cnt)) reverse_face<B, 2, 0, T>(g, k, V, Wsm, o, cnt, f, r);
+    } else {
+        if (f < face_counts<B, 2, 1>(g, o, cnt)) reverse_face<B, 2, 1, T>(g, k, V, Wsm, o, cnt, f, r);
+    }
+    add_slots<2, T>(r, r.act && !second, Acc, B::PN);
+    add_slots<2, T>(r, r.act && second, Acc, B::PN);
+}
+
+// (FP64: one CTA per SM keeps its pipe busy, so the registers are not bounded)
+template <int DIM, typename T, bool SMALL>
+__global__ void __launch_bounds__(FT, sizeof(T) == 4 ? IBM_ADJ_FT_MIN : 1)
 adj_flux_tile_kernel(const GridParams g, const T *__restrict__ U, const T *__restrict__ V,
                      T *__restrict__ tbuf) {
-    using B = AdjBox<DIM, T>;
+    using B = AdjBox<DIM, T, SMALL>;
     using R = T;
     constexpr int NC = DIM + 2;
     constexpr int PN = B::PN;
@@ -507,9 +572,13 @@ adj_flux_tile_kernel(const GridParams g, const T *__restrict__ U, const T *__res
         }
     }
     __syncthreads();
-    tile_faces<DIM, 0, T>(g, k, V, Wsm, Acc, ox, oy, oz);
-    tile_faces<DIM, 1, T>(g, k, V, Wsm, Acc, ox, oy, oz);
-    if constexpr (DIM == 3) tile_faces<DIM, (DIM == 3 ? 2 : 0), T>(g, k, V, Wsm, Acc, ox, oy, oz);
+    if constexpr (SMALL) {
+        tile_faces_xy<B, T>(g, k, V, Wsm, Acc, ox, oy);
+    } else {
+        tile_faces<B, DIM, 0, T>(g, k, V, Wsm, Acc, ox, oy, oz);
+        tile_faces<B, DIM, 1, T>(g, k, V, Wsm, Acc, ox, oy, oz);
+        if constexpr (DIM == 3) tile_faces<B, DIM, (DIM == 3 ? 2 : 0), T>(g, k, V, Wsm, Acc, ox, oy, oz);
+    }
     __syncthreads();
     // the tile-plus-halo sums go to this tile's own slice of the buffer; the
     // chain kernel gathers them per cell in a fixed order
@@ -549,16 +618,17 @@ struct AxisCands {
     }
 };
 
-template <int DIM, typename T>
+template <int DIM, typename T, bool SMALL>
 __device__ __forceinline__ void gather_tiles(const GridParams &g, const T *__restrict__ tbuf,
                                              const int (&c)[3], T (&wv)[DIM + 2]) {
-    using B = AdjBox<DIM, T>;
+    using B = AdjBox<DIM, T, SMALL>;
     constexpr int NC = DIM + 2;
     constexpr int PN = B::PN;
     const int bs[3] = {B::BX, B::BY, B::BZ};
     const int ps[3] = {B::PX, B::PY, B::PZ};
     int nt[3] = {1, 1, 1};
     AxisCands ax[3];
+    bool more = false;     // a third box on some axis
 #pragma unroll
     for (int e = 0; e < 3; ++e) {
         if (e >= DIM) {
@@ -567,6 +637,23 @@ __device__ __forceinline__ void gather_tiles(const GridParams &g, const T *__res
         }
         const int n = g.n[e], be = bs[e];
         nt[e] = (n + be - 1) / be;
+        // away from the domain's ends no ghost is the cell's image, and the
+        // boxes holding it are its own tile's and at most one neighbour's
+        if (c[e] >= 2 && c[e] < n - 2) {
+            const unsigned te = (unsigned)(c[e] / be), l = (unsigned)(c[e] - (int)te * be);
+            const unsigned own = te << 8 | (l + 2u) << 1;
+            if (l < 2u) {   // (te > 0, since c >= 2 and be >= 4)
+                ax[e].v0 = (te - 1u) << 8 | (l + 2u + (unsigned)be) << 1;
+                ax[e].v1 = own;
+                ax[e].n = 2;
+            } else {
+                const bool up = (int)l >= be - 2 && (int)te + 1 < nt[e];
+                ax[e].v0 = own;
+                ax[e].v1 = (te + 1u) << 8 | (l + 2u - (unsigned)be) << 1;
+                ax[e].n = up ? 2 : 1;
+            }
+            continue;
+        }
         // the cell itself, then the ghost positions whose image it is
         const int cand[5] = {c[e], -2, -1, n, n + 1};
 #pragma unroll
@@ -588,30 +675,52 @@ __device__ __forceinline__ void gather_tiles(const GridParams &g, const T *__res
                 ax[e].add(((unsigned)te << 8) | ((unsigned)l << 1) | (flip ? 1u : 0u));
             }
         }
+        more |= ax[e].n > 2;
     }
 #pragma unroll
     for (int q = 0; q < NC; ++q) wv[q] = T(0);
-    for (int iz = 0; iz < ax[2].n; ++iz) {
-        const unsigned wz = ax[2].get(iz);
-        for (int iy = 0; iy < ax[1].n; ++iy) {
-            const unsigned wy = ax[1].get(iy);
-            for (int ix = 0; ix < ax[0].n; ++ix) {
-                const unsigned wx = ax[0].get(ix);
-                const size_t tile =
-                    (wx >> 8) + (size_t)nt[0] * ((wy >> 8) + (size_t)nt[1] * (wz >> 8));
-                const int q = (int)((wx >> 1) & 127u) +
-                              B::PX * ((int)((wy >> 1) & 127u) + B::PY * (int)((wz >> 1) & 127u));
-                const int flip = (int)(wx & 1u) | ((int)(wy & 1u) << 1) | ((int)(wz & 1u) << 2);
-                const T *src = tbuf + tile * NC * PN + q;
+    auto box = [&](unsigned wx, unsigned wy, unsigned wz, T (&v)[NC]) {
+        const size_t tile = (wx >> 8) + (size_t)nt[0] * ((wy >> 8) + (size_t)nt[1] * (wz >> 8));
+        const int q = (int)((wx >> 1) & 127u) +
+                      B::PX * ((int)((wy >> 1) & 127u) + B::PY * (int)((wz >> 1) & 127u));
+        const T *src = tbuf + tile * NC * PN + q;
 #pragma unroll
-                for (int cc = 0; cc < NC; ++cc) {
-                    T v = src[(size_t)cc * PN];
-                    if (cc >= 1 && cc <= DIM && ((flip >> (cc - 1)) & 1)) v = -v;
-                    wv[cc] += v;
-                }
+        for (int cc = 0; cc < NC; ++cc) v[cc] = __ldg(src + cc * PN);
+        if (wx & 1u) v[1] = -v[1];
+        if (wy & 1u) v[2] = -v[2];
+        if (DIM == 3 && (wz & 1u)) v[DIM] = -v[DIM];
+    };
+    // the first two boxes per axis: the loads of a plane of them issue together
+#pragma unroll
+    for (int iz = 0; iz < (DIM == 3 ? 2 : 1); ++iz) {
+        if (iz >= ax[2].n) break;
+        const unsigned wz = iz ? ax[2].v1 : ax[2].v0;
+        T v[4][NC];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const bool in = (i & 1) < ax[0].n && (i >> 1) < ax[1].n;
+            if (in) {
+                box(i & 1 ? ax[0].v1 : ax[0].v0, i >> 1 ? ax[1].v1 : ax[1].v0, wz, v[i]);
+            } else {
+#pragma unroll
+                for (int cc = 0; cc < NC; ++cc) v[i][cc] = T(0);
             }
         }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int cc = 0; cc < NC; ++cc) wv[cc] += v[i][cc];
     }
+    if (!more) return;
+    for (int iz = 0; iz < ax[2].n; ++iz)
+        for (int iy = 0; iy < ax[1].n; ++iy)
+            for (int ix = 0; ix < ax[0].n; ++ix) {
+                if (ix < 2 && iy < 2 && iz < 2) continue;
+                T v[NC];
+                box(ax[0].get(ix), ax[1].get(iy), ax[2].get(iz), v);
+#pragma unroll
+                for (int cc = 0; cc < NC; ++cc) wv[cc] += v[cc];
+            }
 }
 
 // w = (dW/dU)^T W-bar at every cell, W-bar gathered from the tile buffers:
@@ -620,7 +729,7 @@ __device__ __forceinline__ void gather_tiles(const GridParams &g, const T *__res
 // MODE -1 stores w in out; the reverse sweep's two SSP-RK2 updates take w
 // directly: MODE 0 mu = lam/2 + (dt/2) w, MODE 1 lam = lam/2 + mu + dt w.
 // In the grid's type throughout (double arithmetic is slow on this GPU).
-template <int DIM, typename T, int MODE>
+template <int DIM, typename T, int MODE, bool SMALL>
 __global__ void __launch_bounds__(AT)
 adj_prim_kernel(const GridParams g, const T *__restrict__ U, const T *__restrict__ tbuf,
                 T *__restrict__ out, T *__restrict__ lam, T *__restrict__ mu, double dt_d) {
@@ -644,9 +753,9 @@ adj_prim_kernel(const GridParams g, const T *__restrict__ U, const T *__restrict
             const long long nxy = (long long)g.n[0] * g.n[1];
             const int c[3] = {(int)(j % g.n[0]), (int)((j / g.n[0]) % g.n[1]),
                               DIM == 3 ? (int)(j / nxy) : 0};
-            gather_tiles<DIM, T>(g, tbuf, c, wbv);
+            gather_tiles<DIM, T, SMALL>(g, tbuf, c, wbv);
         }
-        const R rho = uc[0], inv = R(1) / rho;
+        const R inv = rcp_of(uc[0]);
         R v[DIM], ke = R(0);
 #pragma unroll
         for (int d = 0; d < DIM; ++d) {
@@ -1010,30 +1119,38 @@ int grid_for(long long work, int per_block = AT) {
 }
 
 // out = J_L(U)^T V (tbuf: the per-tile accumulators, adj_tile_buf_bytes)
-template <int DIM, typename T>
-cudaError_t rhs_vjp_t(const GridParams &g, const void *U, const void *V, void *tbuf_, void *out,
-                      cudaStream_t s, int mode = -1, void *lam = nullptr, void *mu = nullptr,
-                      double dt = 0.0) {
+template <int DIM, typename T, bool SMALL>
+cudaError_t rhs_vjp_box(const GridParams &g, const void *U, const void *V, void *tbuf_, void *out,
+                        cudaStream_t s, int mode, void *lam, void *mu, double dt) {
     const T *u = (const T *)U, *v = (const T *)V;
     T *tbuf = (T *)tbuf_;
-    using B = AdjBox<DIM, T>;
+    using B = AdjBox<DIM, T, SMALL>;
     {
-        cudaError_t e = func_smem_attr((const void *)adj_flux_tile_kernel<DIM, T>, B::SMEM);
+        cudaError_t e = func_smem_attr((const void *)adj_flux_tile_kernel<DIM, T, SMALL>, B::SMEM);
         if (e != cudaSuccess) return e;
     }
     const dim3 grid((g.n[0] + B::BX - 1) / B::BX, (g.n[1] + B::BY - 1) / B::BY,
                     DIM == 3 ? (g.n[2] + B::BZ - 1) / B::BZ : 1);
-    adj_flux_tile_kernel<DIM, T><<<grid, FT, B::SMEM, s>>>(g, u, v, tbuf);
+    adj_flux_tile_kernel<DIM, T, SMALL><<<grid, FT, B::SMEM, s>>>(g, u, v, tbuf);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int nb = grid_for(g.N);
     if (mode == 0)
-        adj_prim_kernel<DIM, T, 0><<<nb, AT, 0, s>>>(g, u, tbuf, nullptr, (T *)lam, (T *)mu, dt);
+        adj_prim_kernel<DIM, T, 0, SMALL><<<nb, AT, 0, s>>>(g, u, tbuf, nullptr, (T *)lam, (T *)mu, dt);
     else if (mode == 1)
-        adj_prim_kernel<DIM, T, 1><<<nb, AT, 0, s>>>(g, u, tbuf, nullptr, (T *)lam, (T *)mu, dt);
+        adj_prim_kernel<DIM, T, 1, SMALL><<<nb, AT, 0, s>>>(g, u, tbuf, nullptr, (T *)lam, (T *)mu, dt);
     else
-        adj_prim_kernel<DIM, T, -1><<<nb, AT, 0, s>>>(g, u, tbuf, (T *)out, nullptr, nullptr, 0.0);
+        adj_prim_kernel<DIM, T, -1, SMALL><<<nb, AT, 0, s>>>(g, u, tbuf, (T *)out, nullptr, nullptr, 0.0);
     return cudaGetLastError();
+}
+template <int DIM, typename T>
+cudaError_t rhs_vjp_t(const GridParams &g, const void *U, const void *V, void *tbuf, void *out,
+                      cudaStream_t s, int mode = -1, void *lam = nullptr, void *mu = nullptr,
+                      double dt = 0.0) {
+    if constexpr (DIM == 2 && sizeof(T) == 8)
+        if (adj_small(DIM, 8, g.n))
+            return rhs_vjp_box<DIM, T, true>(g, U, V, tbuf, out, s, mode, lam, mu, dt);
+    return rhs_vjp_box<DIM, T, false>(g, U, V, tbuf, out, s, mode, lam, mu, dt);
 }
 
 template <int DIM, typename T>
@@ -1114,8 +1231,8 @@ size_t aup(size_t x) { return (x + 255) / 256 * 256; }
 
 // bytes of the flux transpose's per-tile accumulators: every tile of the
 // reverse flux kernel keeps its tile-plus-halo sums (dim+2 fields)
-template <int DIM, typename T> size_t tile_buf_bytes_t(const int *n) {
-    using B = AdjBox<DIM, T>;
+template <int DIM, typename T, bool SMALL = false> size_t tile_buf_bytes_t(const int *n) {
+    using B = AdjBox<DIM, T, SMALL>;
     const size_t tiles = (size_t)((n[0] + B::BX - 1) / B::BX) * ((n[1] + B::BY - 1) / B::BY) *
                          (DIM == 3 ? (n[2] + B::BZ - 1) / B::BZ : 1);
     return tiles * (DIM + 2) * B::PN * sizeof(T);
@@ -1123,6 +1240,7 @@ template <int DIM, typename T> size_t tile_buf_bytes_t(const int *n) {
 size_t adj_tile_buf_bytes(const ibm_grid_desc &d) {
     if (d.dim == 3)
         return d.fp_bytes == 4 ? tile_buf_bytes_t<3, float>(d.n) : tile_buf_bytes_t<3, double>(d.n);
+    if (adj_small(d.dim, d.fp_bytes, d.n)) return tile_buf_bytes_t<2, double, true>(d.n);
     return d.fp_bytes == 4 ? tile_buf_bytes_t<2, float>(d.n) : tile_buf_bytes_t<2, double>(d.n);
 }
 

@@ -51,6 +51,7 @@ struct DoubleConsts {
     double e1, h1, s2, km, kl;     // as in FloatConsts
     double hinv_h, qinv_h;         // 1/(2h), 1/(4h)
     double E_inf;                  // free-stream rho E
+    double invR, lam_fac;          // 1/r, c_p / Pr
     double ks, kn;                 // step-size rate: (2 dim) kvisc / h^2 and mu_inf (1 + S) r^(-1/2)
                                    // with mu = kn T^2 rsqrt(T (T + S r)^2), T = p / rho
 };
@@ -111,6 +112,8 @@ inline DoubleConsts double_consts(const GridParams &g) {
     c.hinv_h = 0.5 * g.inv_h;
     c.qinv_h = 0.25 * g.inv_h;
     c.E_inf = g.p_inf / (g.gamma - 1.0) + 0.5;
+    c.invR = 1.0 / g.R;
+    c.lam_fac = g.cp / g.Pr;
     c.ks = 2.0 * g.dim * g.kvisc * g.inv_h * g.inv_h;
     c.kn = g.mu_inf * (1.0 + g.S) / sqrt(g.R);
     return c;

@@ -75,6 +75,26 @@ def test_rhs_vjp_inviscid_matches_oracle(dim, fp, tol):
     assert np.linalg.norm(out - ref) / np.linalg.norm(ref) < tol
 
 
+@pytest.mark.parametrize("bc", [MIXED, (C.BC_PERIODIC,) * 6, (C.BC_SLIP,) * 6])
+@pytest.mark.parametrize("n,fp", [((4, 4), 8), ((8, 8), 8), ((17, 9), 8), ((33, 31), 8),
+                                  ((257, 255), 8), ((4, 5), 4), ((33, 31), 4),
+                                  ((4, 4, 4), 8), ((17, 9, 5), 8), ((17, 9, 5), 4)])
+def test_rhs_vjp_around_the_tiles(n, fp, bc):
+    """v^T dL/dU around the edges of the reverse flux kernels' tiles (8 x 8 on
+    small FP64 grids, 16 x 16, 8 x 8 x 4), with the tolerances of
+    test_rhs_vjp_matches_oracle"""
+    g = C.small_grid(len(n), n, h=0.1, fp_bytes=fp, Re=60.0, Mach=0.4, bc=bc)
+    dt_ = np.float32 if fp == 4 else np.float64
+    U = C.random_state(g, seed=31, amp=0.05).astype(dt_)
+    V = np.random.default_rng(7).standard_normal(U.shape).astype(dt_)
+    grid = ibm.Grid(g)
+    grid.record(1, 1)
+    out = grid.rhs_vjp(torch.from_numpy(U), torch.from_numpy(V)).cpu().numpy()
+    grid.close()
+    ref = adj().rhs_vjp(g, U.astype(np.float64), V.astype(np.float64))
+    assert np.linalg.norm(out - ref) / np.linalg.norm(ref) < (1e-11 if fp == 8 else 2e-4)
+
+
 def cylinder(fp, n=(40, 32), h=0.1):
     g = C.small_grid(2, n, h=h, fp_bytes=fp, Re=100.0, Mach=0.3)
     X = C.circle_markers(int(np.ceil(np.pi / h)), 0.5, (0.05, -0.03))
