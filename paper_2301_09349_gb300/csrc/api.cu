@@ -643,7 +643,8 @@ ibm_status run_steps(ibm_grid *g, int nsteps, double dt_fixed, cudaStream_t s) {
                                     g->fb.dt, dt_fixed, g->side),
                "motion + bins");
             CU(cudaEventRecord(g->ev_bins, g->side), "bins");
-            CU(launch_quadrature(g->gp, g->mb, g->qb, g->cg_tol, g->cg_maxit, 1, g->side, 1),
+            CU(launch_quadrature(g->gp, g->mb, g->qb, g->cg_tol, g->cg_maxit, 1, g->side,
+                                 small_rebuild_weights(g->gp, g->mb)),
                "quadrature");
             CU(prof_end(g, rec, g->side), "profile");
             CU(cudaEventRecord(g->ev_quad, g->side), "weights");

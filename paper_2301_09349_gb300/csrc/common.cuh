@@ -146,11 +146,15 @@ __device__ __forceinline__ bool dpos(double x) {
 
 // The 1D regularised 3-point delta of Sec. 2.2 (Pinelli et al.); r in cells.
 __device__ __forceinline__ double phi_d(double r) {
-    double a = fabs(r);
-    if (a <= 0.5) return (1.0 + sqrt(1.0 - 3.0 * a * a)) * (1.0 / 3.0);
+    // (the roots are of values in [1/4, 1])
+    const double a = fabs(r);
+    if (a <= 0.5) {
+        const double x = 1.0 - 3.0 * a * a;
+        return (1.0 + x * drsqrt(x)) * (1.0 / 3.0);
+    }
     if (a <= 1.5) {
-        double b = 1.0 - a;
-        return (5.0 - 3.0 * a - sqrt(1.0 - 3.0 * b * b)) * (1.0 / 6.0);
+        const double b = 1.0 - a, x = 1.0 - 3.0 * b * b;
+        return (5.0 - 3.0 * a - x * drsqrt(x)) * (1.0 / 6.0);
     }
     return 0.0;
 }

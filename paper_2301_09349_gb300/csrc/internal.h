@@ -194,6 +194,8 @@ cudaError_t launch_motion(const GridParams &g, const MarkerBuffers &m, double am
 // markers in one launch (motion, bins, forced cells, tile lists); the
 // quadrature follows separately
 constexpr int kSmallRebuildNs = 512;
+// whether that launch also tabulates the support weights (have_weights below)
+int small_rebuild_weights(const GridParams &g, const MarkerBuffers &m);
 cudaError_t launch_small_rebuild(const GridParams &g, MarkerBuffers &m, double amp, double freq,
                                  int axis, const double *dt, double dt_fixed, cudaStream_t s);
 // forced-cell bits and band-tile flags scattered from the markers' supports,

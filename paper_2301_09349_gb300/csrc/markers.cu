@@ -198,20 +198,30 @@ __device__ __forceinline__ void tile_lists(int n_tiles, const int *__restrict__ 
                                            const int *__restrict__ band, int *__restrict__ occ_list,
                                            int *__restrict__ band_list, int *__restrict__ counts,
                                            int *s_warp) {
-    const int chunk = (n_tiles + SORT_T - 1) / SORT_T;
-    const int t0 = threadIdx.x * chunk, t1 = min(n_tiles, t0 + chunk);
+    // each thread's run of tiles in 16-byte words (a run starts at a multiple
+    // of four; the flag arrays are 256-byte aligned): 68 -> 13 us at
+    // 32768 tiles
+    const int chunk = ((n_tiles + SORT_T - 1) / SORT_T + 3) / 4 * 4;
+    const int t0 = min(n_tiles, (int)threadIdx.x * chunk), t1 = min(n_tiles, t0 + chunk);
+    auto four = [&](const int *f, int t) {
+        if (t + 4 <= t1) return *reinterpret_cast<const int4 *>(f + t);
+        return make_int4(f[t], t + 1 < t1 ? f[t + 1] : 0, t + 2 < t1 ? f[t + 2] : 0, 0);
+    };
     int co = 0, cb = 0;
-    for (int t = t0; t < t1; ++t) {
-        co += occ[t];
-        cb += band[t];
+#pragma unroll 4
+    for (int t = t0; t < t1; t += 4) {
+        const int4 o = four(occ, t), n = four(band, t);
+        co += o.x + o.y + o.z + o.w;
+        cb += n.x + n.y + n.z + n.w;
     }
     int to, tb;
     int eo = block_exclusive_scan(co, s_warp, to);
     int eb = block_exclusive_scan(cb, s_warp, tb);
-    for (int t = t0; t < t1; ++t) {
-        if (occ[t]) occ_list[eo++] = t;
-        if (band[t]) band_list[eb++] = t;
-    }
+    if (co | cb)
+        for (int t = t0; t < t1; ++t) {
+            if (occ[t]) occ_list[eo++] = t;
+            if (band[t]) band_list[eb++] = t;
+        }
     if (threadIdx.x == 0) {
         counts[0] = to;
         counts[1] = tb;
@@ -268,37 +278,42 @@ __global__ void motion_kernel(const GridParams g, int ns, const double *__restri
 // must hold exactly the previous marker set's forced cells on entry (it
 // clears them first, from the previous owner cells, instead of a memset of
 // the whole mask); the sorted order goes to keys[0] / perm[0].
-// Support cell sc (0 .. 3^d - 1, x fastest) of marker k from its owner cell:
-// its index in j, false when it lies outside the grid.
-__device__ __forceinline__ bool support_cell(const GridParams &g, const MarkerBuffers &m, int k,
-                                             int sc, long long &j) {
-    const int o[3] = {sc % 3 - 1, (sc / 3) % 3 - 1, g.dim == 3 ? sc / 9 - 1 : 0};
-    int c[3] = {0, 0, 0};
-    for (int d = 0; d < g.dim; ++d) {
-        c[d] = m.cell[(long long)k * 3 + d] + o[d];
-        if (c[d] < 0 || c[d] >= g.n[d]) return false;
-    }
-    j = c[0] + (long long)g.n[0] * (c[1] + (long long)g.n[1] * c[2]);
-    return in_bounds(j, g.N, m.err);
-}
-
 constexpr int SMALL_NS = kSmallRebuildNs;
 static_assert(SMALL_NS <= SORT_T, "one marker per thread");
 __global__ void __launch_bounds__(SORT_T)
 small_rebuild_kernel(const GridParams g, const MarkerBuffers m, double amp, double freq, int axis,
-                     const double *__restrict__ dt, double dt_fixed) {
+                     const double *__restrict__ dt, double dt_fixed, int with_weights) {
     __shared__ unsigned s_key[SMALL_NS];
     __shared__ unsigned s_sorted[SMALL_NS];
     __shared__ int s_warp[33];
+    __shared__ int s_cell[SMALL_NS * 3];
     __shared__ double s_mv[2];
     const int tid = threadIdx.x, ns = m.ns;
     const int nsc = g.dim == 3 ? 27 : 9;
+    // support cell i % 3^d of marker i / 3^d, owner cells in shared memory (a
+    // global load per cell and the divisions that take a cell index apart made
+    // two thirds of this kernel)
+    auto support = [&](int i, int (&c)[3]) {
+        const int k = g.dim == 3 ? i / 27 : i / 9, l = i - k * nsc;
+        c[0] = s_cell[3 * k] + l % 3 - 1;
+        c[1] = s_cell[3 * k + 1] + (l / 3) % 3 - 1;
+        c[2] = g.dim == 3 ? s_cell[3 * k + 2] + l / 9 - 1 : 0;
+        return (unsigned)c[0] < (unsigned)g.n[0] && (unsigned)c[1] < (unsigned)g.n[1] &&
+               (unsigned)c[2] < (unsigned)g.n[2];
+    };
+    auto cell_index = [&](const int (&c)[3]) {
+        return c[0] + (long long)g.n[0] * (c[1] + (long long)g.n[1] * c[2]);
+    };
+    for (int i = tid; i < 3 * ns; i += SORT_T) s_cell[i] = m.cell[i];
     if (tid == 0) motion_offset(amp, freq, m.t, dt, dt_fixed, s_mv[0], s_mv[1]);
     // the previous forced cells off (the same support cells the scatter
     // below sets, from the owner cells of the previous step)
+    __syncthreads();
     for (int i = tid; i < ns * nsc; i += SORT_T) {
-        long long j;
-        if (support_cell(g, m, i / nsc, i % nsc, j)) atomicAnd(m.band_bits + (j >> 5), ~(1u << (j & 31)));
+        int c[3];
+        if (!support(i, c)) continue;
+        const long long j = cell_index(c);
+        if (in_bounds(j, g.N, m.err)) atomicAnd(m.band_bits + (j >> 5), ~(1u << (j & 31)));
     }
     __syncthreads();
     int bad = 0;
@@ -310,9 +325,11 @@ small_rebuild_kernel(const GridParams g, const MarkerBuffers m, double amp, doub
             m.Ub[q] = m.Ub0[q] + (d == axis ? s_mv[1] : 0.0);
         }
         s_key[k] = owner_cell(g, m.X, k, m.cell, m.frac_d, m.frac_f, bad);
+        for (int d = 0; d < 3; ++d) s_cell[3 * k + d] = m.cell[3ll * k + d];
         // the marker's 1D support weights for the assembly (those of
-        // support_weights_kernel, which the quadrature then skips)
-        for (int d = 0; d < g.dim; ++d) {
+        // support_weights_kernel, which the quadrature then skips); many
+        // markers leave them to that kernel, which has every SM's FP64 pipe
+        for (int d = 0; with_weights && d < g.dim; ++d) {
             const double fk = m.frac_d[(long long)k * 3 + d];
 #pragma unroll
             for (int i = 0; i < 3; ++i)
@@ -354,12 +371,13 @@ small_rebuild_kernel(const GridParams g, const MarkerBuffers m, double amp, doub
     __syncthreads();
     // forced cells: the 3^d support cells of every marker
     for (int i = tid; i < ns * nsc; i += SORT_T) {
-        long long j;
-        if (!support_cell(g, m, i / nsc, i % nsc, j)) continue;
+        int c[3];
+        if (!support(i, c)) continue;
+        const long long j = cell_index(c);
+        if (!in_bounds(j, g.N, m.err)) continue;
         atomicOr(m.band_bits + (j >> 5), 1u << (j & 31));
-        const int cx = (int)(j % g.n[0]), cy = (int)((j / g.n[0]) % g.n[1]),
-                  cz = (int)(j / ((long long)g.n[0] * g.n[1]));
-        m.band_flag[cell_key(g, cx, cy, cz) / cpt] = 1;
+        m.band_flag[c[0] / g.tile[0] +
+                    g.ntile[0] * (c[1] / g.tile[1] + g.ntile[1] * (c[2] / g.tile[2]))] = 1;
     }
     __syncthreads();
     tile_lists(g.n_tiles, m.occ_flag, m.band_flag, m.occ_list, m.band_list, m.counts, s_warp);
@@ -385,25 +403,67 @@ __device__ __forceinline__ void interp_fields(const R *__restrict__ U, long long
     v[DIM + 1] = U[(DIM + 1) * N + j] - R(0.5) * rdiv<R>(ke, rho);
 }
 
-// rho_L and the forcing of marker k from its interpolated sums (lane 0):
-// G = dt F = rho_L U_b - I[rho u], H = dt Q = rho_L c_v T_w - I[rho e].
-template <int DIM, typename R>
-__device__ __forceinline__ void store_forcing(const GridParams &g, const MarkerBuffers &m, int k,
-                                              const R (&acc)[DIM + 2]) {
-    const double rk = (double)acc[0];
-    const double e = m.eps[k];
-    R *gs = reinterpret_cast<R *>(m.gs) + 4 * (long long)k;
-    m.rhoL[k] = rk;
+// Interpolation and forcing of marker k by one warp, lane l on support cell l
+// (Eqs. interp, forceMomentum, corr3.8): rho_L, G = dt F = rho_L U_b -
+// I[rho u], H = dt Q = rho_L c_v T_w - I[rho e], and the eps~-scaled forcing in
+// the field precision.  A chain of latencies: the cell's values are loaded
+// ahead of the weights (FP64 grids take the tabulated ones, an FP64 square
+// root costs a warp a thousand cycles), the sums share their butterflies, and
+// lane d forms component d.  Heated cylinder (FP64) 10.5 -> 5.6 us.
+template <int DIM> __device__ __forceinline__ float support_weight(const MarkerBuffers &m, int k,
+                                                                   const int (&o)[3], float) {
+    float w = 1.0f;
 #pragma unroll
-    for (int d = 0; d < DIM; ++d) {
-        const double Gd = rk * m.Ub[(long long)k * DIM + d] - (double)acc[1 + d];
-        m.G[(long long)k * DIM + d] = Gd;
-        gs[d] = (R)(Gd * e);
+    for (int d = 0; d < DIM; ++d) w *= phi_r<float>(cell_offset<float>(o[d], marker_frac<float>(m, k, d)));
+    return w;
+}
+template <int DIM> __device__ __forceinline__ double support_weight(const MarkerBuffers &m, int k,
+                                                                    const int (&o)[3], double) {
+    double w = 1.0;
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) w *= __ldg(m.wphi + (long long)k * 9 + d * 3 + o[d] + 1);
+    return w;
+}
+template <int DIM, typename R>
+__device__ __forceinline__ void interp_marker(const GridParams &g, const MarkerBuffers &m,
+                                              const R *__restrict__ U, int k, int lane) {
+    constexpr int NS = DIM == 3 ? 27 : 9;
+    const int o[3] = {lane % 3 - 1, (lane / 3) % 3 - 1, DIM == 3 ? lane / 9 - 1 : 0};
+    R v[DIM + 2];
+#pragma unroll
+    for (int f = 0; f < DIM + 2; ++f) v[f] = R(0);
+    if (lane < NS) {
+        int c[3] = {0, 0, 0};
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) c[d] = m.cell[(long long)k * 3 + d] + o[d];
+        const long long j = c[0] + (long long)g.n[0] * (c[1] + (long long)g.n[1] * c[2]);
+        if (in_bounds(j, g.N, m.err)) {
+            interp_fields<DIM, R>(U, g.N, j, v);
+            const R w = support_weight<DIM>(m, k, o, R(0));
+#pragma unroll
+            for (int f = 0; f < DIM + 2; ++f) v[f] *= w;
+        }
     }
-    if (DIM == 2) gs[2] = R(0);
-    const double H = rk * g.cv * m.Tw[k] - (double)acc[DIM + 1];
-    m.H[k] = H;
-    gs[3] = (R)(H * e);
+    // lane d < DIM: U_b of component d; lane 3: c_v T_w
+    double target = 0.0;
+    const double e = __ldg(m.eps + k);
+    if (lane < DIM) target = m.Ub[(long long)k * DIM + lane];
+    else if (lane == 3) target = g.cv * m.Tw[k];
+    R s[4] = {v[0], v[1], v[2], v[3]};
+    warp_sum4<R>(s, lane);
+    R en = s[3];
+    if (DIM == 3) en = warp_sum_r<R>(v[DIM + 1]);
+    const double rk = (double)s[0];
+    const R mine = lane == 0 ? s[1] : lane == 1 ? s[2] : lane == 2 && DIM == 3 ? s[3] : en;
+    if (lane < 4) {
+        R *gs = reinterpret_cast<R *>(m.gs) + 4 * (long long)k;
+        const double q = rk * target - (double)mine;
+        const bool real = lane < DIM || lane == 3;
+        gs[lane] = real ? (R)(q * e) : R(0);
+        if (lane < DIM) m.G[(long long)k * DIM + lane] = q;
+        if (lane == 3) m.H[k] = q;
+        if (lane == 0) m.rhoL[k] = rk;
+    }
 }
 
 // Batched form: one warp per (case, marker) item, the 3^DIM support cells
@@ -414,8 +474,6 @@ __global__ void __launch_bounds__(512)
 batch_interp_kernel(const BatchCase *__restrict__ cases, const int2 *__restrict__ items,
                     int n_items) {
     using R = T;
-    constexpr int NF = DIM + 2;
-    constexpr int NS = DIM == 3 ? 27 : 9;
     const int lane = threadIdx.x & 31;
     const int nw = blockDim.x >> 5;
     for (int it = blockIdx.x * nw + (threadIdx.x >> 5); it < n_items; it += gridDim.x * nw) {
@@ -424,31 +482,7 @@ batch_interp_kernel(const BatchCase *__restrict__ cases, const int2 *__restrict_
         const GridParams &g = bc.g;
         const MarkerBuffers &m = bc.m;
         const R *U = (const R *)bc.Us;
-        const int k = w.y;
-        R fr[3] = {R(0), R(0), R(0)};
-        int ck[3] = {0, 0, 0};
-#pragma unroll
-        for (int d = 0; d < DIM; ++d) {
-            ck[d] = m.cell[(long long)k * 3 + d];
-            fr[d] = marker_frac<R>(m, k, d);
-        }
-        R acc[NF];
-#pragma unroll
-        for (int f = 0; f < NF; ++f) acc[f] = R(0);
-        if (lane < NS) {
-            int cell[3];
-            const R wgt = lane_weight<DIM, R>(fr, ck, lane, cell);
-            const long long j = cell[0] + (long long)g.n[0] * (cell[1] + (long long)g.n[1] * cell[2]);
-            R v[NF];
-            if (in_bounds(j, g.N, m.err)) {
-                interp_fields<DIM, R>(U, g.N, j, v);
-#pragma unroll
-                for (int f = 0; f < NF; ++f) acc[f] = wgt * v[f];
-            }
-        }
-#pragma unroll
-        for (int f = 0; f < NF; ++f) acc[f] = warp_sum_r<R>(acc[f]);
-        if (lane == 0) store_forcing<DIM, R>(g, m, k, acc);
+        interp_marker<DIM, R>(g, m, U, w.y, lane);
     }
 }
 
@@ -462,36 +496,9 @@ batch_interp_kernel(const BatchCase *__restrict__ cases, const int2 *__restrict_
 template <int DIM, typename T>
 __global__ void __launch_bounds__(256)
 interp_direct_kernel(const GridParams g, const T *__restrict__ U, const MarkerBuffers m) {
-    using R = T;
-    constexpr int NF = DIM + 2;
-    constexpr int NS = DIM == 3 ? 27 : 9;
-    const int lane = threadIdx.x & 31;
     const int k = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
     if (k >= m.ns) return;
-    R fr[3] = {R(0), R(0), R(0)};
-    int ck[3] = {0, 0, 0};
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) {
-        ck[d] = m.cell[(long long)k * 3 + d];
-        fr[d] = marker_frac<R>(m, k, d);
-    }
-    R acc[NF];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) acc[f] = R(0);
-    if (lane < NS) {
-        int cell[3];
-        const R wgt = lane_weight<DIM, R>(fr, ck, lane, cell);
-        const long long j = cell[0] + (long long)g.n[0] * (cell[1] + (long long)g.n[1] * cell[2]);
-        R v[NF];
-        if (in_bounds(j, g.N, m.err)) {
-            interp_fields<DIM, R>(U, g.N, j, v);
-#pragma unroll
-            for (int f = 0; f < NF; ++f) acc[f] = wgt * v[f];
-        }
-    }
-#pragma unroll
-    for (int f = 0; f < NF; ++f) acc[f] = warp_sum_r<R>(acc[f]);
-    if (lane == 0) store_forcing<DIM, R>(g, m, k, acc);
+    interp_marker<DIM, T>(g, m, U, k, threadIdx.x & 31);
 }
 
 // ---------------------------------------------------------------------------
@@ -509,6 +516,9 @@ size_t spread_smem_bytes(const GridParams &g) {
     const size_t bn = (size_t)(g.tile[0] + 2) * (g.tile[1] + 2) * (g.dim == 3 ? g.tile[2] + 2 : 1);
     return SP_MAXC * (7 * sizeof(R) + 2 * sizeof(int)) + 2 * bn * sizeof(int);
 }
+
+__device__ __forceinline__ float quot(float a, float b) { return a / b; }
+__device__ __forceinline__ double quot(double a, double b) { return a * drcp(b); }
 
 // Forced update of one band cell (App. B, Eqs. u_centralF2 and e_centralF2;
 // f.u dropped): momentum += dt f, internal energy += dt q, rho unchanged, so
@@ -529,9 +539,9 @@ __device__ __forceinline__ void force_cell(const GridParams &g, R (&u)[DIM + 2],
         u[1 + d] = m1;
     }
     const R E = u[DIM + 1];
-    const R qmin = -(R)kHeatSourceCap * (E - R(0.5) * ke0 / rho);
+    const R qmin = -(R)kHeatSourceCap * (E - quot(R(0.5) * ke0, rho));
     if (qh < qmin) qh = qmin;
-    u[DIM + 1] = g.energy_reading == 1 ? E + qh : E + (qh + R(0.5) * dke / rho);
+    u[DIM + 1] = g.energy_reading == 1 ? E + qh : E + (qh + quot(R(0.5) * dke, rho));
 }
 
 template <int DIM, typename T, typename R>
@@ -936,6 +946,11 @@ __device__ __forceinline__ void spread_static_cell(const GridParams &g, T *__res
 // terms and the order of spread_tile, so the results are bitwise the same),
 // then applies the forcing.  One step-size maximum per CTA in bandmax.
 constexpr int SPS_T = 256;
+// the first cell of a thread: runs of 32 cells go to the CTAs in turn, so that
+// few cells still meet as many FP64 pipes as there are runs
+__device__ __forceinline__ int static_cell0(int tid) {
+    return (int)(blockIdx.x + gridDim.x * (tid >> 5)) * 32 + (tid & 31);
+}
 template <int DIM, typename T>
 __global__ void __launch_bounds__(SPS_T)
 spread_static_kernel(const GridParams g, T *__restrict__ U, const MarkerBuffers m) {
@@ -943,7 +958,7 @@ spread_static_kernel(const GridParams g, T *__restrict__ U, const MarkerBuffers 
     const int nc = min(m.counts[2], m.sp_cap);
     T smax = T(0);
     bool ok = true;
-    for (int i = blockIdx.x * SPS_T + threadIdx.x; i < nc; i += gridDim.x * SPS_T)
+    for (int i = static_cell0(threadIdx.x); i < nc; i += gridDim.x * SPS_T)
         spread_static_cell<DIM, T>(g, U, m, i, smax, ok);
 #pragma unroll
     for (int o2 = 16; o2 > 0; o2 >>= 1) smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, o2));
@@ -1056,12 +1071,12 @@ constexpr int FIN_T = 256;   // threads of the batch finish and of the stage-1 s
 // A warp's five partials (sums 0..3, maximum 4) combined as a fixed
 // shuffle tree; the result in every lane.
 __device__ __forceinline__ void finish_combine(double a[5]) {
+    double v[4] = {a[0], a[1], a[2], a[3]};
+    warp_sum4<double>(v, threadIdx.x & 31);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int i = 0; i < 4; ++i) a[i] = v[i];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) a[i] += __shfl_xor_sync(0xffffffffu, a[i], o);
-        a[4] = dmax_nonneg(a[4], __shfl_xor_sync(0xffffffffu, a[4], o));
-    }
+    for (int o = 16; o > 0; o >>= 1) a[4] = dmax_nonneg(a[4], __shfl_xor_sync(0xffffffffu, a[4], o));
 }
 
 // The finish of a grid splits its markers (and its maxima) into C chunks,
@@ -1141,16 +1156,21 @@ __device__ __forceinline__ void finish_chunk(const GridParams &g, const MarkerBu
 __device__ __forceinline__ void finish_update(const GridParams &g, const MarkerBuffers &m,
                                               const double a[5], double *__restrict__ dt_ptr,
                                               int *__restrict__ err, double dt_fixed) {
-    for (int i = 0; i < 4; ++i) {
-        // forcing per stage: the first stage's sources count with weight 1/2
-        m.sums[i] = g.forcing_per_stage ? a[i] + 0.5 * m.sums[8 + i] : a[i];
-    }
-    const double mx = a[4];
+    // every load ahead of the first store: one latency instead of five
     const double dt_used = dt_fixed > 0.0 ? dt_fixed : *dt_ptr;
+    const double t = *m.t;
+    const long long steps = *m.steps;
+    const int e = __ldcg(err);
+    double first[4] = {0.0, 0.0, 0.0, 0.0};
+    if (g.forcing_per_stage)
+        for (int i = 0; i < 4; ++i) first[i] = m.sums[8 + i];
+    // forcing per stage: the first stage's sources count with weight 1/2
+    for (int i = 0; i < 4; ++i) m.sums[i] = g.forcing_per_stage ? a[i] + 0.5 * first[i] : a[i];
+    const double mx = a[4];
     m.sums[4] = dt_used;
-    *m.t += dt_used;
-    *m.steps += 1;
-    const bool good = mx > 0.0 && mx <= DBL_MAX && !(__ldcg(err) & ERR_NONFINITE);
+    *m.t = t + dt_used;
+    *m.steps = steps + 1;
+    const bool good = mx > 0.0 && mx <= DBL_MAX && !(e & ERR_NONFINITE);
     if (!good) record_error(err, ERR_NONFINITE);
     *dt_ptr = good ? g.cfl / mx : 0.0;
 }
@@ -1230,7 +1250,7 @@ spread_static_finish_kernel(const GridParams g, T *__restrict__ U, const MarkerB
     __shared__ int s_last;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int ns = m.ns, Cm = finish_chunks(ns);
-    if ((int)blockIdx.x < Cm && w == 0) {
+    if ((int)blockIdx.x < Cm && w == SPS_T / 32 - 1) {
         double a[5];
         finish_chunk(g, m, finish_cut(ns, blockIdx.x, Cm), finish_cut(ns, blockIdx.x + 1, Cm),
                      f.blockmax, 0, 0, m.bandmax, 0, 0, lane, a);
@@ -1240,7 +1260,7 @@ spread_static_finish_kernel(const GridParams g, T *__restrict__ U, const MarkerB
     const int nc = min(m.counts[2], m.sp_cap);
     T smax = T(0);
     bool ok = true;
-    for (int i = blockIdx.x * SPS_T + tid; i < nc; i += gridDim.x * SPS_T)
+    for (int i = static_cell0(tid); i < nc; i += gridDim.x * SPS_T)
         spread_static_cell<DIM, T>(g, U, m, i, smax, ok);
 #pragma unroll
     for (int o2 = 16; o2 > 0; o2 >>= 1) smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, o2));
@@ -1382,25 +1402,64 @@ surface_pressure_kernel(const GridParams g, const T *__restrict__ U, const Marke
     if (lane == 0) m.cp[k] = 2.0 * (acc - g.p_inf);
 }
 
+// one warp per marker, lane l on support cell l; the nc fields one after the
+// other (128^3, 5 fields: 36 -> 8.4 us against one thread per marker summing
+// into global memory)
 template <int DIM, typename T>
-__global__ void interpolate_op_kernel(const GridParams g, const T *__restrict__ field, int nc,
-                                      const MarkerBuffers m, double *__restrict__ out) {
+__global__ void __launch_bounds__(256)
+interpolate_op_kernel(const GridParams g, const T *__restrict__ field, int nc,
+                      const MarkerBuffers m, double *__restrict__ out) {
     using R = T;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= m.ns) return;
-    R fr[3] = {R(0), R(0), R(0)};
-    int ck[3] = {0, 0, 0};
-    for (int d = 0; d < DIM; ++d) {
-        ck[d] = m.cell[(long long)k * 3 + d];
-        fr[d] = marker_frac<R>(m, k, d);
-    }
-    for (int c = 0; c < nc; ++c) out[(long long)k * nc + c] = 0.0;
     constexpr int NS = DIM == 3 ? 27 : 9;
-    for (int l = 0; l < NS; ++l) {
-        int cell[3];
-        const double w = (double)lane_weight<DIM, R>(fr, ck, l, cell);
-        const long long j = cell[0] + (long long)g.n[0] * (cell[1] + (long long)g.n[1] * cell[2]);
-        for (int c = 0; c < nc; ++c) out[(long long)k * nc + c] += w * (double)field[c * g.N + j];
+    const int lane = threadIdx.x & 31;
+    const int k = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5);
+    if (k >= m.ns) return;
+    double w = 0.0;
+    long long j = 0;
+    if (lane < NS) {
+        R fr[3] = {R(0), R(0), R(0)};
+        int ck[3] = {0, 0, 0}, cell[3];
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) {
+            ck[d] = m.cell[(long long)k * 3 + d];
+            fr[d] = marker_frac<R>(m, k, d);
+        }
+        w = (double)lane_weight<DIM, R>(fr, ck, lane, cell);
+        j = cell[0] + (long long)g.n[0] * (cell[1] + (long long)g.n[1] * cell[2]);
+    }
+    for (int c = 0; c < nc; ++c) {
+        const double v = warp_sum_r<double>(lane < NS ? w * (double)field[c * g.N + j] : 0.0);
+        if (lane == 0) out[(long long)k * nc + c] = v;
+    }
+}
+
+// Spreading of nc marker quantities through the operator of static markers:
+// one thread per forced cell, its entries in the stored (gather) order, four
+// quantities at a time.  128^3, 4 quantities: 269 -> 9.1 us against the gather
+// below, which searches the bins of 27 cells per cell and quantity.
+template <typename T>
+__global__ void __launch_bounds__(128)
+spread_op_static_kernel(const GridParams g, const double *__restrict__ R_, int nc,
+                        const MarkerBuffers m, T *__restrict__ out) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= min(m.counts[2], m.sp_cap)) return;
+    const SpreadCell rc = m.sp_cell[i];
+    if (rc.n <= 0 || !in_bounds(rc.j, g.N, m.err)) return;
+    const T *ew = reinterpret_cast<const T *>(m.sp_w);
+    for (int c0 = 0; c0 < nc; c0 += 4) {
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+        for (int p = rc.start; p < rc.start + rc.n; ++p) {
+            const int k = in_bounds(p, m.sp_cap, m.err) ? __ldg(m.sp_k + p) : -1;
+            if (k < 0 || !in_bounds(k, m.ns, m.err)) continue;
+            const double w = (double)__ldg(ew + p) * __ldg(m.eps + k);
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (c0 + c < nc) acc[c] += __ldg(R_ + (long long)k * nc + c0 + c) * w;
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if (c0 + c < nc) out[(c0 + c) * g.N + rc.j] = (T)acc[c];
     }
 }
 
@@ -1447,11 +1506,20 @@ cudaError_t launch_motion(const GridParams &g, const MarkerBuffers &m, double am
     return cudaGetLastError();
 }
 
+// One CTA forms ~25 weights a microsecond beside its other work; the launch
+// that spreads them over all SMs takes 4 us (388 markers in 3D, 3492 weights:
+// the rebuild takes 17 us more with them; 98 in 2D, 588, leave
+// it at 16).
+int small_rebuild_weights(const GridParams &g, const MarkerBuffers &m) {
+    return m.ns * g.dim * 3 <= 600;
+}
+
 cudaError_t launch_small_rebuild(const GridParams &g, MarkerBuffers &m, double amp, double freq,
                                  int axis, const double *dt, double dt_fixed, cudaStream_t s) {
     if (m.ns <= 0 || m.ns > SMALL_NS) return cudaErrorInvalidValue;
     m.sorted = 0;
-    small_rebuild_kernel<<<1, SORT_T, 0, s>>>(g, m, amp, freq, axis, dt, dt_fixed);
+    small_rebuild_kernel<<<1, SORT_T, 0, s>>>(g, m, amp, freq, axis, dt, dt_fixed,
+                                              small_rebuild_weights(g, m));
     return cudaGetLastError();
 }
 
@@ -1503,10 +1571,19 @@ template <int DIM, typename T>
 static cudaError_t spread_apply_t(const GridParams &g, void *U, const MarkerBuffers &m,
                                   int grid_ctas, cudaStream_t s, const FinishArgs *fin) {
     if (m.sp_ready) {
+        // a CTA per run of 32 cells up to one per SM, then one per 256 cells
+        // (at most 3^d per marker), and the marker chunks of the finish: 608
+        // CTAs for the ~200 cells of a small cylinder spent their time on the
+        // ticket, one CTA on its FP64 pipe (16.0 and 12.6 us; now 12.1, a
+        // chain of latencies)
+        const long long cells = (DIM == 3 ? 27ll : 9ll) * m.ns;
+        const long long runs = std::min<long long>((cells + 31) / 32, 152);
+        const int ctas = (int)std::min<long long>(
+            grid_ctas, std::max<long long>({runs, (cells + SPS_T - 1) / SPS_T, finish_chunks(m.ns)}));
         if (fin)
-            spread_static_finish_kernel<DIM, T><<<grid_ctas, SPS_T, 0, s>>>(g, (T *)U, m, *fin);
+            spread_static_finish_kernel<DIM, T><<<ctas, SPS_T, 0, s>>>(g, (T *)U, m, *fin);
         else
-            spread_static_kernel<DIM, T><<<grid_ctas, SPS_T, 0, s>>>(g, (T *)U, m);
+            spread_static_kernel<DIM, T><<<ctas, SPS_T, 0, s>>>(g, (T *)U, m);
         return cudaGetLastError();
     }
     if (fin) return cudaErrorInvalidValue;
@@ -1671,17 +1748,17 @@ cudaError_t launch_surface_pressure(const GridParams &g, int fp_bytes, const voi
 cudaError_t launch_interpolate_op(const GridParams &g, int fp_bytes, const void *field, int nc,
                                   const MarkerBuffers &m, double *out, cudaStream_t s) {
     if (m.ns <= 0) return cudaSuccess;
-    const int nb = (m.ns + 127) / 128;
+    const unsigned nb = (unsigned)((32ll * m.ns + 255) / 256);
     if (g.dim == 3) {
         if (fp_bytes == 4)
-            interpolate_op_kernel<3, float><<<nb, 128, 0, s>>>(g, (const float *)field, nc, m, out);
+            interpolate_op_kernel<3, float><<<nb, 256, 0, s>>>(g, (const float *)field, nc, m, out);
         else
-            interpolate_op_kernel<3, double><<<nb, 128, 0, s>>>(g, (const double *)field, nc, m, out);
+            interpolate_op_kernel<3, double><<<nb, 256, 0, s>>>(g, (const double *)field, nc, m, out);
     } else {
         if (fp_bytes == 4)
-            interpolate_op_kernel<2, float><<<nb, 128, 0, s>>>(g, (const float *)field, nc, m, out);
+            interpolate_op_kernel<2, float><<<nb, 256, 0, s>>>(g, (const float *)field, nc, m, out);
         else
-            interpolate_op_kernel<2, double><<<nb, 128, 0, s>>>(g, (const double *)field, nc, m, out);
+            interpolate_op_kernel<2, double><<<nb, 256, 0, s>>>(g, (const double *)field, nc, m, out);
     }
     return cudaGetLastError();
 }
@@ -1692,6 +1769,14 @@ cudaError_t launch_spread_op(const GridParams &g, int fp_bytes, const double *R,
     if (e != cudaSuccess || m.ns <= 0) return e;
     const unsigned *keys = m.keys[m.sorted];
     const int *perm = m.perm[m.sorted];
+    if (m.sp_ready) {
+        const unsigned nc_cells = (unsigned)((m.ns * (g.dim == 3 ? 27ll : 9ll) + 127) / 128);
+        if (fp_bytes == 4)
+            spread_op_static_kernel<float><<<nc_cells, 128, 0, s>>>(g, R, nc, m, (float *)out);
+        else
+            spread_op_static_kernel<double><<<nc_cells, 128, 0, s>>>(g, R, nc, m, (double *)out);
+        return cudaGetLastError();
+    }
     const int nb = 4 * 152;
     if (g.dim == 3) {
         if (fp_bytes == 4)

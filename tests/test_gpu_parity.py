@@ -723,3 +723,25 @@ def test_2d_fp32_single_rows_equal_the_march(nx, bc):
     assert a.time()[0] == b.time()[0]
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("nc", [1, 4, 6])
+@pytest.mark.parametrize("dim,n,fp", [(2, (41, 37), 4), (2, (41, 37), 8),
+                                      (3, (21, 19, 17), 4), (3, (21, 19, 17), 8)])
+def test_spread_through_the_stored_operator_equals_the_gather(dim, n, fp, nc):
+    """Spreading with static markers (their operator is stored) against the
+    same markers declared moving (gathered from the bins), several per cell:
+    sums of at most ~60 FP64 terms, one rounding to the grid's type."""
+    g = C.small_grid(dim, n, h=0.1, fp_bytes=fp)
+    rng = np.random.default_rng(11)
+    X = np.asarray(g.lo)[:dim] + 0.1 * np.asarray(n) * rng.uniform(0.3, 0.7, (150, dim))
+    X[:4] = X[0] + 0.03 * rng.uniform(-1.0, 1.0, (4, dim))
+    R = torch.from_numpy(rng.standard_normal((150, nc))).cuda()
+    out = []
+    for motion in (None, C.Motion(amp=0.01, freq=0.2, axis=0)):
+        grid = ibm.Grid(g, max_markers=150)
+        assert grid.set_markers(X, np.ones(150), motion=motion, dedup=False) == 150
+        out.append(grid.spread(R).double())
+        grid.close()
+    scale = float(out[1].abs().max())
+    assert float((out[0] - out[1]).abs().max()) <= (2.4e-7 if fp == 4 else 1e-13) * scale
