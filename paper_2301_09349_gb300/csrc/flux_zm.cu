@@ -4,8 +4,8 @@
 //
 // A CTA of 256 threads owns a 32 x 16 column of cells and walks up a chunk of
 // z-planes; each thread owns two neighbouring cells of one row, (2t, r) and
-// (2t+1, r).  Shared memory holds a ring of four primitive planes (z-1 ..
-// z+2) with a two-cell halo in x and y, so every cell is loaded from memory
+// (2t+1, r).  Shared memory holds a ring of five primitive planes (z-1 ..
+// z+3) with a two-cell halo in x and y, so every cell is loaded from memory
 // and converted to primitives once per chunk.  Per plane and thread:
 //   - the x-faces 2t-1/2 and 2t+1/2 of its row as one packed FP32x2 pair:
 //     the five cells 2t-2 .. 2t+2 give the three limited slopes of cells
@@ -15,25 +15,31 @@
 //     of plane z+1 and the z-face fluxes are carried in registers to the
 //     next plane, where they are the lower plane's;
 //   - warp 7 also evaluates the tile's upper x- and y-edge faces;
+//   - plane z+3 is converted into the ring slot of plane z-2;
 // one barrier, then each thread forms the flux divergence of its two cells
 // from its own faces (registers), the x-face of its right neighbour (a warp
-// shuffle), the y-faces of the row above (shared memory), and writes both
-// cells with 8-byte accesses; the next plane is converted into the ring and
-// a second barrier closes the plane.  Neighbouring cells sit in adjacent
+// shuffle), the y-faces of the row above (a shuffle within a warp's two rows,
+// shared memory between warps), and writes both cells with 8-byte accesses.
+// The five ring slots and two sets of exchanged faces make that barrier the
+// only one: what a thread ahead of the others overwrites was last read before
+// the barrier it has passed.  Neighbouring cells sit in adjacent
 // 32-bit words of the ring, so most stencil loads are 8-byte (two cells).
 // All constants are single precision: the kernel issues no FP64 work except
 // the per-CTA step-size maximum.
 //
-// Bound: instruction issue and latency (16 warps per SM at 56 % issue; the
-// plane barriers and fixed-latency waits are the rest).  Folding the halves
-// and 1/h out of the fluxes, one special-function operation for the sound
-// speed and one for Sutherland's law, plain reciprocals, and scalar arithmetic
-// where a one-cell shift breaks the register pairs took 777 -> 710 and 892 ->
-// 838 thread instructions per cell (192^3): 256^3 533 -> 487 us (stage 1) and
-// 616 -> 575 us (stage 2).  Measured and not kept: converting pairs of cells
-// (18 x 20 of them do not divide among 256 threads: 532 us), and per-pair
-// source tables with asynchronous copies in place of the mapped loads (510
-// and 679 us, stage 2 spilling).
+// Bound: instruction issue and latency (16 warps per SM at 61 % issue in stage
+// 1, 56 % in stage 2, 680 and 770 thread instructions per cell; fixed-latency
+// waits, the barrier and the FMA pipe's throttle are the rest).  What was
+// gained, both stages of 256^3 (192^3): 1151 us (561) at two barriers per plane; 1067 (511) with the halves and 1/h folded out of the
+// fluxes, one special-function operation for the sound speed and one for
+// Sutherland's law, plain reciprocals, and scalar arithmetic where a one-cell
+// shift breaks the register pairs; 1026 (462) with one barrier per plane,
+// ghosts found once per chunk and taken from the staged plane, and the rates
+// of stage 2 as pairs; 979 (443) with chunks of full waves, the columns at the
+// domain's edge first.  Measured and not kept: converting pairs of cells
+// (18 x 20 of them do not divide among 256 threads: 532 us for stage 1), and
+// per-pair source tables with asynchronous copies in place of the mapped loads
+// (510 and 679 us, stage 2 spilling).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <float.h>
@@ -52,15 +58,16 @@ constexpr int TX = 32, TY = 16, NTH = 256;               // tile cells; 16 threa
 constexpr int PX = TX + 4, PY = TY + 4, PP = PX * PY;    // plane with a 2-cell halo
 constexpr int NW = 6;                                     // rho, u, v, w, p, T
 constexpr int NC = 5;
-constexpr int RING = 4;
+constexpr int RING = 5;
 constexpr int SLOT = NW * PP;
 // TMA staging box of one plane: x from ox-4 (16-byte aligned) over 40 cells,
 // y from oy-2 over 20 rows, the five conserved components
 constexpr int SBX = TX + 8, SBY = TY + 4;
 constexpr int STAGE = NC * SBX * SBY;                     // floats
-constexpr int FYN = NC * (TY + 1) * TX;                   // y-face fluxes, row r = face r-1/2
+constexpr int FYR = TY / 2 + 1;                           // y-faces below the even rows and the edge
+constexpr int FYN = NC * FYR * TX;
 constexpr int FXE = NC * TY;                              // x-face fluxes of the upper x edge
-constexpr size_t SMEM_BASE = sizeof(float) * (size_t)(RING * SLOT + FYN + FXE);
+constexpr size_t SMEM_BASE = sizeof(float) * (size_t)(RING * SLOT + 2 * (FYN + FXE));
 constexpr size_t SMEM_TMA_OFF = (SMEM_BASE + 127) / 128 * 128;
 constexpr size_t SMEM = SMEM_TMA_OFF + sizeof(float) * STAGE + 16;   // + mbarrier
 constexpr long long TMA_WAIT_LIMIT = 1ll << 20;           // bounded mbarrier waits
@@ -68,23 +75,23 @@ static_assert(PX % 2 == 0 && PP % 2 == 0 && SLOT % 2 == 0, "8-byte ring loads ne
 
 using FC = FloatConsts;
 
-// step-size rate of one cell from its conserved state, single precision
-// throughout (same formula as the shared step_rate helper)
-__device__ __forceinline__ float rate_f(const FC &c, const float *u, bool &ok) {
-    const float rho = u[0], inv = __fdividef(1.0f, rho);
-    const float vx = u[1] * inv, vy = u[2] * inv, vz = u[3] * inv;
-    const float p = c.gm1 * (u[4] - 0.5f * rho * (vx * vx + vy * vy + vz * vz));
-    const float c2 = c.gamma * p * inv;
-    const float snd = c2 * rsqrtf(c2);
-    float mu = 0.0f;
-    if (c.viscous) {
-        const float Tt = p * inv * c.invR;
-        mu = __fdividef(c.mu_inf * Tt * (Tt * rsqrtf(Tt)) * c.onepS, Tt + c.S);
-    }
-    const float s = (fabsf(vx) + fabsf(vy) + fabsf(vz) + 3.0f * snd) * c.inv_h +
-                    6.0f * (c.kvisc * mu * inv) * c.inv_h * c.inv_h;
-    if (!(rho > 0.0f && p > 0.0f && s <= 3.0e38f)) ok = false;
-    return s;
+// step-size rates of two cells, or one, from their conserved states, single
+// precision throughout (step_rate's formula); p the pressure
+template <typename V>
+__device__ __forceinline__ V rate_of(const FC &c, const V (&u)[NC], V &p) {
+    const V inv = rcp2(u[0]);
+    const V vx = u[1] * inv, vy = u[2] * inv, vz = u[3] * inv;
+    const V rk = fma2(u[1], vx, fma2(u[2], vy, u[3] * vz));   // rho |u|^2
+    p = cmul(c.gm1, cfma(-0.5f, rk, u[4]));
+    const V T = p * inv, c2 = cmul(c.gamma, T), Tf = T + T;
+    const V y = cadd(c.s2, Tf);
+    const V m = cmul(c.km, Tf) * (Tf * rsqrt2(Tf * y * y));   // 2 mu / h
+    const V snd = c2 * rsqrt2(c2);
+    return cfma(c.inv_h, cfma(3.0f, snd, abs2(vx) + abs2(vy) + abs2(vz)),
+                cmul(3.0f * c.kvisc * c.inv_h, m) * inv);
+}
+__device__ __forceinline__ bool rate_ok(float rho, float p, float s) {
+    return rho > 0.0f && p > 0.0f && s <= 3.0e38f;
 }
 
 FC make_fc(const GridParams &g) { return float_consts(g); }
@@ -405,22 +412,81 @@ __device__ __forceinline__ void mapped_cell(const GridParams &g, const FC &c,
         if ((flip >> d) & 1) u[1 + d] = -u[1 + d];
 }
 
-// Convert the staged plane gz into one ring slot.  Cells outside the domain in
-// x or y (zero-filled by the copy) are taken through the boundary conditions.
+// The thread's cells of a plane (ring cells tid, tid + 256, tid + 512), their
+// source cells through the x and y boundary conditions, found once per chunk:
+// the tiles at the domain's edge, a third of 256^3 and most of 96^3, otherwise
+// map every ghost again in every plane, in all lanes of their warps.
+// off: in-plane index of the source; flags, four bits a cell: slip flips of u
+// and v, free stream.
+constexpr int NQ = (PP + NTH - 1) / NTH;
+constexpr unsigned SRC_FREE = 4, SRC_FAR = 8;
+constexpr int SRC_BITS = 14;
+struct Sources {
+    int off[NQ];
+    unsigned flags;
+};
+__device__ __forceinline__ Sources plane_sources(const GridParams &g, int ox, int oy) {
+    Sources s;
+    s.flags = 0u;
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
+        const int q = min((int)threadIdx.x + i * NTH, PP - 1);
+        int flip = 0, fs = 0;
+        const int sx = map_axis(ox + q % PX - 2, g.n[0], g.bc[0], g.bc[1], 0, flip, fs);
+        const int sy = map_axis(oy + q / PX - 2, g.n[1], g.bc[2], g.bc[3], 1, flip, fs);
+        s.off[i] = sx + g.n[0] * sy;
+        s.flags |= ((unsigned)flip | (fs ? SRC_FREE : 0u)) << (4 * i);
+    }
+    return s;
+}
+// the same for a staged plane, 14 bits a cell: stage index, with the flags
+// from bit 10; FAR: the source is not in the staging box (a periodic image)
+static_assert(SBX * SBY <= 1024 && NQ * SRC_BITS <= 64, "packed stage sources");
+__device__ __forceinline__ unsigned long long stage_sources(const GridParams &g, const Sources &p,
+                                                            int ox, int oy) {
+    unsigned long long st = 0;
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
+        const int x = p.off[i] % g.n[0] - (ox - 4), y = p.off[i] / g.n[0] - (oy - 2);
+        const bool in = x >= 0 && x < SBX && y >= 0 && y < SBY;
+        const unsigned f = ((p.flags >> (4 * i)) & 7u) | (in ? 0u : SRC_FAR);
+        st |= (unsigned long long)((in ? y * SBX + x : 0) | (int)(f << 10)) << (SRC_BITS * i);
+    }
+    return st;
+}
+
+__device__ __forceinline__ void apply_source(const FC &c, unsigned f, float (&u)[NC]) {
+    if (f & 1u) u[1] = -u[1];
+    if (f & 2u) u[2] = -u[2];
+    if (f & SRC_FREE) {
+        u[0] = 1.0f;
+        u[1] = 1.0f;
+        u[2] = 0.0f;
+        u[3] = 0.0f;
+        u[4] = c.E_inf;
+    }
+}
+
+// Convert the staged plane gz into one ring slot.  (One cell after the other:
+// three at once do not fit the registers.)
 __device__ __forceinline__ void convert_staged(const GridParams &g, const FC &c,
                                                const float *__restrict__ U,
                                                const float *__restrict__ st,
-                                               float *__restrict__ slot, int ox, int oy, int gz,
-                                               bool xy_interior, int *err) {
+                                               float *__restrict__ slot, unsigned long long src,
+                                               int ox, int oy, int gz, int *err) {
+#pragma unroll 1
     for (int q = threadIdx.x; q < PP; q += NTH) {
-        const int lx = q % PX, ly = q / PX;
-        const int gx = ox + lx - 2, gy = oy + ly - 2;
+        const unsigned e = (unsigned)src & ((1u << SRC_BITS) - 1u);
+        src >>= SRC_BITS;
+        const float *p = st + (e & 1023u);
         float u[NC];
-        if (xy_interior || (gx >= 0 && gx < g.n[0] && gy >= 0 && gy < g.n[1])) {
 #pragma unroll
-            for (int m = 0; m < NC; ++m) u[m] = st[(m * SBY + ly) * SBX + lx + 2];
-        } else {
-            mapped_cell(g, c, U, gx, gy, gz, u, err);
+        for (int m = 0; m < NC; ++m) u[m] = p[m * (SBX * SBY)];
+        if (e >> 10) {
+            if (e >> 10 & SRC_FAR)
+                mapped_cell(g, c, U, ox + q % PX - 2, oy + q / PX - 2, gz, u, err);
+            else
+                apply_source(c, e >> 10, u);
         }
         to_primitive(c, u, slot, q);
     }
@@ -430,24 +496,29 @@ __device__ __forceinline__ void convert_staged(const GridParams &g, const FC &c,
 // primitives into one ring slot.
 __device__ __forceinline__ void load_plane(const GridParams &g, const FC &c,
                                            const float *__restrict__ U, float *__restrict__ slot,
-                                           int ox, int oy, int gz, bool xy_interior, int *err) {
+                                           const Sources &s, int gz, int *err) {
     const long long N = g.N;
-    const bool fast = xy_interior && gz >= 0 && gz < g.n[2];
+    int flip = 0, fs = 0;
+    const int sz = map_axis(gz, g.n[2], g.bc[4], g.bc[5], 2, flip, fs);
+    const float *P = U + (long long)g.n[0] * g.n[1] * sz;
+    int o = s.off[0], o1 = s.off[1], o2 = s.off[2];
+    unsigned fl = s.flags;
+#pragma unroll 1
     for (int q = threadIdx.x; q < PP; q += NTH) {
-        const int lx = q % PX, ly = q / PX;
+        const bool okj = in_bounds((P - U) + o, N, err);
         float u[NC];
-        if (fast) {
-            const long long j =
-                (ox + lx - 2) + (long long)g.n[0] * ((oy + ly - 2) + (long long)g.n[1] * gz);
-            const bool okj = in_bounds(j, N, err);
 #pragma unroll
-            for (int m = 0; m < NC; ++m) u[m] = okj ? __ldg(U + m * N + j) : 0.0f;
-        } else {
-            mapped_cell(g, c, U, ox + lx - 2, oy + ly - 2, gz, u, err);
-        }
+        for (int m = 0; m < NC; ++m) u[m] = okj ? __ldg(P + m * N + o) : 0.0f;
+        if (flip) u[3] = -u[3];
+        const unsigned f = (fl & 7u) | (fs ? SRC_FREE : 0u);
+        if (f) apply_source(c, f, u);
         to_primitive(c, u, slot, q);
+        o = o1;
+        o1 = o2;
+        fl >>= 4;
     }
 }
+static_assert(NQ == 3, "load_plane's sources");
 
 __device__ __forceinline__ double warp_max_d(double v) {
 #pragma unroll
@@ -461,6 +532,31 @@ __device__ __forceinline__ double warp_max_d(double v) {
 #ifndef IBM_ZM_PREFETCH
 #define IBM_ZM_PREFETCH 1
 #endif
+
+// The chunk of this CTA (column x, y and z), CTAs taken in launch order: with
+// more than one wave of them the columns at the domain's edge come first,
+// since they take longer and what starts last should be short (256^3, both
+// stages: 992 -> 977 us, 192^3 450 -> 438; grids whose planes arrive by thread
+// loads lose more of their neighbours' cached lines than that: 837 -> 887 us
+// at 255 x 201 x 190).
+constexpr int ZM_SLOTS = 2 * 152;
+__device__ __forceinline__ int3 chunk_order() {
+    const int nbx = gridDim.x, nby = gridDim.y;
+    const int inner = max(nbx - 2, 0) * max(nby - 2, 0);
+    if (inner == 0 || nbx * nby * (int)gridDim.z <= ZM_SLOTS)
+        return make_int3(blockIdx.x, blockIdx.y, blockIdx.z);
+    const int edges = nbx * nby - inner;
+    const int L = blockIdx.x + nbx * (blockIdx.y + nby * blockIdx.z), first = edges * gridDim.z;
+    if (L >= first) {
+        const int e = (L - first) % inner;
+        return make_int3(1 + e % (nbx - 2), 1 + e / (nbx - 2), (L - first) / inner);
+    }
+    int e = L % edges;
+    if (e < nbx) return make_int3(e, 0, L / edges);
+    if (e < 2 * nbx) return make_int3(e - nbx, nby - 1, L / edges);
+    e -= 2 * nbx;
+    return make_int3(e & 1 ? nbx - 1 : 0, 1 + (e >> 1), L / edges);
+}
 
 // MODE 0: out = L(Uin).  MODE 1: out = U1 = Uin + dt L(Uin).
 // MODE 2: out = U* = Un/2 + (Uin + dt L(Uin))/2 with Uin = U1, plus the
@@ -477,18 +573,21 @@ zmarch_kernel(const __grid_constant__ CUtensorMap tmap, const GridParams g, cons
               const unsigned *__restrict__ band_bits, double dt_fixed) {
     extern __shared__ __align__(128) float smem_zm[];
     float *ring = smem_zm;
-    float *FY = ring + RING * SLOT;           // [NC][TY+1][TX]: y-faces, row r = face r-1/2
-    float *FXe = FY + FYN;                    // [NC][TY]: x-faces between cells 31 and 32
+    // exchanged faces, two sets (even and odd planes): y-faces below the even
+    // rows and above row 15 ([NC][FYR][TX]), x-faces between cells 31 and 32
+    // ([NC][TY])
+    float *FYs = ring + RING * SLOT;
     __shared__ double s_red[NTH / 32];
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int r = tid >> 4, t = tid & 15;     // row of the thread, its cells 2t and 2t+1
-    const int ox = blockIdx.x * TX, oy = blockIdx.y * TY;
-    const int z0 = blockIdx.z * zc, z1 = min(z0 + zc, g.n[2]);
+    const int3 blk = TMA ? chunk_order() : make_int3(blockIdx.x, blockIdx.y, blockIdx.z);
+    const int ox = blk.x * TX, oy = blk.y * TY;
+    const int z0 = blk.z * zc, z1 = min(z0 + zc, g.n[2]);
     const long long N = g.N;
     const float dt = MODE == 0 ? 0.0f : (float)(dt_fixed > 0.0 ? dt_fixed : *dt_ptr);
-    const bool xyint = ox >= 2 && oy >= 2 && ox + TX + 2 <= g.n[0] && oy + TY + 2 <= g.n[1];
-    auto slot_of = [](int z) { return ((z + RING) & (RING - 1)) * SLOT; };   // z >= -2
+    const Sources src = plane_sources(g, ox, oy);
+    const unsigned long long ssrc = TMA ? stage_sources(g, src, ox, oy) : 0ull;
     const int b = (2 * t + 2) + PX * (r + 2);   // ring index of cell (2t, r)
 
     float *stage = reinterpret_cast<float *>(reinterpret_cast<char *>(smem_zm) + SMEM_TMA_OFF);
@@ -519,22 +618,11 @@ zmarch_kernel(const __grid_constant__ CUtensorMap tmap, const GridParams g, cons
         }
         __syncthreads();
     }
-    // planes z0-2 .. z0+1 by threads; z0+2 comes from the copy just issued
-    for (int zz = z0 - 2; zz <= z0 + 1; ++zz)
-        load_plane(g, c, Uin, ring + slot_of(zz), ox, oy, zz, xyint, err);
-    __syncthreads();
-
-    // carried from plane to plane: the halved limited z-slopes of the current
-    // plane and the z-face fluxes below it
-    float2 sig[NC], Fzl[NC];
-    {
-        float2 sgm[NC];
-        z_slopes(ring, slot_of(z0 - 2), slot_of(z0 - 1), slot_of(z0), b, sgm);
-        z_slopes(ring, slot_of(z0 - 1), slot_of(z0), slot_of(z0 + 1), b, sig);
-        z_pair(c, ring, slot_of(z0 - 1), slot_of(z0), b, sgm, sig, Fzl);
-    }
-    __syncthreads();   // plane z0-2's slot is about to take plane z0+2
-    // plane z0+2 (the ring needs planes z-1 .. z+2 at plane z)
+    // planes z0-2 .. z0+1 by threads; z0+2 comes from the copy just issued.
+    // Ring slots of planes z-2 (the next to be overwritten) .. z+2 at plane z:
+    int sm2 = 0, sm1 = SLOT, s0 = 2 * SLOT, s1 = 3 * SLOT, s2 = 4 * SLOT;
+    for (int i = 0; i < 4; ++i)
+        load_plane(g, c, Uin, ring + i * SLOT, src, z0 - 2 + i, err);
     {
         bool use_stage = TMA && z0 + 2 < nz;
         if (use_stage && !tma_wait(mbar, parity, err)) {
@@ -544,9 +632,9 @@ zmarch_kernel(const __grid_constant__ CUtensorMap tmap, const GridParams g, cons
         if (use_stage) {
             parity ^= 1u;
             if (tid == 0) outstanding = false;
-            convert_staged(g, c, Uin, stage, ring + slot_of(z0 + 2), ox, oy, z0 + 2, xyint, err);
+            convert_staged(g, c, Uin, stage, ring + s2, ssrc, ox, oy, z0 + 2, err);
         } else {
-            load_plane(g, c, Uin, ring + slot_of(z0 + 2), ox, oy, z0 + 2, xyint, err);
+            load_plane(g, c, Uin, ring + s2, src, z0 + 2, err);
         }
     }
     __syncthreads();
@@ -554,6 +642,17 @@ zmarch_kernel(const __grid_constant__ CUtensorMap tmap, const GridParams g, cons
         tma_issue(&tmap, st_addr, mbar, ox - 4, oy - 2, z0 + 3);
         outstanding = true;
     }
+
+    // carried from plane to plane: the halved limited z-slopes of the current
+    // plane and the z-face fluxes below it
+    float2 sig[NC], Fzl[NC];
+    {
+        float2 sgm[NC];
+        z_slopes(ring, sm2, sm1, s0, b, sgm);
+        z_slopes(ring, sm1, s0, s1, b, sig);
+        z_pair(c, ring, sm1, s0, b, sgm, sig, Fzl);
+    }
+    __syncthreads();   // plane z0-2's slot is about to take plane z0+3
 
     // the edge lanes of warp 7: 0-15 the y-faces above row 15 (columns 2l,
     // 2l+1), 16-23 the x-faces right of column 31 (rows q and q + 8)
@@ -580,8 +679,8 @@ zmarch_kernel(const __grid_constant__ CUtensorMap tmap, const GridParams g, cons
     float smaxf = 0.0f;
     bool ok = true;
     for (int z = z0; z < z1; ++z) {
-        const int sm1 = slot_of(z - 1), s0 = slot_of(z), s1 = slot_of(z + 1), s2 = slot_of(z + 2);
         const int up = s1 - s0, dn = sm1 - s0;
+        float *FY = FYs + (z & 1) * (FYN + FXE), *FXe = FY + FYN;
 #if IBM_ZM_PREFETCH
         // stage 2 reads U^n at its output cells, which nothing has touched:
         // start those lines toward L2 two planes ahead
@@ -592,25 +691,32 @@ zmarch_kernel(const __grid_constant__ CUtensorMap tmap, const GridParams g, cons
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(Un + m * N + jp));
         }
 #endif
-        // faces of plane z: x pair, y pair (stored for the row below), z pair
-        float2 Fx[NC], Fy[NC], Fzh[NC];
+        // faces of plane z: x pair, y pair (an even row's stored for the row
+        // below, which the warp below holds), z pair
+        float2 Fx[NC], Fy[NC], acc[NC];
         x_pair(c, ring + s0, b, up, dn, Fx);
         y_pair(c, ring + s0, b, up, dn, Fy);
+        if (!(r & 1)) {
 #pragma unroll
-        for (int m = 0; m < NC; ++m) st2(FY + (m * (TY + 1) + r) * TX + 2 * t, Fy[m]);
+            for (int m = 0; m < NC; ++m) st2(FY + (m * FYR + (r >> 1)) * TX + 2 * t, Fy[m]);
+        }
         {
-            float2 sgh[NC];
+            float2 sgh[NC], Fzh[NC];
             z_slopes(ring, s0, s1, s2, b, sgh);
             z_pair(c, ring, s0, s1, b, sig, sgh, Fzh);
 #pragma unroll
-            for (int m = 0; m < NC; ++m) sig[m] = sgh[m];
+            for (int m = 0; m < NC; ++m) {
+                sig[m] = sgh[m];
+                acc[m] = Fzl[m] - Fzh[m];
+                Fzl[m] = Fzh[m];
+            }
         }
         if (edge) {
             float2 Fe[NC];
             edge_pair(c, ring + s0, eA, eB, esn, est, enf, up, dn, Fe);
             if (lane < 16) {
 #pragma unroll
-                for (int m = 0; m < NC; ++m) st2(FY + (m * (TY + 1) + TY) * TX + 2 * lane, Fe[m]);
+                for (int m = 0; m < NC; ++m) st2(FY + (m * FYR + FYR - 1) * TX + 2 * lane, Fe[m]);
             } else {
                 const int q = lane - 16;
 #pragma unroll
@@ -620,31 +726,19 @@ zmarch_kernel(const __grid_constant__ CUtensorMap tmap, const GridParams g, cons
                 }
             }
         }
-        __syncthreads();
-
-        // flux divergence of the two cells
-        float2 acc[NC];
-#pragma unroll
-        for (int m = 0; m < NC; ++m) {
-            // x-face right of cell 2t+1: the neighbour's first face, or the edge
-            float fr = __shfl_down_sync(0xffffffffu, Fx[m].x, 1);
-            if (t == 15) fr = FXe[m * TY + r];
-            const float2 dx = make_float2(__fsub_rn(Fx[m].x, Fx[m].y), __fsub_rn(Fx[m].y, fr));
-            const float2 Fyu = ld2(FY + (m * (TY + 1) + r + 1) * TX + 2 * t);
-            acc[m] = cmul(m == NC - 1 ? c.qinv_h : c.hinv_h, (dx + (Fy[m] - Fyu)) + (Fzl[m] - Fzh[m]));
-            Fzl[m] = Fzh[m];
-        }
         // output operands of the two cells: U^n (stage 2) is issued now and
         // used after the next plane's conversion, so its latency overlaps it;
         // the input state at the cells is rebuilt from the ring at the output
         const long long j = gx + (long long)g.n[0] * (gy + (long long)g.n[1] * z);
         float2 o1[NC], o2[NC];
+        unsigned bits = 0u;   // the band word of the two cells (vec: one word holds both)
         if (MODE == 2 && vec && in_bounds(j + 1, N, err)) {
 #pragma unroll
             for (int m = 0; m < NC; ++m) o2[m] = ld2(Un + m * N + j);
+            if (band_bits) bits = __ldg(band_bits + (j >> 5)) >> (j & 31);
         }
 
-        // plane z+3 into the slot of z-1 (read only before the barrier above)
+        // plane z+3 into the slot of z-2 (last read before the last barrier)
         if (z + 1 < z1) {
             bool use_stage = TMA && z + 3 < nz && !*tma_dead;
             if (use_stage && !tma_wait(mbar, parity, err)) {
@@ -654,10 +748,29 @@ zmarch_kernel(const __grid_constant__ CUtensorMap tmap, const GridParams g, cons
             if (use_stage) {
                 parity ^= 1u;
                 if (tid == 0) outstanding = false;
-                convert_staged(g, c, Uin, stage, ring + slot_of(z + 3), ox, oy, z + 3, xyint, err);
+                convert_staged(g, c, Uin, stage, ring + sm2, ssrc, ox, oy, z + 3, err);
             } else {
-                load_plane(g, c, Uin, ring + slot_of(z + 3), ox, oy, z + 3, xyint, err);
+                load_plane(g, c, Uin, ring + sm2, TMA ? plane_sources(g, ox, oy) : src, z + 3, err);
             }
+        }
+        __syncthreads();
+        if (TMA && tid == 0 && !*tma_dead && z + 2 < z1 && z + 4 < nz) {
+            tma_issue(&tmap, st_addr, mbar, ox - 4, oy - 2, z + 4);
+            outstanding = true;
+        }
+
+        // flux divergence of the two cells
+#pragma unroll
+        for (int m = 0; m < NC; ++m) {
+            // x-face right of cell 2t+1: the neighbour's first face, or the edge
+            float fr = __shfl_down_sync(0xffffffffu, Fx[m].x, 1);
+            if (t == 15) fr = FXe[m * TY + r];
+            const float2 dx = make_float2(__fsub_rn(Fx[m].x, Fx[m].y), __fsub_rn(Fx[m].y, fr));
+            // y-face above: the warp's other row holds it, or the next warp
+            float2 Fyu = make_float2(__shfl_down_sync(0xffffffffu, Fy[m].x, 16),
+                                     __shfl_down_sync(0xffffffffu, Fy[m].y, 16));
+            if (r & 1) Fyu = ld2(FY + (m * FYR + (r >> 1) + 1) * TX + 2 * t);
+            acc[m] = cmul(m == NC - 1 ? c.qinv_h : c.hinv_h, (dx + (Fy[m] - Fyu)) + acc[m]);
         }
 
         if (in0 && in_bounds(j + (vec ? 1 : 0), N, err)) {
@@ -685,17 +798,21 @@ zmarch_kernel(const __grid_constant__ CUtensorMap tmap, const GridParams g, cons
 #pragma unroll
                     for (int m = 0; m < NC; ++m) st2(out + m * N + j, cfma(dt, acc[m], o1[m]));
                 } else {
-                    float ua[NC], ub[NC];
+                    float2 us[NC], p;
 #pragma unroll
                     for (int m = 0; m < NC; ++m) {
-                        const float2 us =
-                            cfma(0.5f, o2[m], cmul(0.5f, cfma(dt, acc[m], o1[m])));
-                        st2(out + m * N + j, us);
-                        ua[m] = us.x;
-                        ub[m] = us.y;
+                        us[m] = cfma(0.5f, o2[m], cmul(0.5f, cfma(dt, acc[m], o1[m])));
+                        st2(out + m * N + j, us[m]);
                     }
-                    if (!band_bit(band_bits, j)) smaxf = fmaxf(smaxf, rate_f(c, ua, ok));
-                    if (!band_bit(band_bits, j + 1)) smaxf = fmaxf(smaxf, rate_f(c, ub, ok));
+                    const float2 sr = rate_of(c, us, p);
+                    if (!(bits & 1u)) {
+                        smaxf = fmaxf(smaxf, sr.x);
+                        ok = ok && rate_ok(us[0].x, p.x, sr.x);
+                    }
+                    if (!(bits & 2u)) {
+                        smaxf = fmaxf(smaxf, sr.y);
+                        ok = ok && rate_ok(us[0].y, p.y, sr.y);
+                    }
                 }
             } else {
 #pragma unroll
@@ -717,16 +834,23 @@ zmarch_kernel(const __grid_constant__ CUtensorMap tmap, const GridParams g, cons
                             out[m * N + jk] = us[m];
                         }
                     }
-                    if (MODE == 2 && !band_bit(band_bits, jk)) smaxf = fmaxf(smaxf, rate_f(c, us, ok));
+                    if (MODE == 2 && !band_bit(band_bits, jk)) {
+                        F1 v[NC], p;
+#pragma unroll
+                        for (int m = 0; m < NC; ++m) v[m].x = us[m];
+                        const float sr = rate_of(c, v, p).x;
+                        smaxf = fmaxf(smaxf, sr);
+                        ok = ok && rate_ok(us[0], p.x, sr);
+                    }
                 }
             }
         }
-        __syncthreads();
-        if (TMA && tid == 0 && !*tma_dead && z + 2 < z1 && z + 4 < nz) {
-            tma_issue(&tmap, st_addr, mbar, ox - 4, oy - 2, z + 4);
-            outstanding = true;
-        }
-
+        const int sn = sm2;
+        sm2 = sm1;
+        sm1 = s0;
+        s0 = s1;
+        s1 = s2;
+        s2 = sn;
     }
 
     // thread 0 flips its parity only on copies it saw complete, so `parity`
@@ -750,21 +874,18 @@ zmarch_kernel(const __grid_constant__ CUtensorMap tmap, const GridParams g, cons
 
 }  // namespace
 
-// Planes per CTA.  A chunk of zc planes costs about zc + 2.5 plane times (its
-// four-plane prologue, the z-faces below it), and the grid runs in waves of
-// two CTAs per SM, so the chunk count k is the one with the least
-// waves(k) * (zc + 2.5); a grid of at most one CTA per SM runs each of them
-// in ~0.6 of the time.  At most ZM_CHUNK_MAX planes: the tiles at the domain's
-// edge take longer, and short chunks even that out (256^3, both stages: 19
-// planes 1062 us, 37 planes, three full waves, 1080).  The former rule halved
-// 19-plane chunks until there were three waves, which left four planes per
-// chunk below ~150^3 and doubled the work: 131 x 97 x 113 237 -> 202 us for
-// both stages, 96^3 118 -> 88, 48^3 (L alone) 26 -> 18, 128^3 (L alone) 101 ->
-// 82.
-constexpr int ZM_CHUNK_MAX = 24;
+// Planes per CTA.  A chunk of zc planes costs about zc + 1 plane times (its
+// prologue of five planes, whose loads overlap, and the z-faces below it), and
+// the grid runs in waves of two CTAs per SM, so the chunk count k is the one
+// with the least waves(k) * (zc + 1); a grid of at most one CTA per SM runs
+// each of them in ~0.7 of the time.  Both stages, with 2.5 and 0.6 in their
+// place, of which the prologue once took its share -> now: 48^3 32.5 -> 30.4,
+// 64^3 44.9 -> 39.1, 150 x 90 x 74 124.8 -> 96.8 us.  At most ZM_CHUNK_MAX
+// planes (24: 192^3 462, 256^3 1026 us; 48: 450, 992; 96: 448, 992).
+constexpr int ZM_CHUNK_MAX = 96;
 int zmarch_chunk(const GridParams &g) {
     const long long cols = (long long)((g.n[0] + TX - 1) / TX) * ((g.n[1] + TY - 1) / TY);
-    const long long slots = 2 * 152;
+    const long long slots = ZM_SLOTS;
     const int kmin = (g.n[2] + ZM_CHUNK_MAX - 1) / ZM_CHUNK_MAX;
     const long long most = std::max<long long>(kmin, 8 * slots / cols + 1);
     const int kmax = (int)std::min<long long>(most, g.n[2]);
@@ -773,7 +894,7 @@ int zmarch_chunk(const GridParams &g) {
     for (int k = kmin; k <= kmax; ++k) {
         const int zc = (g.n[2] + k - 1) / k;
         const long long ctas = cols * ((g.n[2] + zc - 1) / zc);
-        const double c = (double)((ctas + slots - 1) / slots) * (zc + 2.5) * (2 * ctas <= slots ? 0.6 : 1.0);
+        const double c = (double)((ctas + slots - 1) / slots) * (zc + 1.0) * (2 * ctas <= slots ? 0.7 : 1.0);
         if (c < cost) {
             cost = c;
             best = zc;

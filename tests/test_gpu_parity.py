@@ -745,3 +745,21 @@ def test_spread_through_the_stored_operator_equals_the_gather(dim, n, fp, nc):
         grid.close()
     scale = float(out[1].abs().max())
     assert float((out[0] - out[1]).abs().max()) <= (2.4e-7 if fp == 4 else 1e-13) * scale
+
+
+@pytest.mark.parametrize("bc", [MIXED_BC, (C.BC_PERIODIC,) * 6, (C.BC_SLIP,) * 6])
+@pytest.mark.parametrize("n", [(4, 4, 4), (36, 18, 5), (33, 17, 6), (68, 33, 70), (65, 48, 31),
+                               (128, 256, 97)])
+def test_3d_fp32_march_equals_the_tile_kernel(n, bc):
+    """L(U) of the 3D FP32 march (staged and thread-loaded planes, ghosts from
+    the staged plane or a periodic image, several waves of chunks) against the
+    FP64 tile kernel on the same FP32 values, with the tolerance of the 2D
+    march's test."""
+    g4 = C.small_grid(3, n, h=0.1, fp_bytes=4, bc=bc)
+    g8 = C.small_grid(3, n, h=0.1, fp_bytes=8, bc=bc)
+    U = torch.from_numpy(C.random_state(g4, 9).astype(np.float32)).cuda()
+    a, b = ibm.Grid(g4), ibm.Grid(g8)
+    L4, L8 = a.rhs(U).double(), b.rhs(U.double())
+    assert float((L4 - L8).norm() / L8.norm()) < 1e-4
+    a.close()
+    b.close()
