@@ -1474,7 +1474,7 @@ ibm_status ibm_backward(ibm_grid *g, double dJ_dCd, double dJ_dNu, double *dJ_dX
     double scale = 0.0;
     for (double v : le) scale = fmax(scale, fabs(v));
     if (scale > 0.0) {
-        ACU(launch_quadrature_solve(ns, g->qb, a.lamEps, a.z, 1e-12 * scale, g->cg_maxit, g->err_d, s),
+        ACU(launch_quadrature_solve(g->gp.dim, ns, g->qb, a.lamEps, a.z, 1e-12 * scale, g->cg_maxit, g->err_d, s),
             "adjoint quadrature solve");
         ACU(launch_eps_adjoint_x(g->gp, g->mb, a, g->n_sm, s), "weights adjoint");
     }

@@ -354,7 +354,7 @@ int quad_row_width(int dim);
 // have_weights: m.wphi already holds the current positions' support weights)
 cudaError_t launch_quadrature(const GridParams &g, const MarkerBuffers &m, const QuadBuffers &qb,
                               double tol, int maxit, int warm, cudaStream_t s, int have_weights = 0);
-cudaError_t launch_quadrature_solve(int ns, const QuadBuffers &qb, const double *rhs, double *x,
+cudaError_t launch_quadrature_solve(int dim, int ns, const QuadBuffers &qb, const double *rhs, double *x,
                                     double tol, int maxit, int *err, cudaStream_t s);
 
 }  // namespace ibmk

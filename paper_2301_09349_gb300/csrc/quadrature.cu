@@ -984,6 +984,7 @@ __device__ __forceinline__ bool small_cg(int ns, const QuadBuffers &q, int k, in
 // one CTA per launch: the register file is the CTA's alone, so the
 // registers a thread may take are bounded for one resident block (the
 // diagonal-block factor keeps a 32-float row per lane)
+template <bool CG>
 __global__ void __launch_bounds__(CHOL_T, 1)
 chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ rhs, double tol,
             int maxit, int warm, int *err) {
@@ -1010,16 +1011,24 @@ chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ r
     if (tid == 0) s_bad = 0;
     if (tid < 2 * SCG_W) s_part[tid] = 0.0f;
     // the rows' first CHOL_EC entries and their lengths, kept for the
-    // residuals; their FP32 values for the conjugate gradients in F's place
+    // residuals; without the conjugate gradients (whose FP32 values take F's
+    // place) the lower triangle of A~ too (the upper stays zero)
+    if (!CG) {
+        for (int i = tid; i < ns * ld; i += CHOL_T) F[i] = 0.0f;
+        __syncthreads();
+    }
     for (int k = tid; k < ns; k += CHOL_T) {
         const int c = q.cnt[k];
         ecnt[k] = c;
-        for (int i = 0; i < min(c, CHOL_EC); ++i) {
+        for (int i = 0; i < (CG ? min(c, CHOL_EC) : c); ++i) {
             int l = q.col[(long long)i * q.cap + k];
             double v = q.val[(long long)i * q.cap + k];
             if (!in_bounds(l, ns, err)) { l = k; v = 0.0; }
-            ec[(size_t)i * ns + k] = l;
-            ev[(size_t)i * ns + k] = v;
+            if (CG || i < CHOL_EC) {
+                ec[(size_t)i * ns + k] = l;
+                ev[(size_t)i * ns + k] = v;
+            }
+            if (!CG && l <= k && v != 0.0) F[(size_t)k * ld + l] = (float)v;
         }
         sx[k] = warm ? x[k] : 0.0;
     }
@@ -1067,7 +1076,7 @@ chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ r
     double rmax = 0.0, rprev = 0.0;
     int it = 0;
     bool done = false;   // the residual is at its floor
-    if (ns > SCG_MIN && !__syncthreads_or(tid < ns && ecnt[tid] > SCG_ROW)) {
+    if (CG && !__syncthreads_or(tid < ns && ecnt[tid] > SCG_ROW)) {
         // corrections by FP32 conjugate gradients first
         float rv[SCG_REG], inv = 0.0f;
         int rc[SCG_REG];
@@ -1109,22 +1118,24 @@ chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ r
         }
     }
     if (!done) {
-    // the dense factor: the lower triangle of A~ (the upper stays zero)
-    for (int i = tid; i < ns * ld; i += CHOL_T) F[i] = 0.0f;
-    __syncthreads();
-    for (int k = tid; k < ns; k += CHOL_T) {
-        const int c = ecnt[k], cc = min(c, CHOL_EC);
-        for (int i = 0; i < cc; ++i) {
-            const int l = ec[(size_t)i * ns + k];
-            if (l <= k) F[(size_t)k * ld + l] = (float)ev[(size_t)i * ns + k];
+    if (CG) {
+        // the dense factor: the lower triangle of A~ (the upper stays zero)
+        for (int i = tid; i < ns * ld; i += CHOL_T) F[i] = 0.0f;
+        __syncthreads();
+        for (int k = tid; k < ns; k += CHOL_T) {
+            const int c = ecnt[k], cc = min(c, CHOL_EC);
+            for (int i = 0; i < cc; ++i) {
+                const int l = ec[(size_t)i * ns + k];
+                if (l <= k) F[(size_t)k * ld + l] = (float)ev[(size_t)i * ns + k];
+            }
+            for (int i = CHOL_EC; i < c; ++i) {
+                const int l = q.col[(long long)i * q.cap + k];
+                if (in_bounds(l, ns, err) && l <= k)
+                    F[(size_t)k * ld + l] = (float)q.val[(long long)i * q.cap + k];
+            }
         }
-        for (int i = CHOL_EC; i < c; ++i) {
-            const int l = q.col[(long long)i * q.cap + k];
-            if (in_bounds(l, ns, err) && l <= k)
-                F[(size_t)k * ld + l] = (float)q.val[(long long)i * q.cap + k];
-        }
+        __syncthreads();
     }
-    __syncthreads();
     // blocked Cholesky over 32-column panels, then the diagonal blocks' inverses
     for (int c0 = 0; c0 < ns; c0 += CHOL_PB) {
         const int w = min(CHOL_PB, ns - c0);
@@ -1252,14 +1263,18 @@ int quad_row_width(int dim) { return dim == 3 ? 125 * 4 : 25 * 4; }
 // A~ x = rhs (rhs == nullptr: all ones), warm-started if asked.  One CTA up
 // to BCG_MAX markers, one cluster to CL_MAX (both sides of each line measured
 // at the kernels), the FP64 PCG above
-static cudaError_t launch_quadrature_solve_w(int ns, const QuadBuffers &qb, const double *rhs,
+static cudaError_t launch_quadrature_solve_w(int dim, int ns, const QuadBuffers &qb, const double *rhs,
                                             double *x, double tol, int maxit, int warm, int *err,
                                             cudaStream_t s) {
     if (ns <= 0) return cudaSuccess;
     if (ns <= CHOL_MAX) {
-        cudaError_t e = func_smem_attr((const void *)chol_kernel, chol_smem(CHOL_MAX));
+        // conjugate gradients are worth a try where rows may be short (curves
+        // in 2D) and there is more to factor than two panels; a try that is
+        // sure to fail costs 103 markers in 3D 78 -> 84 us
+        const auto kernel = dim == 2 && ns > SCG_MIN ? chol_kernel<true> : chol_kernel<false>;
+        cudaError_t e = func_smem_attr((const void *)kernel, chol_smem(CHOL_MAX));
         if (e != cudaSuccess) return e;
-        chol_kernel<<<1, CHOL_T, chol_smem(ns), s>>>(ns, qb, x, rhs, tol, maxit, warm, err);
+        kernel<<<1, CHOL_T, chol_smem(ns), s>>>(ns, qb, x, rhs, tol, maxit, warm, err);
     } else if (ns <= BCG_MAX) {
         return ns <= 512 ? launch_block_cg<512>(ns, qb, x, rhs, tol, maxit, warm, err, s)
                          : launch_block_cg<1024>(ns, qb, x, rhs, tol, maxit, warm, err, s);
@@ -1287,14 +1302,14 @@ cudaError_t launch_quadrature(const GridParams &g, const MarkerBuffers &m, const
     if (e != cudaSuccess) return e;
     QuadBuffers q = qb;
     q.order = perm;   // the solvers may take the rows in bin order
-    return launch_quadrature_solve_w(m.ns, q, nullptr, m.eps, tol, maxit, warm, m.err, s);
+    return launch_quadrature_solve_w(g.dim, m.ns, q, nullptr, m.eps, tol, maxit, warm, m.err, s);
 }
 
 // A~ x = rhs with the matrix assembled by the last launch_quadrature (the
 // adjoint of the weights); x starts from zero.
-cudaError_t launch_quadrature_solve(int ns, const QuadBuffers &qb, const double *rhs, double *x,
+cudaError_t launch_quadrature_solve(int dim, int ns, const QuadBuffers &qb, const double *rhs, double *x,
                                     double tol, int maxit, int *err, cudaStream_t s) {
-    return launch_quadrature_solve_w(ns, qb, rhs, x, tol, maxit, 0, err, s);
+    return launch_quadrature_solve_w(dim, ns, qb, rhs, x, tol, maxit, 0, err, s);
 }
 
 }  // namespace ibmk
