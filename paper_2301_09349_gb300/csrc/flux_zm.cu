@@ -27,8 +27,8 @@
 // All constants are single precision: the kernel issues no FP64 work except
 // the per-CTA step-size maximum.
 //
-// Bound: instruction issue and latency (16 warps per SM at 61 % issue in stage
-// 1, 56 % in stage 2, 680 and 770 thread instructions per cell; fixed-latency
+// Bound: instruction issue and latency (16 warps per SM at 62 % issue in stage
+// 1, 57 % in stage 2, 636 and 729 thread instructions per cell; fixed-latency
 // waits, the barrier and the FMA pipe's throttle are the rest).  What was
 // gained, both stages of 256^3 (192^3): 1151 us (561) at two barriers per plane; 1067 (511) with the halves and 1/h folded out of the
 // fluxes, one special-function operation for the sound speed and one for
