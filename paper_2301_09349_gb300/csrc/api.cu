@@ -435,9 +435,8 @@ ibm_status ibm_set_state(ibm_grid *g, const void *U) {
     if (!U) return fail(g, IBM_ERR_ARG, "null state pointer");
     CU(cudaMemcpyAsync(g->U[g->cur], U, state_bytes(g->desc), cudaMemcpyDeviceToDevice, g->stream),
        "set_state copy");
-    CU(launch_dt_init(g->gp, g->desc.fp_bytes, g->U[g->cur], g->fb, g->stream), "initial dt");
-    CU(cudaMemsetAsync(g->mb.t, 0, sizeof(double), g->stream), "reset time");
-    CU(cudaMemsetAsync(g->mb.steps, 0, sizeof(long long), g->stream), "reset steps");
+    CU(launch_dt_init(g->gp, g->desc.fp_bytes, g->U[g->cur], g->fb, g->stream, g->mb.t, g->mb.steps),
+       "initial dt, time and steps");
     g->has_state = true;
     g->rec_steps = 0;
     return IBM_OK;
@@ -449,9 +448,8 @@ ibm_status ibm_set_state_host(ibm_grid *g, const void *U_host) {
     CU(cudaMemcpyAsync(g->U[g->cur], U_host, state_bytes(g->desc), cudaMemcpyHostToDevice,
                        g->stream),
        "set_state_host copy");
-    CU(launch_dt_init(g->gp, g->desc.fp_bytes, g->U[g->cur], g->fb, g->stream), "initial dt");
-    CU(cudaMemsetAsync(g->mb.t, 0, sizeof(double), g->stream), "reset time");
-    CU(cudaMemsetAsync(g->mb.steps, 0, sizeof(long long), g->stream), "reset steps");
+    CU(launch_dt_init(g->gp, g->desc.fp_bytes, g->U[g->cur], g->fb, g->stream, g->mb.t, g->mb.steps),
+       "initial dt, time and steps");
     g->has_state = true;
     g->rec_steps = 0;
     return IBM_OK;

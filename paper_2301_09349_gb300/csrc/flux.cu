@@ -233,12 +233,6 @@ __device__ __forceinline__ void direction_pass(const GridParams &g, const double
     // above, and its faces only after its own)
 }
 
-__device__ __forceinline__ double warp_max(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-
 // One tile of one stage.  MODE 0: out = L(Uin).  MODE 1: out = U1 = Uin +
 // dt L(Uin).  MODE 2: out = U* = Un/2 + (Uin + dt L(Uin))/2 with Uin = U1,
 // and the maximum of s_j(U*) over the tile's cells outside the band is
@@ -427,32 +421,44 @@ batch_stage_kernel(const BatchCase *__restrict__ cases, const int2 *__restrict__
 
 // *dt = cfl / max_j s_j(U) over every cell: per-CTA maxima, then the last
 // CTA to finish reduces them.
+// First step size of a new state, and its time and step count (where given).
+// Bound by memory on large grids; maxima stay in the grid's type and double
+// maxima are integer work: a conversion and an FP64 maximum per cell kept the
+// FP64 pipe busy for most of 103 us at 256^3 (now 56, 50 for its
+// bytes; 1024 x 512 17.0 -> 10.8).
 template <int DIM, typename T>
 __global__ void __launch_bounds__(NT)
 dt_init_kernel(const GridParams g, const T *__restrict__ U, double *__restrict__ blockmax,
                unsigned *__restrict__ counter, double *__restrict__ dt, int *__restrict__ err,
-               int cells) {
+               int cells, double *__restrict__ t, long long *__restrict__ steps) {
     constexpr int NC = DIM + 2;
     __shared__ double s_red[NT / 32];
     __shared__ int s_last;
     const long long N = g.N;
     const long long j0 = (long long)blockIdx.x * cells;
     const long long j1 = j0 + cells < N ? j0 + cells : N;
-    double smax = 0.0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    T smax = T(0);
     bool ok = true;
-    for (long long j = j0 + threadIdx.x; j < j1; j += NT) {
-        T u[NC];
+    constexpr int B = sizeof(T) == 4 ? 4 : 1;   // cells whose loads are issued together
+    for (long long jb = j0 + threadIdx.x; jb < j1; jb += B * NT) {
+        T u[B][NC];
 #pragma unroll
-        for (int c = 0; c < NC; ++c) u[c] = U[c * N + j];
-        smax = fmax(smax, (double)step_rate<DIM, T>(g, u, ok));
+        for (int i = 0; i < B; ++i)
+#pragma unroll
+            for (int c = 0; c < NC; ++c) u[i][c] = jb + i * NT < j1 ? U[c * N + jb + i * NT] : T(0);
+#pragma unroll
+        for (int i = 0; i < B; ++i)
+            if (jb + i * NT < j1) smax = fmax(smax, step_rate<DIM, T>(g, u[i], ok));
     }
-    smax = warp_max(smax);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) smax = fmax(smax, __shfl_xor_sync(0xffffffffu, smax, o));
     const int bad = __syncthreads_or(!ok);
-    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = smax;
+    if (lane == 0) s_red[warp] = (double)smax;
     __syncthreads();
     if (threadIdx.x == 0) {
         double m = s_red[0];
-        for (int w = 1; w < NT / 32; ++w) m = fmax(m, s_red[w]);
+        for (int w = 1; w < NT / 32; ++w) m = dmax_nonneg(m, s_red[w]);
         blockmax[blockIdx.x] = m;
         if (bad) record_error(err, ERR_NONFINITE);
         __threadfence();
@@ -462,17 +468,22 @@ dt_init_kernel(const GridParams g, const T *__restrict__ U, double *__restrict__
     if (!s_last) return;
     __threadfence();
     double m = 0.0;
-    for (unsigned b = threadIdx.x; b < gridDim.x; b += NT) m = fmax(m, __ldcg(blockmax + b));
-    m = warp_max(m);
-    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = m;
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += NT) m = dmax_nonneg(m, __ldcg(blockmax + b));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = dmax_nonneg(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (lane == 0) s_red[warp] = m;
     __syncthreads();
     if (threadIdx.x == 0) {
         double mm = s_red[0];
-        for (int w = 1; w < NT / 32; ++w) mm = fmax(mm, s_red[w]);
+        for (int w = 1; w < NT / 32; ++w) mm = dmax_nonneg(mm, s_red[w]);
         const bool good = mm > 0.0 && mm <= DBL_MAX && !(__ldcg(err) & ERR_NONFINITE);
         if (!good) record_error(err, ERR_NONFINITE);
         *dt = good ? g.cfl / mm : 0.0;
         *counter = 0u;
+        if (t) {
+            *t = 0.0;
+            *steps = 0;
+        }
     }
 }
 
@@ -597,18 +608,20 @@ cudaError_t launch_rhs(const GridParams &g, int fp_bytes, const void *U, void *L
     return dispatch<0>(g, fp_bytes, U, U, L, fb, 0.0, s);
 }
 
-cudaError_t launch_dt_init(const GridParams &g, int fp_bytes, const void *U,
-                           const FluidBuffers &fb, cudaStream_t s) {
-    const unsigned nb = (unsigned)dt_init_blocks(g);
-    const int c = dt_cells_per_cta(g.N);
-    if (g.dim == 3) {
-        if (fp_bytes == 4) dt_init_kernel<3, float><<<nb, NT, 0, s>>>(g, (const float *)U, fb.blockmax, fb.counter, fb.dt, fb.err, c);
-        else dt_init_kernel<3, double><<<nb, NT, 0, s>>>(g, (const double *)U, fb.blockmax, fb.counter, fb.dt, fb.err, c);
-    } else {
-        if (fp_bytes == 4) dt_init_kernel<2, float><<<nb, NT, 0, s>>>(g, (const float *)U, fb.blockmax, fb.counter, fb.dt, fb.err, c);
-        else dt_init_kernel<2, double><<<nb, NT, 0, s>>>(g, (const double *)U, fb.blockmax, fb.counter, fb.dt, fb.err, c);
-    }
+template <int DIM, typename T>
+static cudaError_t dt_init_t(const GridParams &g, const void *U, const FluidBuffers &fb, double *t,
+                             long long *steps, cudaStream_t s) {
+    dt_init_kernel<DIM, T><<<(unsigned)dt_init_blocks(g), NT, 0, s>>>(
+        g, (const T *)U, fb.blockmax, fb.counter, fb.dt, fb.err, dt_cells_per_cta(g.N), t, steps);
     return cudaGetLastError();
+}
+cudaError_t launch_dt_init(const GridParams &g, int fp_bytes, const void *U,
+                           const FluidBuffers &fb, cudaStream_t s, double *t, long long *steps) {
+    if (g.dim == 3)
+        return fp_bytes == 4 ? dt_init_t<3, float>(g, U, fb, t, steps, s)
+                             : dt_init_t<3, double>(g, U, fb, t, steps, s);
+    return fp_bytes == 4 ? dt_init_t<2, float>(g, U, fb, t, steps, s)
+                         : dt_init_t<2, double>(g, U, fb, t, steps, s);
 }
 
 }  // namespace ibmk

@@ -51,7 +51,8 @@ cudaError_t launch_stage2(const GridParams &g, int fp_bytes, const void *Un, con
 cudaError_t launch_rhs(const GridParams &g, int fp_bytes, const void *U, void *L,
                        const FluidBuffers &fb, cudaStream_t s);
 cudaError_t launch_dt_init(const GridParams &g, int fp_bytes, const void *U,
-                           const FluidBuffers &fb, cudaStream_t s);
+                           const FluidBuffers &fb, cudaStream_t s,
+                           double *t = nullptr, long long *steps = nullptr);
 // the z-marching form used for 3D FP32 grids (flux_zm.cu); mode 0/1/2 as above
 cudaError_t launch_zmarch(int mode, const GridParams &g, const void *Uin, const void *Un,
                           void *out, const FluidBuffers &fb, double dt_fixed, cudaStream_t s);
