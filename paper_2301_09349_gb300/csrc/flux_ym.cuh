@@ -661,7 +661,10 @@ batch_ymarch_kernel(const BatchCase *__restrict__ cases, const int2 *__restrict_
 // resident at once: a second wave of few warps takes as long as the first, and
 // a march takes ~1.4 us per row however few warps there are (one wave of 8 / 4 /
 // 2 / 1 rows of 219 x 103: 41 / 26 / 20 / 16.5 us a step).  Where single rows
-// of 28 columns are one wave, those (XXX us).  At most `most` rows.
+// of 28 columns are one wave, those: 11.6 us, and 13.1 / 14.7 us at 300 x 150 /
+// 350 x 200 against 18.1 and 19 by the march; the 16 x 16 tiles these forms
+// replace took 13.8, 15.9 and 16.1.  Larger: 467 x 428 23.2 (23.8 by tiles),
+// 640 x 480 25.0 (26.6).  At most 64 rows.
 struct YmPlan {
     int width, rows;
 };
