@@ -42,6 +42,7 @@ struct FloatConsts {
     // mu = (..) T^2 rsqrt(T (T + 2 S r)^2) of the two cells' summed T = p/rho,
     // and 2 c_p / (Pr r)
     float e1, h1, s2, km, kl;
+    float kr;              // 2 kvisc / h: the 2D step-size rate's viscous factor less 2 mu / h
 };
 
 // The same folded constants for the FP64 kernels: a division costs an FP64
@@ -99,6 +100,7 @@ inline FloatConsts float_consts(const GridParams &g) {
     c.s2 = (float)(2.0 * g.S * g.R);
     c.km = (float)(2.0 * g.mu_inf * (1.0 + g.S) * sqrt(8.0) / 4.0 / sqrt(g.R) * g.inv_h);
     c.kl = (float)(2.0 * g.cp / (g.Pr * g.R));
+    c.kr = 2.0f * c.kvisc * c.inv_h;
     return c;
 }
 

@@ -65,5 +65,32 @@ __device__ __forceinline__ F1 cfma(float c, F1 a, F1 b) { return {__fmaf_rn(c, a
 __device__ __forceinline__ F1 fabs_fma(F1 a, F1 b, F1 u) { return {__fmaf_rn(a.x, b.x, fabsf(u.x))}; }
 __device__ __forceinline__ F1 vlh2(F1 a, F1 b) { return {vlh1(a.x, b.x)}; }
 
+// Step-size rates of two cells, or one, of a 2D FP32 grid from their conserved
+// states: s = sum_d (|u_d| + c)/h + 4 nu / h^2; p the pressure.  The one formula
+// of the march, the first step size and the forced cells: every operation is an
+// explicit rounding, so all of them give a state the same step size, bit for
+// bit (a run continued from its own state repeats the uninterrupted one).
+struct RateK {
+    float gamma, gm1, s2, km, kr, ih;   // FloatConsts, ih = 1/h
+};
+__device__ __forceinline__ RateK rate_k(const FloatConsts &c) {
+    return RateK{c.gamma, c.gm1, c.s2, c.km, c.kr, c.inv_h};
+}
+template <typename V>
+__device__ __forceinline__ V rate_2d(const RateK &k, const V (&u)[4], V &p) {
+    const V inv = rcp2(u[0]);
+    const V vx = u[1] * inv, vy = u[2] * inv;
+    const V rk = fma2(u[1], vx, u[2] * vy);   // rho |u|^2
+    p = cmul(k.gm1, cfma(-0.5f, rk, u[3]));
+    const V T = p * inv, c2 = cmul(k.gamma, T), Tf = T + T;
+    const V y = cadd(k.s2, Tf);
+    const V m = cmul(k.km, Tf) * (Tf * rsqrt2(Tf * y * y));   // 2 mu / h
+    const V snd = c2 * rsqrt2(c2);
+    return cfma(k.ih, cfma(2.0f, snd, abs2(vx) + abs2(vy)), cmul(k.kr, m) * inv);
+}
+__device__ __forceinline__ bool rate_ok(float rho, float p, float s) {
+    return rho > 0.0f && p > 0.0f && s <= 3.0e38f;
+}
+
 }  // namespace
 }  // namespace ibmk

@@ -64,7 +64,7 @@ struct YK {
     float km;              // 2 mu / h less T^2 rsqrt(T (T + 2 S r)^2), T the two cells' sum
     float kl;              // 2 c_p / (Pr r)
     float ih2, ih4;        // 1/(2h), 1/(4h)
-    float ih, kr;          // 1/h, 2 max(4/3, gamma/Pr) / h, for the step-size rate
+    float ih, kr;          // 1/h and FloatConsts::kr, for the step-size rate
     bool viscous;
 };
 
@@ -89,9 +89,13 @@ __device__ __forceinline__ YK make_yk(const GridParams &g) {
     k.ih2 = 0.5f * c.inv_h;
     k.ih4 = c.qinv_h;
     k.ih = c.inv_h;
-    k.kr = 2.0f * c.kvisc * c.inv_h;
+    k.kr = c.kr;
     k.viscous = c.viscous != 0;
     return k;
+}
+
+__device__ __forceinline__ RateK rate_k(const YK &k) {
+    return RateK{k.gamma, k.gm1, k.s2, k.km, k.kr, k.ih};
 }
 
 // primitives (rho, u, v, p) and p / rho of one row
@@ -226,24 +230,6 @@ __device__ __forceinline__ void to_primitive(const YK &c, const V (&u)[NC], RowT
     r.T = r.w[3] * inv;
 }
 
-// step-size rates of two cells, or one, from their conserved states:
-// s = sum_d (|u_d| + c)/h + 4 nu / h^2 (step_rate's formula with this unit's
-// constants); p the pressure.  A cell is valid if rate_ok.
-template <typename V>
-__device__ __forceinline__ V rate_of(const YK &k, const V (&u)[NC], V &p) {
-    RowT<V> r;
-    to_primitive(k, u, r);
-    const V c2 = cmul(k.gamma, r.T), Tf = r.T + r.T;
-    const V y = cadd(k.s2, Tf);
-    const V m = cmul(k.km, Tf) * (Tf * rsqrt2(Tf * y * y));   // 2 mu / h
-    const V snd = c2 * rsqrt2(c2);
-    p = r.w[3];
-    return cfma(k.ih, cfma(2.0f, snd, abs2(r.w[1]) + abs2(r.w[2])), cmul(k.kr, m) * rcp2(u[0]));
-}
-__device__ __forceinline__ bool rate_ok(float rho, float p, float s) {
-    return rho > 0.0f && p > 0.0f && s <= 3.0e38f;
-}
-
 // x-neighbours of the lane's pair: column 2t - 1 (lane below) and 2t + 2
 struct Side {
     float l, r;
@@ -348,7 +334,7 @@ __device__ __forceinline__ void row_out(const YK &k, bool paired, bool in1, long
     }
     if (MODE == 2) {
         float2 p;
-        const float2 sr = rate_of(k, r, p);
+        const float2 sr = rate_2d(rate_k(k), r, p);
         if (!band_bit(band_bits, j)) {
             smax = fmaxf(smax, sr.x);
             ok = ok && rate_ok(r[0].x, p.x, sr.x);
@@ -562,7 +548,7 @@ __device__ __forceinline__ void one_row(const YK &k, int x, int y, const float *
     }
     if (MODE == 2 && !band_bit(band_bits, j)) {
         F1 p;
-        const F1 sr = rate_of(k, r, p);
+        const F1 sr = rate_2d(rate_k(k), r, p);
         smax = fmaxf(smax, sr.x);
         ok = ok && rate_ok(r[0].x, p.x, sr.x);
     }

@@ -90,9 +90,6 @@ __device__ __forceinline__ V rate_of(const FC &c, const V (&u)[NC], V &p) {
     return cfma(c.inv_h, cfma(3.0f, snd, abs2(vx) + abs2(vy) + abs2(vz)),
                 cmul(3.0f * c.kvisc * c.inv_h, m) * inv);
 }
-__device__ __forceinline__ bool rate_ok(float rho, float p, float s) {
-    return rho > 0.0f && p > 0.0f && s <= 3.0e38f;
-}
 
 FC make_fc(const GridParams &g) { return float_consts(g); }
 

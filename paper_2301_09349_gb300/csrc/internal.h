@@ -7,6 +7,7 @@
 
 #include "../../include/ibm.h"
 #include "common.cuh"
+#include "flux_pair.cuh"
 
 namespace ibmk {
 
@@ -68,7 +69,7 @@ size_t ymarch_blocks(const GridParams &g);
 template <int DIM, typename T>
 __device__ __forceinline__ T step_rate(const GridParams &g, const T *u, bool &ok);
 
-// FP32 grids: single precision throughout, from the host-rounded constants.
+// 3D FP32 grids: single precision throughout, from the host-rounded constants.
 template <int DIM>
 __device__ __forceinline__ float step_rate_f(const GridParams &g, const float *u, bool &ok) {
     const FloatConsts &c = g.f;
@@ -135,7 +136,11 @@ __device__ __forceinline__ double step_rate<2, double>(const GridParams &g, cons
 }
 template <>
 __device__ __forceinline__ float step_rate<2, float>(const GridParams &g, const float *u, bool &ok) {
-    return step_rate_f<2>(g, u, ok);
+    const F1 v[4] = {{u[0]}, {u[1]}, {u[2]}, {u[3]}};
+    F1 p;
+    const float s = rate_2d(rate_k(g.f), v, p).x;
+    if (!rate_ok(u[0], p.x, s)) ok = false;
+    return s;
 }
 
 __device__ __forceinline__ bool band_bit(const unsigned *bits, long long j) {

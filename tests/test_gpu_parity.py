@@ -763,3 +763,26 @@ def test_3d_fp32_march_equals_the_tile_kernel(n, bc):
     assert float((L4 - L8).norm() / L8.norm()) < 1e-4
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("markers", [0, 40])
+@pytest.mark.parametrize("n,fp", [((128, 64), 4), ((219, 103), 4), ((601, 400), 4), ((128, 64), 8)])
+def test_2d_run_continued_from_its_state_keeps_its_step_size(n, fp, markers):
+    """The step size a run takes next, formed by the fluid stage and (in the
+    forced cells) by the spreading kernel, and the one that set_state forms
+    from the same state: the same bits."""
+    g = C.small_grid(2, n, h=0.1, fp_bytes=fp)
+    grid = ibm.Grid(g, max_markers=max(markers, 1))
+    if markers:
+        X = C.circle_markers(markers)
+        assert grid.set_markers(X, np.full(markers, 1.3)) > 0
+    for seed in range(6):
+        grid.set_state(cast(C.random_state(g, seed=seed, amp=0.05), g))
+        grid.step(3)
+        U = grid.get_state()
+        grid.step(1)
+        dt = grid.time()[0]
+        grid.set_state(U)
+        grid.step(1)
+        assert grid.time()[0] == dt
+    grid.close()
