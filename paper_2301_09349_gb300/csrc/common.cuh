@@ -43,6 +43,7 @@ struct FloatConsts {
     // and 2 c_p / (Pr r)
     float e1, h1, s2, km, kl;
     float kr;              // 2 kvisc / h: the 2D step-size rate's viscous factor less 2 mu / h
+    float p2;              // 2 p_inf, which the 2D march takes off its y-fluxes of normal momentum
 };
 
 // The same folded constants for the FP64 kernels: a division costs an FP64
@@ -101,6 +102,7 @@ inline FloatConsts float_consts(const GridParams &g) {
     c.km = (float)(2.0 * g.mu_inf * (1.0 + g.S) * sqrt(8.0) / 4.0 / sqrt(g.R) * g.inv_h);
     c.kl = (float)(2.0 * g.cp / (g.Pr * g.R));
     c.kr = 2.0f * c.kvisc * c.inv_h;
+    c.p2 = (float)(2.0 * g.p_inf);
     return c;
 }
 
