@@ -142,9 +142,13 @@ ibm_status ibm_set_wall_temperature(ibm_grid *g, const double *Tw);
 
 /* Stopping rule of the quadrature solve A~ eps~ = 1 (Sec. 2.2): the
  * solver of more than 160 markers stops when
- * max_k |1 - (A~ eps~)_k| <= tol, after at most maxit iterations
- * (IBM_ERR_NOCONV otherwise); up to 160 markers the solution is refined
- * to its rounding floor and the same bound checked.  Defaults 1e-12 and 4000.
+ * max_k |1 - (A~ eps~)_k| <= tol, after at most maxit iterations of the
+ * conjugate gradients in FP64 (IBM_ERR_NOCONV otherwise).  Up to 16384 markers
+ * corrections in FP32 come first, in at most maxit iterations too and a few
+ * hundred a correction; where they do not get there, the FP64 iterations start
+ * from the call's own first guess with all of maxit.  Up to 160 markers the
+ * solution is refined to its rounding floor and the same bound checked.
+ * Defaults 1e-12 and 4000.
  * Takes effect from the next ibm_set_markers (and every step of a moving
  * body).  Errors: IBM_ERR_ARG (tol outside (0, 1) or maxit < 1). */
 ibm_status ibm_set_quadrature(ibm_grid *g, double tol, int maxit);

@@ -284,6 +284,51 @@ __device__ __forceinline__ float cg_stop(float ru, float inner, int ns, double t
     return fmaxf(ru * inner * inner, (float)ns * t * t);
 }
 
+// When FP32 corrections give up.  A first pass takes 17 to 72 iterations with one
+// marker per cell (200 to 16000 markers), 90 to 600 with 1.4 markers per cell;
+// the next one 1.1 to 4 times as many, on a residual that the first has left
+// where A~ is weakest.  A nearly singular A~ (two markers 0.01 to 0.9 cells apart
+// in one cell, condition 1e8 and more) shows itself there: eight iterations
+// beyond the first pass's its r.u has grown by 200 and more, where it is below
+// 0.05 of its start in the others (one that went on took up to 1000 iterations,
+// all of them lost).  Besides, a first pass of more iterations than unknowns and
+// a later one of over four times the first are ended, and a pass that does not
+// contract the residual by four is the last.  A whole set_markers, before these
+// limits -> now, and by the FP64 solver alone: 5000 markers, two of them 0.1
+// cells apart, 7.5 -> 2.8 ms (2.9), 700 0.97 -> 0.77 (0.69), 300 markers on 150
+// cells 14.4 -> 4.2 (3.9).
+//
+// The FP64 solver then starts where the call started (from zero if its guess is
+// no better): what FP32 got wrong lies along the near-null vectors, where it
+// costs the FP64 solver more than the corrections save (200 markers, two of them
+// 0.9 cells apart: 108 iterations from zero, no convergence from the corrected
+// values).  After two contracting passes A~ is well conditioned, and it goes on
+// from the last good values.  maxit bounds the FP32 iterations, and those of the
+// FP64 solver, which then has all of maxit: FP32 passes take 1.1 to 9 times its
+// iterations, so that counting them as well would refuse what it solves within
+// maxit.
+struct CgPass {
+    int left, look;   // iterations left, and how many will be when r.u is looked at
+};
+__device__ __forceinline__ CgPass cg_pass(int outer, int first, int ns, int left) {
+    if (outer == 0) return CgPass{min(ns, left), 0};
+    const int last = min(4 * first + 32, left);
+    return CgPass{last, max(last - first - 8, 0)};
+}
+
+// The FP64 solver for what FP32 could not contract, from x: by the CTA's NTH
+// threads, or 256 of them up to 2048 markers (5 us an iteration at 200 markers, 7
+// with 512: its block sums and barriers).  A call, so that it takes no registers
+// from the corrections (inlined, 2 % of their time).
+template <int NTH>
+__device__ __noinline__ bool pcg_takes_over(int ns, const QuadBuffers &q, double *x,
+                                            const double *rhs, double tol, int maxit, double *s_red,
+                                            int *iters, double *resid, int *err) {
+    if (ns > 2048) return pcg_solve<NTH>(ns, q, x, rhs, tol, maxit, 1, s_red, iters, resid, err);
+    return pcg_solve<256>(ns, q, x, rhs, tol, maxit, 1, s_red, iters, resid, err);
+}
+__device__ __forceinline__ bool pcg_idle(int ns, int tid) { return ns <= 2048 && tid >= 256; }
+
 // BCG_MAX to CL_MAX markers: FP32 conjugate gradients inside FP64 iterative
 // refinement, on one thread-block cluster.
 //
@@ -358,6 +403,13 @@ cluster_cg_kernel(int ns, const ClusterShape sh, const QuadBuffers q, double *x,
     unsigned short *scol = reinterpret_cast<unsigned short *>(sval + CL_SM * NTH);
     __shared__ float s_warp[64];
     __shared__ double s_red[32];
+    // what a pass needs at its ends only, out of the registers: r.u at its
+    // start, max|r| before it, its iterations, those so far and of the first
+    __shared__ struct {
+        double rprev;
+        float ru0;
+        int last, it, first;
+    } s_pass;
     if (tid < 64) s_warp[tid] = 0.0f;
     // entry j of this thread: number sub + j LPR of its row
     const int cnt = own ? q.cnt[k] : 0;
@@ -389,8 +441,15 @@ cluster_cg_kernel(int ns, const ClusterShape sh, const QuadBuffers q, double *x,
         scol[(j - REG) * NTH + tid] = (unsigned short)l;
     }
     const float inv = own ? (float)(1.0 / q.diag[k]) : 0.0f;
-    double xk = own && warm ? x[k] : 0.0;
-    if (own && !warm && sub == 0) x[k] = 0.0;
+    // a row's first thread holds its value, in x; the first guess and the value
+    // at the start of a pass wait in the FP64 solver's workspace
+    const bool writes = own && sub == 0;
+    bool guess = warm != 0;
+    if (tid == 0) s_pass.it = s_pass.first = 0;
+    if (writes) {
+        if (!warm) x[k] = 0.0;
+        q.z[k] = x[k];
+    }
     __threadfence();
     cl.sync();
 
@@ -428,9 +487,8 @@ cluster_cg_kernel(int ns, const ClusterShape sh, const QuadBuffers q, double *x,
         cl.sync();
     };
 
-    int it = 0;
-    bool converged = false;
-    double rmax = 0.0, rprev = 0.0;
+    bool converged = false, over = false;   // over: the last pass was given up
+    double rmax = 0.0;
     for (int outer = 0;; ++outer) {
         // r = rhs - A~ x in FP64 from the ELL rows; x was written by its rows'
         // owners before the last cluster barrier
@@ -451,14 +509,24 @@ cluster_cg_kernel(int ns, const ClusterShape sh, const QuadBuffers q, double *x,
             rmax = dmax_nonneg(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
         if (rmax <= tol) { converged = true; break; }
         // no contraction, or a value FP32 cannot hold: the FP64 solver
-        if (!(rmax < 1e15) || rmax < 1e-15 || (outer > 0 && !(rmax < 0.25 * rprev)) ||
-            outer == CL_OUTER_MAX || it >= maxit)
+        if (outer == 0 && !(rmax < 1.0)) guess = false;   // worse than none
+        const bool failed = outer > 0 && (over || !(rmax < 0.25 * s_pass.rprev));
+        if (failed || !(rmax < 1e15) || rmax < 1e-15 || outer == CL_OUTER_MAX ||
+            s_pass.it >= maxit) {
+            if (writes && (s_pass.it >= maxit || outer - (failed ? 1 : 0) < 2)) x[k] = guess ? q.z[k] : 0.0;
+            else if (writes && failed) x[k] = q.r[k];
             break;
-        rprev = rmax;
+        }
+        if (writes) q.r[k] = x[k];
+        CgPass pass = cg_pass(outer, s_pass.first, ns, maxit - s_pass.it);
         // the correction d, from zero (a row's threads all hold its values)
         float r = (float)r64, u = r * inv, p = 0.0f, sv = 0.0f, d = 0.0f, gam = 1.0f, alpha = 1.0f,
               stop = 0.0f;
         send_u(u);
+        if (tid == 0) {   // (every thread is past the tests above)
+            s_pass.rprev = rmax;
+            s_pass.last = pass.left;
+        }
         for (bool first = true;; first = false) {
             float w = 0.0f;
             if (on) {
@@ -484,11 +552,19 @@ cluster_cg_kernel(int ns, const ClusterShape sh, const QuadBuffers q, double *x,
             }
             const float2 tot = reduce_all(sub == 0 ? r * u : 0.0f, sub == 0 ? w * u : 0.0f);
             const float g1 = tot.x, del = tot.y;
-            if (first) stop = cg_stop(g1, CL_INNER, ns, tol);
+            if (first) {
+                stop = cg_stop(g1, CL_INNER, ns, tol);
+                if (tid == 0) s_pass.ru0 = g1;
+            }
             if (g1 <= stop) break;
             const float beta = first ? 0.0f : __fdividef(g1, gam);
             const float den = first ? del : del - beta * __fdividef(g1, alpha);
-            if (!(den > 0.0f) || ++it >= maxit) break;   // (a NaN sum ends here too)
+            if (!(den > 0.0f) || pass.left == pass.look) {   // (a NaN sum ends here too)
+                over = pass.left == 0 || (pass.left == pass.look && g1 > s_pass.ru0);
+                if (over || !(den > 0.0f)) break;
+                pass.look = 0;
+            }
+            --pass.left;
             alpha = __fdividef(g1, den);
             gam = g1;
             p = u + beta * p;
@@ -498,19 +574,25 @@ cluster_cg_kernel(int ns, const ClusterShape sh, const QuadBuffers q, double *x,
             u = r * inv;
             send_u(u);
         }
+        if (tid == 0) {
+            s_pass.it += s_pass.last - pass.left;
+            if (outer == 0) s_pass.first = s_pass.it;
+        }
         // the next residual reads every CTA's rows
-        xk += (double)d;
-        if (own && sub == 0) x[k] = xk;
+        if (writes) x[k] += (double)d;
         __threadfence();
         cl.sync();
     }
+    __threadfence();
     cl.sync();   // no CTA leaves while another may still write to it
     if (rank != 0) return;
-    // x holds the refined values: kept if finite with a residual below 1
-    if (!converged)
-        converged = pcg_solve<NTH>(ns, q, x, rhs, tol, maxit, rmax < 1.0, s_red, &it, &rmax, err);
+    int n = 0;
+    if (!converged) {
+        if (pcg_idle(ns, tid)) return;
+        converged = pcg_takes_over<NTH>(ns, q, x, rhs, tol, maxit, s_red, &n, &rmax, err);
+    }
     if (tid == 0) {
-        *q.iters = it;
+        *q.iters = s_pass.it + n;
         *q.resid = rmax;
         if (!converged) record_error(err, ERR_NOCONV);
     }
@@ -581,11 +663,13 @@ block_cg_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict
     unsigned short *srow = scol + BCG_SM * NTH;                   // [NTH] row of a marker
     __shared__ float s_part[64];
     __shared__ double s_red[32];
+    __shared__ float s_ru0;   // r.u at the start of a pass
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool own = tid < ns, on = 32 * warp < ns;               // a row; a warp with rows
     const int k = own ? (q.order ? q.order[tid] : tid) : 0;
     const int cnt = own ? q.cnt[k] : 0;
     if (tid < 64) s_part[tid] = 0.0f;
+    bool guess = warm != 0;   // x holds the first guess until the end
     if (own) {
         srow[k] = (unsigned short)tid;
         sx[k] = warm ? x[k] : 0.0;
@@ -629,8 +713,8 @@ block_cg_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict
     static_assert(BCG_REP == 8, "put_u writes eight copies");
     __syncthreads();
 
-    int it = 0;
-    bool converged = false;
+    int it = 0, first_its = 0;
+    bool converged = false, over = false;   // over: the last pass was given up
     double rmax = 0.0, rprev = 0.0;
     for (int outer = 0;; ++outer) {
         // r = rhs - A~ x in FP64 from the ELL rows
@@ -643,10 +727,18 @@ block_cg_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict
         const double r64 = own ? (rhs ? rhs[k] : 1.0) - a : 0.0;
         rmax = block_max<NTH>(fabs(r64), s_red);
         if (rmax <= tol) { converged = true; break; }
-        if (!(rmax < 1e15) || rmax < 1e-15 || (outer > 0 && !(rmax < 0.25 * rprev)) ||
-            outer == BCG_OUTER_MAX || it >= maxit)
+        if (outer == 0 && !(rmax < 1.0)) guess = false;   // worse than none
+        const bool failed = outer > 0 && (over || !(rmax < 0.25 * rprev));
+        if (failed || !(rmax < 1e15) || rmax < 1e-15 || outer == BCG_OUTER_MAX || it >= maxit) {
+            // (each row's value is its owner's alone from here on)
+            if (own && (it >= maxit || outer - (failed ? 1 : 0) < 2)) sx[k] = guess ? x[k] : 0.0;
+            else if (own && failed) sx[k] = q.r[k];
             break;
+        }
         rprev = rmax;
+        if (own) q.r[k] = sx[k];   // (the FP64 solver's workspace)
+        CgPass pass = cg_pass(outer, first_its, ns, maxit - it);
+        it += pass.left;
         float r = (float)r64, u = r * inv, p = 0.0f, sv = 0.0f, d = 0.0f, gam = 1.0f, alpha = 1.0f,
               stop = 0.0f;
         put_u(u);
@@ -677,11 +769,19 @@ block_cg_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict
             __syncthreads();
             const float2 tot = part_sum2(s_part, lane);
             const float g1 = tot.x;
-            if (first) stop = cg_stop(g1, BCG_INNER, ns, tol);
+            if (first) {
+                stop = cg_stop(g1, BCG_INNER, ns, tol);
+                if (tid == 0) s_ru0 = g1;
+            }
             if (g1 <= stop) break;
             const float beta = first ? 0.0f : __fdividef(g1, gam);
             const float den = first ? tot.y : tot.y - beta * __fdividef(g1, alpha);
-            if (!(den > 0.0f) || ++it >= maxit) break;   // (a NaN sum ends here too)
+            if (!(den > 0.0f) || pass.left == pass.look) {   // (a NaN sum ends here too)
+                over = pass.left == 0 || (pass.left == pass.look && g1 > s_ru0);
+                if (over || !(den > 0.0f)) break;
+                pass.look = 0;
+            }
+            --pass.left;
             alpha = __fdividef(g1, den);
             gam = g1;
             p = u + beta * p;
@@ -692,15 +792,18 @@ block_cg_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict
             put_u(u);
             __syncthreads();
         }
+        it -= pass.left;
+        if (outer == 0) first_its = it;
         if (own) sx[k] += (double)d;
         __syncthreads();
     }
     if (own) x[k] = sx[k];
     __syncthreads();
     if (!converged) {
-        // what FP32 cannot contract: the FP64 solver, from the refined values
-        // if they are finite with a residual below 1, else from zero
-        converged = pcg_solve<NTH>(ns, q, x, rhs, tol, maxit, rmax < 1.0, s_red, &it, &rmax, err);
+        if (pcg_idle(ns, tid)) return;
+        int n = 0;
+        converged = pcg_takes_over<NTH>(ns, q, x, rhs, tol, maxit, s_red, &n, &rmax, err);
+        it += n;
     }
     if (tid == 0) {
         *q.iters = it;
@@ -1119,7 +1222,10 @@ chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ r
     }
     if (!done) {
     if (CG) {
-        // the dense factor: the lower triangle of A~ (the upper stays zero)
+        // the dense factor: the lower triangle of A~ (the upper stays zero),
+        // and the refinement from where the call started (what FP32 did not
+        // contract may be of any size along the near-null vectors)
+        for (int k = tid; k < ns; k += CHOL_T) sx[k] = warm ? x[k] : 0.0;
         for (int i = tid; i < ns * ld; i += CHOL_T) F[i] = 0.0f;
         __syncthreads();
         for (int k = tid; k < ns; k += CHOL_T) {

@@ -812,3 +812,70 @@ def test_2d_fp32_fluxes_are_as_accurate_along_y_as_along_x(n, m):
         a.close()
         b.close()
     assert abs(rms[1] / rms[0] - 1.0) < 0.025
+
+
+def _curve(n, dim, sep=None):
+    """n markers one cell apart on a line with sub-cell jitter (sep None), or
+    exactly a cell apart with the last one `sep` cells beside another"""
+    g = C.small_grid(dim, (n + 16, 24, 1) if dim == 2 else (n + 16, 12, 12), h=0.1, fp_bytes=8)
+    cells = np.full((n, dim), 5.0)
+    cells[:, 0] = 8 + np.arange(n)
+    if sep is None:
+        cells += np.random.default_rng(n).uniform(-0.3, 0.3, cells.shape)
+    else:
+        cells[-1] = cells[5]
+        cells[-1, 0] += sep
+    return g, np.asarray(g.lo)[:dim] + (cells + 0.5) * g.h
+
+
+@pytest.mark.parametrize("kind,n", [("line", 200), ("line", 700), ("line", 2000), ("sphere", 200),
+                                    ("sphere", 700), ("sphere", 2000), ("pair", 200), ("pair", 700)])
+def test_quadrature_maxit_bounds_the_solver(oracle, kind, n):
+    """A system that the FP64 conjugate gradients (the oracle's) solve in some
+    number of iterations is solved when maxit allows two more, and refused
+    with IBM_ERR_NOCONV at three quarters of it, whatever FP32 corrections
+    come first."""
+    if kind == "sphere":
+        h = np.sqrt(np.pi / n)
+        g = C.small_grid(3, (int(2 / h) + 8,) * 3, h=h, fp_bytes=4)
+        X = C.fibonacci_sphere_markers(n)
+    else:
+        g, X = _curve(n, 2, 0.5 if kind == "pair" else None)
+    rc, _, it, _ = oracle.quadrature(g, X)
+    assert rc == 0
+    for maxit, fine in ((it + 2, True), (int(0.75 * it), False)):
+        grid = ibm.Grid(g, max_markers=n)
+        grid.set_quadrature(1e-12, maxit)
+        if fine:
+            assert grid.set_markers(X, np.ones(n), dedup=False) == n
+            grid.sync()
+        else:
+            with pytest.raises(ibm.IbmError) as e:
+                grid.set_markers(X, np.ones(n), dedup=False)
+                grid.sync()
+            assert e.value.status == 4
+        grid.close()
+
+
+@pytest.mark.parametrize("dim,n", [(3, 300), (2, 5000)])
+def test_near_singular_quadrature_hands_over_early(dim, n):
+    """Two markers 0.1 cells apart: the FP32 corrections cannot finish and end
+    by their own limits, so that the solve takes no longer than with a maxit
+    that ends them (the FP64 solver needs about 70 iterations; an FP32 pass
+    that only maxit = 4000 ends was measured at 1000 and more)."""
+    g, X = _curve(n, dim, 0.1)
+    ms = {}
+    for maxit in (110, 4000):
+        grid = ibm.Grid(g, max_markers=n)
+        grid.set_quadrature(1e-12, maxit)
+        t = []
+        for _ in range(9):
+            e0, e1 = torch.cuda.Event(True), torch.cuda.Event(True)
+            e0.record()
+            grid.set_markers(X, np.ones(n), dedup=False)
+            e1.record()
+            torch.cuda.synchronize()
+            t.append(e0.elapsed_time(e1))
+        ms[maxit] = float(np.median(t))
+        grid.close()
+    assert ms[4000] < 1.4 * ms[110], ms
