@@ -277,8 +277,21 @@ __device__ __forceinline__ float2 part_sum2(const float *part, int lane) {
     const float w = __shfl_xor_sync(0xffffffffu, v, 16);
     return lane & 16 ? make_float2(w, v) : make_float2(v, w);
 }
+// The power of two at or below x: FP32 corrections are solved for r / cg_unit(max
+// |r|), so that they give the same bits at every scale of the right-hand side
+// (the adjoint's may have any) and nothing underflows.
+__device__ __forceinline__ double cg_unit(double x) {
+    return __longlong_as_double(__double_as_longlong(x) & 0x7ff0000000000000ll);
+}
+// 1 / cg_unit(x) (an FP64 division is a chain of some 40 operations of 64 cycles)
+__device__ __forceinline__ double cg_per_unit(double x) {
+    return __longlong_as_double(0x7fe0000000000000ll - (__double_as_longlong(x) & 0x7ff0000000000000ll));
+}
+// residuals whose unit and its reciprocal are normal numbers (not NaN, not inf)
+__device__ __forceinline__ bool cg_in_range(double rmax) { return rmax > 1e-290 && rmax < 1e290; }
 // r.u at which max|r| has fallen far enough: by `inner` from rmax's own r.u,
 // or (the diagonal of A~ is at most one) to a tenth of tol in the mean square
+// (r and tol in units of cg_unit)
 __device__ __forceinline__ float cg_stop(float ru, float inner, int ns, double tol) {
     const float t = 0.1f * (float)tol;
     return fmaxf(ru * inner * inner, (float)ns * t * t);
@@ -511,7 +524,7 @@ cluster_cg_kernel(int ns, const ClusterShape sh, const QuadBuffers q, double *x,
         // no contraction, or a value FP32 cannot hold: the FP64 solver
         if (outer == 0 && !(rmax < 1.0)) guess = false;   // worse than none
         const bool failed = outer > 0 && (over || !(rmax < 0.25 * s_pass.rprev));
-        if (failed || !(rmax < 1e15) || rmax < 1e-15 || outer == CL_OUTER_MAX ||
+        if (failed || !cg_in_range(rmax) || outer == CL_OUTER_MAX ||
             s_pass.it >= maxit) {
             if (writes && (s_pass.it >= maxit || outer - (failed ? 1 : 0) < 2)) x[k] = guess ? q.z[k] : 0.0;
             else if (writes && failed) x[k] = q.r[k];
@@ -520,8 +533,8 @@ cluster_cg_kernel(int ns, const ClusterShape sh, const QuadBuffers q, double *x,
         if (writes) q.r[k] = x[k];
         CgPass pass = cg_pass(outer, s_pass.first, ns, maxit - s_pass.it);
         // the correction d, from zero (a row's threads all hold its values)
-        float r = (float)r64, u = r * inv, p = 0.0f, sv = 0.0f, d = 0.0f, gam = 1.0f, alpha = 1.0f,
-              stop = 0.0f;
+        float r = (float)(r64 * cg_per_unit(rmax)), u = r * inv, p = 0.0f, sv = 0.0f, d = 0.0f,
+              gam = 1.0f, alpha = 1.0f, stop = 0.0f;
         send_u(u);
         if (tid == 0) {   // (every thread is past the tests above)
             s_pass.rprev = rmax;
@@ -553,7 +566,7 @@ cluster_cg_kernel(int ns, const ClusterShape sh, const QuadBuffers q, double *x,
             const float2 tot = reduce_all(sub == 0 ? r * u : 0.0f, sub == 0 ? w * u : 0.0f);
             const float g1 = tot.x, del = tot.y;
             if (first) {
-                stop = cg_stop(g1, CL_INNER, ns, tol);
+                stop = cg_stop(g1, CL_INNER, ns, tol * cg_per_unit(s_pass.rprev));
                 if (tid == 0) s_pass.ru0 = g1;
             }
             if (g1 <= stop) break;
@@ -579,7 +592,7 @@ cluster_cg_kernel(int ns, const ClusterShape sh, const QuadBuffers q, double *x,
             if (outer == 0) s_pass.first = s_pass.it;
         }
         // the next residual reads every CTA's rows
-        if (writes) x[k] += (double)d;
+        if (writes) x[k] += (double)d * cg_unit(s_pass.rprev);
         __threadfence();
         cl.sync();
     }
@@ -729,7 +742,7 @@ block_cg_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict
         if (rmax <= tol) { converged = true; break; }
         if (outer == 0 && !(rmax < 1.0)) guess = false;   // worse than none
         const bool failed = outer > 0 && (over || !(rmax < 0.25 * rprev));
-        if (failed || !(rmax < 1e15) || rmax < 1e-15 || outer == BCG_OUTER_MAX || it >= maxit) {
+        if (failed || !cg_in_range(rmax) || outer == BCG_OUTER_MAX || it >= maxit) {
             // (each row's value is its owner's alone from here on)
             if (own && (it >= maxit || outer - (failed ? 1 : 0) < 2)) sx[k] = guess ? x[k] : 0.0;
             else if (own && failed) sx[k] = q.r[k];
@@ -739,8 +752,8 @@ block_cg_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict
         if (own) q.r[k] = sx[k];   // (the FP64 solver's workspace)
         CgPass pass = cg_pass(outer, first_its, ns, maxit - it);
         it += pass.left;
-        float r = (float)r64, u = r * inv, p = 0.0f, sv = 0.0f, d = 0.0f, gam = 1.0f, alpha = 1.0f,
-              stop = 0.0f;
+        float r = (float)(r64 * cg_per_unit(rmax)), u = r * inv, p = 0.0f, sv = 0.0f, d = 0.0f,
+              gam = 1.0f, alpha = 1.0f, stop = 0.0f;
         put_u(u);
         __syncthreads();
         for (bool first = true;; first = false) {
@@ -770,7 +783,7 @@ block_cg_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict
             const float2 tot = part_sum2(s_part, lane);
             const float g1 = tot.x;
             if (first) {
-                stop = cg_stop(g1, BCG_INNER, ns, tol);
+                stop = cg_stop(g1, BCG_INNER, ns, tol * cg_per_unit(rprev));
                 if (tid == 0) s_ru0 = g1;
             }
             if (g1 <= stop) break;
@@ -794,7 +807,7 @@ block_cg_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict
         }
         it -= pass.left;
         if (outer == 0) first_its = it;
-        if (own) sx[k] += (double)d;
+        if (own) sx[k] += (double)d * cg_unit(rprev);
         __syncthreads();
     }
     if (own) x[k] = sx[k];
@@ -1143,8 +1156,8 @@ chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ r
         rscale = block_max<CHOL_T>(lr, s_red);   // synchronizes
     }
     __syncthreads();
-    // r = rhs - A~ x in FP64 from the ELL rows (one thread per row) into r32,
-    // its largest entry returned (synchronizes)
+    // r = rhs - A~ x in FP64 from the ELL rows (one thread per row) into r32 in
+    // units of cg_unit(rscale), its largest entry returned (synchronizes)
     auto residual = [&]() {
         double lm = 0.0;
         for (int k = tid; k < ns; k += CHOL_T) {
@@ -1171,7 +1184,7 @@ chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ r
                 if (in_bounds(l, ns, err)) sum += q.val[(long long)i * q.cap + k] * sx[l];
             }
             const double r = (rhs ? rhs[k] : 1.0) - sum;
-            r32[k] = (float)r;
+            r32[k] = (float)(r * cg_per_unit(rscale));
             lm = dmax_nonneg(lm, fabs(r));
         }
         return block_max<CHOL_T>(lm, s_red);
@@ -1206,16 +1219,18 @@ chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ r
                 break;
             }
             // no contraction by ten, or nothing FP32 can hold: factor A~
-            if (!(rmax < 1e15) || rmax < 1e-16 || (outer > 0 && !(rmax < 0.1 * rprev)) ||
+            if (!(rmax < 1e30 * rscale) || (outer > 0 && !(rmax < 0.1 * rprev)) ||
                 outer == CHOL_REFINE_MAX)
                 break;
             rprev = rmax;
+            const double m = rmax * cg_per_unit(rscale);   // r32's largest entry
             float d = 0.0f;
             bool got = true;
             if (warp < (ns + 31) / 32) {
-                got = small_cg(ns, q, tid, cnt, rv, rc, inv, ev32, ec, tid < ns ? r32[tid] : 0.0f, st,
+                got = small_cg(ns, q, tid, cnt, rv, rc, inv, ev32, ec,
+                               tid < ns ? r32[tid] * (float)cg_per_unit(m) : 0.0f, st,
                                s_part, d, it);
-                if (got && tid < ns) sx[tid] += (double)d;
+                if (got && tid < ns) sx[tid] += (double)d * (cg_unit(m) * cg_unit(rscale));
             }
             if (__syncthreads_or(!got)) break;
         }
@@ -1341,7 +1356,7 @@ chol_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ r
             }
             __syncthreads();
         }
-        for (int c = tid; c < ns; c += CHOL_T) sx[c] += (double)st[c];
+        for (int c = tid; c < ns; c += CHOL_T) sx[c] += (double)st[c] * cg_unit(rscale);
         __syncthreads();
     }
     }   // !done

@@ -449,3 +449,31 @@ def test_backward_at_the_benchmark_size_fp32_equals_fp64():
     for i in (0, 1):
         a32, a64 = out[4][i], out[8][i]
         assert np.abs(a32 - a64).max() <= 1e-4 * np.abs(a64).max(), (i, np.abs(a32 - a64).max())
+
+
+@pytest.mark.parametrize("exponent", [20, 40, 70])
+@pytest.mark.parametrize("dim,n", [(2, 100), (2, 200), (3, 200), (3, 700)])
+def test_gradient_is_linear_in_small_coefficients(dim, n, exponent):
+    """The reverse sweep is linear in (a, b), and a power of two scales every
+    FP64 number of it exactly: with coefficients 2^-20 to 2^-70 the gradients
+    are the scaled ones bit for bit, through each of the quadrature solvers
+    (up to 160, 512 and more markers, whose right-hand side is scaled)."""
+    if dim == 2:
+        h = np.pi / n
+        size, X = (int(1 / h) + 24, int(1 / h) + 20), C.circle_markers(n)
+    else:
+        h = np.sqrt(np.pi / n)
+        size, X = (int(1 / h) + 12,) * 3, C.fibonacci_sphere_markers(n)
+    g = C.small_grid(dim, size, h=h, fp_bytes=8)
+    grid = ibm.Grid(g, max_markers=n)
+    grid.set_markers(X, np.full(n, 1.3))
+    grid.set_state(C.initial_state(g, 5))
+    grid.record(4, 2)
+    grid.step(4)
+    gX, gT = grid.backward(1.0, 0.5)
+    s = 2.0 ** -exponent
+    sX, sT = grid.backward(s, 0.5 * s)
+    assert np.abs(gX).max() > 0.0
+    np.testing.assert_array_equal(sX / s, gX)
+    np.testing.assert_array_equal(sT / s, gT)
+    grid.close()
