@@ -123,13 +123,18 @@ inline DoubleConsts double_consts(const GridParams &g) {
     return c;
 }
 
-// 1/x and 1/sqrt(x) in FP64 from the hardware seeds (a relative error e below
-// 2^-18) by one step of the third-order Householder iteration, whose error is
-// e^3 plus rounding: r (1 + e + e^2) with e = 1 - x r, and y (1 + e/2 + 3 e^2/8)
-// with e = 1 - x y^2.  Within 2 ulp for positive normal x (the kernels divide
-// by densities, pressures and sums of their differences); four and six
-// operations against ten and more of an IEEE division or square root, on a
-// pipe of two operations per SM cycle.
+// 1/x and 1/sqrt(x) in FP64 from the hardware seeds by one step of the
+// third-order Householder iteration: r (1 + e + e^2) with e = 1 - x r, whose
+// truncation is e^3, and y (1 + e/2 + 3 e^2/8) with e = 1 - x y^2, twice the
+// seed's error, whose truncation is 5 e^3/16; then rounding (in the latter that
+// of x y too).  Seeds good to 2^-19.9 and 2^-20.0, results to 0.51 and 1.0 ulp,
+// measured over the range they are meant for: 2^-1021 <= |x| <= 2^1021, the root
+// of positive x (the kernels divide by densities, pressures and sums of their
+// differences; held to 2 ulp by a test).  Outside it there is no result: x = 0,
+// subnormal or infinite gives NaN, where a division gives infinity or zero - a
+// cell of zero density or pressure is reported by its step-size rate either way.
+// Four and six operations against ten and more of an IEEE division or square
+// root, on a pipe of two operations per SM cycle.
 __device__ __forceinline__ double drcp(double x) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
