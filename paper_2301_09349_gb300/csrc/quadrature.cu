@@ -18,8 +18,9 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <atomic>
 
-#include "device_table.h"
+#include "cluster_plan.h"
 #include "internal.h"
 
 namespace cg = cooperative_groups;
@@ -366,28 +367,10 @@ __device__ __forceinline__ bool pcg_idle(int ns, int tid) { return ns <= 2048 &&
 // the same branches and the result is bitwise reproducible.  A system that
 // FP32 cannot contract (near-singular A~: two markers in one cell placed
 // without dedup) goes to the FP64 PCG in the same launch.
-constexpr int CL_CTAS = 8, CL_CTAS_WIDE = 16;
-constexpr int CL_WIDE = 1536;            // above, the product of 8 CTAs outweighs 16's exchange
-constexpr int CL_MAX = 16384;            // 16 CTAs of 1024 rows, 16-bit columns
 constexpr int CL_SM = 16;                // entries of a thread in shared memory
 constexpr float CL_INNER = 1e-5f;
 constexpr int CL_OUTER_MAX = 24;
 template <int NTH> constexpr int CL_REG = NTH <= 512 ? 24 : 12;   // entries in registers
-
-struct ClusterShape {
-    int ctas;       // CTAs of the cluster
-    int rows;       // rows per CTA, a multiple of 4
-    int lpr_log;    // log2 of the threads per row
-};
-
-ClusterShape cluster_shape(int ns) {
-    ClusterShape c;
-    c.ctas = ns > CL_WIDE ? CL_CTAS_WIDE : CL_CTAS;
-    c.rows = ((ns + c.ctas - 1) / c.ctas + 3) / 4 * 4;   // chunks of u move as 16-byte words
-    c.lpr_log = 0;
-    while (c.lpr_log < 4 && (2 << c.lpr_log) * c.rows <= 512) ++c.lpr_log;
-    return c;
-}
 
 // u of every row (16-byte aligned), the CTAs' FP64 maxima and partial sums,
 // the threads' entries past their registers
@@ -612,31 +595,63 @@ cluster_cg_kernel(int ns, const ClusterShape sh, const QuadBuffers q, double *x,
 }
 
 template <int NTH>
-cudaError_t launch_cluster_cg(int ns, const ClusterShape &sh, const QuadBuffers &qb, double *x,
-                              const double *rhs, double tol, int maxit, int warm, int *err,
-                              cudaStream_t s) {
-    const void *fn = (const void *)cluster_cg_kernel<NTH>;
-    const size_t smem = cluster_smem<NTH>(sh);
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = func_smem_attr(fn, smem);
-    if (e != cudaSuccess) return e;
-    static DeviceAttrTable wide;   // clusters of 16 are an opt-in of the kernel, per device
-    e = (cudaError_t)wide.ensure(fn, dev, 1, [&]() -> int {
-        return (int)cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    });
-    if (e != cudaSuccess) return e;
+cudaLaunchConfig_t cluster_config(const ClusterShape &sh, cudaLaunchAttribute *at, cudaStream_t s) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)sh.ctas);
     cfg.blockDim = dim3(NTH);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = cluster_smem<NTH>(sh);
     cfg.stream = s;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = (unsigned)sh.ctas;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = (unsigned)sh.ctas;
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    cfg.attrs = at;
     cfg.numAttrs = 1;
+    return cfg;
+}
+
+// Whether the device can hold one cluster of `ctas` CTAs of the kernel at its
+// largest (16 need as many SMs with room in one GPC, which a partition of the
+// device may lack).
+template <int NTH> bool cluster_fits(int ctas) {
+    const void *fn = (const void *)cluster_cg_kernel<NTH>;
+    const ClusterShape sh{ctas, NTH < CL_ROWS ? NTH : CL_ROWS, 0};
+    if (func_smem_attr(fn, cluster_smem<NTH>(sh)) != cudaSuccess) return false;
+    if (ctas > CL_CTAS &&
+        cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    cudaLaunchAttribute at{};
+    const cudaLaunchConfig_t cfg = cluster_config<NTH>(sh, &at, nullptr);
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess) return n > 0;
+    cudaGetLastError();   // not a launch error of the caller's
+    return false;
+}
+
+// CTAs of the widest cluster that both kernels can run as (16, 8 or 0), asked
+// of a device once.
+int widest_cluster() {
+    static std::atomic<int> of_device[64];   // 0: not yet asked, else CTAs + 1
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    int w = dev < 64 ? of_device[dev].load() : 0;
+    if (w == 0) {
+        auto both = [](int ctas) { return cluster_fits<512>(ctas) && cluster_fits<1024>(ctas); };
+        w = 1 + (both(CL_CTAS_WIDE) ? CL_CTAS_WIDE : both(CL_CTAS) ? CL_CTAS : 0);
+        if (dev < 64) of_device[dev].store(w);
+    }
+    return w - 1;
+}
+
+template <int NTH>
+cudaError_t launch_cluster_cg(int ns, const ClusterShape &sh, const QuadBuffers &qb, double *x,
+                              const double *rhs, double tol, int maxit, int warm, int *err,
+                              cudaStream_t s) {
+    const cudaError_t e = func_smem_attr((const void *)cluster_cg_kernel<NTH>, cluster_smem<NTH>(sh));
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at{};
+    const cudaLaunchConfig_t cfg = cluster_config<NTH>(sh, &at, s);
     return cudaLaunchKernelEx(&cfg, cluster_cg_kernel<NTH>, ns, sh, qb, x, rhs, tol, maxit, warm, err);
 }
 
@@ -1383,7 +1398,7 @@ int quad_row_width(int dim) { return dim == 3 ? 125 * 4 : 25 * 4; }
 
 // A~ x = rhs (rhs == nullptr: all ones), warm-started if asked.  One CTA up
 // to BCG_MAX markers, one cluster to CL_MAX (both sides of each line measured
-// at the kernels), the FP64 PCG above
+// at the kernels), the FP64 PCG above and where no cluster can be placed
 static cudaError_t launch_quadrature_solve_w(int dim, int ns, const QuadBuffers &qb, const double *rhs,
                                             double *x, double tol, int maxit, int warm, int *err,
                                             cudaStream_t s) {
@@ -1399,13 +1414,16 @@ static cudaError_t launch_quadrature_solve_w(int dim, int ns, const QuadBuffers 
     } else if (ns <= BCG_MAX) {
         return ns <= 512 ? launch_block_cg<512>(ns, qb, x, rhs, tol, maxit, warm, err, s)
                          : launch_block_cg<1024>(ns, qb, x, rhs, tol, maxit, warm, err, s);
-    } else if (ns <= CL_MAX) {
-        const ClusterShape sh = cluster_shape(ns);
-        return sh.rows <= 512
-                   ? launch_cluster_cg<512>(ns, sh, qb, x, rhs, tol, maxit, warm, err, s)
-                   : launch_cluster_cg<1024>(ns, sh, qb, x, rhs, tol, maxit, warm, err, s);
     } else {
-        pcg_kernel<1024><<<1, 1024, 0, s>>>(ns, qb, x, rhs, tol, maxit, warm, err);
+        const ClusterShape sh = ns <= CL_MAX ? cluster_shape(ns, widest_cluster()) : ClusterShape{0, 0, 0};
+        if (sh.ctas > 0)
+            return sh.rows <= 512
+                       ? launch_cluster_cg<512>(ns, sh, qb, x, rhs, tol, maxit, warm, err, s)
+                       : launch_cluster_cg<1024>(ns, sh, qb, x, rhs, tol, maxit, warm, err, s);
+        if (ns <= 2048)
+            pcg_kernel<256><<<1, 256, 0, s>>>(ns, qb, x, rhs, tol, maxit, warm, err);
+        else
+            pcg_kernel<1024><<<1, 1024, 0, s>>>(ns, qb, x, rhs, tol, maxit, warm, err);
     }
     return cudaGetLastError();
 }

@@ -879,3 +879,25 @@ def test_near_singular_quadrature_hands_over_early(dim, n):
         ms[maxit] = float(np.median(t))
         grid.close()
     assert ms[4000] < 1.4 * ms[110], ms
+
+
+@pytest.mark.parametrize("count", [600, 1700])
+def test_cluster_solve_inside_captured_steps(count):
+    """A moving body of more markers than one CTA takes: its weights are solved
+    by a cluster every step, launched and replayed from graphs alike."""
+    g = C.small_grid(3, (44, 40, 36), h=0.1, fp_bytes=4, Re=100.0, Mach=0.3)
+    X = C.random_markers(g, count, seed=61)
+    out = []
+    for graphs in (0, 4):
+        grid = ibm.Grid(g, max_markers=count)
+        if graphs:
+            grid.use_graphs(graphs)
+        assert grid.set_markers(X, np.full(count, 1.2), dedup=False,
+                                motion=C.Motion(0.05, 2.0, 1)) == count
+        grid.set_state(C.initial_state(g, 5).astype(np.float32))
+        grid.step(8)
+        grid.sync()
+        out.append((grid.get_state(), grid.markers()[1]))
+        grid.close()
+    assert torch.equal(out[0][0], out[1][0])
+    np.testing.assert_array_equal(out[0][1], out[1][1])
