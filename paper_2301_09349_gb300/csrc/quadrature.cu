@@ -9,11 +9,12 @@
 // assembled in ELL form (column-major, one warp per marker, neighbours
 // found through the marker bins in a fixed order).  The solution is FP64:
 // residuals rhs - A~ x and the stopping test are formed in FP64, and only the
-// corrections come from FP32 conjugate gradients, on one CTA (up to 512
-// markers) or one thread-block cluster (up to 16384).  Systems FP32 cannot
-// contract go to a dense FP32 Cholesky refined in FP64 (up to 160 markers)
-// and to Jacobi-preconditioned CG in FP64 on one CTA, which also takes the
-// systems of more than 16384 markers.  Fixed-order sums throughout: the
+// corrections are FP32.  Up to 160 markers they come from a dense Cholesky
+// factor on one CTA, in 2D with more than 64 markers and short rows from
+// conjugate gradients first; above, from conjugate gradients on one CTA (up to
+// 512 markers) or one thread-block cluster (up to 16384).  Systems that these
+// cannot contract, and those of more than 16384 markers, go to Jacobi-
+// preconditioned CG in FP64 on one CTA.  Fixed-order sums throughout: the
 // result is bitwise reproducible; every loop is bounded.
 #include <cooperative_groups.h>
 
@@ -670,19 +671,16 @@ constexpr int BCG_REP = 8;              // copies of u: lane l gathers from copy
                                         // lanes of a warp can meet in a bank
 constexpr int BCG_OUTER_MAX = 24;
 constexpr float BCG_INNER = 1e-5f;
-template <int NTH> constexpr int BCG_REG = NTH <= 512 ? 32 : 12;   // entries in registers
+constexpr int BCG_REG = 32;             // entries of a thread in registers
 
-template <int NTH>
-constexpr size_t block_cg_smem() {
-    return sizeof(double) * NTH + (sizeof(float) + sizeof(unsigned short)) * (size_t)BCG_SM * NTH +
-           sizeof(float) * BCG_REP * NTH + sizeof(unsigned short) * NTH;
-}
+constexpr size_t BCG_SMEM = sizeof(double) * BCG_MAX +
+                            (sizeof(float) + sizeof(unsigned short)) * (size_t)BCG_SM * BCG_MAX +
+                            sizeof(float) * BCG_REP * BCG_MAX + sizeof(unsigned short) * BCG_MAX;
 
-template <int NTH>
-__global__ void __launch_bounds__(NTH, 1)
+__global__ void __launch_bounds__(BCG_MAX, 1)
 block_cg_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict__ rhs, double tol,
                 int maxit, int warm, int *err) {
-    constexpr int REG = BCG_REG<NTH>;
+    constexpr int NTH = BCG_MAX, REG = BCG_REG;
     extern __shared__ __align__(16) double smem_b[];
     double *sx = smem_b;                                          // [NTH] solution, marker order
     float *sval = reinterpret_cast<float *>(sx + NTH);            // [BCG_SM][NTH]
@@ -840,19 +838,19 @@ block_cg_kernel(int ns, const QuadBuffers q, double *x, const double *__restrict
     }
 }
 
-template <int NTH>
 cudaError_t launch_block_cg(int ns, const QuadBuffers &qb, double *x, const double *rhs, double tol,
                             int maxit, int warm, int *err, cudaStream_t s) {
-    cudaError_t e = func_smem_attr((const void *)block_cg_kernel<NTH>, block_cg_smem<NTH>());
+    cudaError_t e = func_smem_attr((const void *)block_cg_kernel, BCG_SMEM);
     if (e != cudaSuccess) return e;
-    block_cg_kernel<NTH><<<1, NTH, block_cg_smem<NTH>(), s>>>(ns, qb, x, rhs, tol, maxit, warm, err);
+    block_cg_kernel<<<1, BCG_MAX, BCG_SMEM, s>>>(ns, qb, x, rhs, tol, maxit, warm, err);
     return cudaGetLastError();
 }
 
-// Small systems (up to CHOL_MAX markers) on one CTA: corrections by FP32
-// conjugate gradients first (small_cg); a system they do not contract by ten
-// per pass is factored.  A~ is then copied dense, in FP32, into shared memory
-// from the ELL rows.  FP64 runs at a small fraction of the FP32 rate on this GPU, so
+// Small systems (up to CHOL_MAX markers) on one CTA.  In 2D, above SCG_MIN
+// markers and with rows of at most SCG_ROW entries, corrections come from FP32
+// conjugate gradients first (small_cg); a system they do not contract by ten per
+// pass, and every other one, is factored.  A~ is then copied dense, in FP32, into
+// shared memory from the ELL rows.  FP64 runs at a small fraction of the FP32 rate on this GPU, so
 // the O(ns^3) work is done in FP32: a blocked right-looking Cholesky
 // A~ = L L^T over 32-column panels (one warp factors the panel's diagonal
 // block without block barriers, one thread per row solves the rows below
@@ -1412,8 +1410,7 @@ static cudaError_t launch_quadrature_solve_w(int dim, int ns, const QuadBuffers 
         if (e != cudaSuccess) return e;
         kernel<<<1, CHOL_T, chol_smem(ns), s>>>(ns, qb, x, rhs, tol, maxit, warm, err);
     } else if (ns <= BCG_MAX) {
-        return ns <= 512 ? launch_block_cg<512>(ns, qb, x, rhs, tol, maxit, warm, err, s)
-                         : launch_block_cg<1024>(ns, qb, x, rhs, tol, maxit, warm, err, s);
+        return launch_block_cg(ns, qb, x, rhs, tol, maxit, warm, err, s);
     } else {
         const ClusterShape sh = ns <= CL_MAX ? cluster_shape(ns, widest_cluster()) : ClusterShape{0, 0, 0};
         if (sh.ctas > 0)
