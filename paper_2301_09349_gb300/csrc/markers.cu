@@ -1506,10 +1506,15 @@ cudaError_t launch_motion(const GridParams &g, const MarkerBuffers &m, double am
     return cudaGetLastError();
 }
 
-// One CTA forms ~25 weights a microsecond beside its other work; the launch
-// that spreads them over all SMs takes 4 us (388 markers in 3D, 3492 weights:
-// the rebuild takes 17 us more with them; 98 in 2D, 588, leave
-// it at 16).
+// Whether the rebuild's one CTA forms the support weights itself or a launch
+// after it does, which has every SM's FP64 pipe and costs its place in the chain.
+// Us a step, within - apart, for a moving circle (6 weights a marker) and sphere
+// (9): replayed from graphs -0.2 at 360 and 552 weights of the circle, +0.4 at
+// 648, +1.1 at 936, +1.7 at 1152, +3.1 at 1488; sphere +0.6 at 306, +1.3 at 549,
+// +1.5 at 810, +3.3 at 1224.  Launched step by step, where a launch costs more,
+// -3.3 at 480 and 552 of the circle, -1.6 at 936 and 1152, +1 at 1488; sphere 0
+// to -1.5 up to 1242, +1.7 at 1593.  The line is the circle's crossing under
+// graphs.
 int small_rebuild_weights(const GridParams &g, const MarkerBuffers &m) {
     return m.ns * g.dim * 3 <= 600;
 }
