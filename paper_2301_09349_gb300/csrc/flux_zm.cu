@@ -672,7 +672,8 @@ zmarch_kernel(const __grid_constant__ CUtensorMap tmap, const GridParams g, cons
     const int gx = ox + 2 * t, gy = oy + r;
     const bool row_in = gy < g.n[1];
     const bool in0 = row_in && gx < g.n[0], in1 = row_in && gx + 1 < g.n[0];
-    const bool vec = in1 && (g.n[0] % 2 == 0);   // both cells, 8-byte aligned
+    // both cells at once, 8-byte aligned (a caller's L may be 4-byte aligned only)
+    const bool vec = in1 && g.n[0] % 2 == 0 && (MODE != 0 || ((uintptr_t)out & 7) == 0);
     float smaxf = 0.0f;
     bool ok = true;
     for (int z = z0; z < z1; ++z) {

@@ -901,3 +901,25 @@ def test_cluster_solve_inside_captured_steps(count):
         grid.close()
     assert torch.equal(out[0][0], out[1][0])
     np.testing.assert_array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("offset", [1, 2, 3])
+@pytest.mark.parametrize("n", [(36, 18, 5), (34, 17, 6), (33, 17, 6)])
+def test_3d_fp32_rhs_of_arrays_at_any_float(n, offset):
+    """L(U) of a state and into an array that start 4, 8 or 12 bytes past a
+    16-byte boundary: the bits of the aligned call, and nothing written past
+    its end."""
+    g = C.small_grid(3, n, h=0.1, fp_bytes=4)
+    U = torch.from_numpy(C.random_state(g, 9).astype(np.float32)).cuda()
+    buf = torch.zeros(2 * U.numel() + 16, dtype=torch.float32, device="cuda")
+    Ua = buf[offset:offset + U.numel()].view(U.shape)
+    start = (U.numel() + 7) // 4 * 4 + offset
+    La = buf[start:start + U.numel()].view(U.shape)
+    Ua.copy_(U)
+    grid = ibm.Grid(g)
+    L = grid.rhs(U)
+    ibm.ibm_rhs(grid.h, Ua.data_ptr(), La.data_ptr())
+    torch.cuda.synchronize()
+    assert torch.equal(La, L)
+    assert float(buf[start + U.numel():].abs().max()) == 0.0
+    grid.close()
