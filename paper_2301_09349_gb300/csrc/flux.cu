@@ -419,13 +419,12 @@ batch_stage_kernel(const BatchCase *__restrict__ cases, const int2 *__restrict__
     }
 }
 
-// *dt = cfl / max_j s_j(U) over every cell: per-CTA maxima, then the last
-// CTA to finish reduces them.
-// First step size of a new state, and its time and step count (where given).
-// Bound by memory on large grids; maxima stay in the grid's type and double
-// maxima are integer work: a conversion and an FP64 maximum per cell kept the
-// FP64 pipe busy for most of 103 us at 256^3 (now 56, 50 for its
-// bytes; 1024 x 512 17.0 -> 10.8).
+// First step size of a new state, *dt = cfl / max_j s_j(U) over every cell, and
+// its time and step count (where given): per-CTA maxima, which the last CTA to
+// finish reduces.  Bound by memory on large grids; the cells' and a warp's maxima
+// stay in the grid's type, and those of warps and CTAs are integer work: on FP32
+// grids a conversion and an FP64 maximum per cell kept the FP64 pipe busy for
+// most of 103 us at 256^3 (now 56, 50 for its bytes; 1024 x 512 17.0 -> 10.8).
 template <int DIM, typename T>
 __global__ void __launch_bounds__(NT)
 dt_init_kernel(const GridParams g, const T *__restrict__ U, double *__restrict__ blockmax,

@@ -14,7 +14,7 @@
 // the first row of a chunk repeat their neighbours' work: 64/60 of the
 // columns, and about 0.7 row per chunk).
 //
-// Bound: instruction issue and latency (345 / 425 thread instructions per
+// Bound: instruction issue and latency (348 / 430 thread instructions per
 // cell and stage at 50 % issue with three to four warps per scheduler, against
 // 32 or 48 bytes of memory traffic).  The form this replaces - one cell per
 // thread of a 16 x 16 tile, primitives and face fluxes in shared memory, both
@@ -660,8 +660,12 @@ batch_ymarch_kernel(const BatchCase *__restrict__ cases, const int2 *__restrict_
 // 2 / 1 rows of 219 x 103: 41 / 26 / 20 / 16.5 us a step).  Where single rows
 // of 28 columns are one wave, those: 11.6 us, and 13.1 / 14.7 us at 300 x 150 /
 // 350 x 200 against 18.1 and 19 by the march; the 16 x 16 tiles these forms
-// replace took 13.8, 15.9 and 16.1.  Larger: 467 x 428 23.2 (23.8 by tiles),
-// 640 x 480 25.0 (26.6).  At most 64 rows.
+// replace took 13.8, 15.9 and 16.1.  Larger, with the step's finish: 468 x 428
+// 28.8 (30.9 by tiles), 640 x 480 28.9 (34.8), 2048 x 1024 86 (136).  Odd nx,
+// whose pairs are loaded and stored one by one, gains less: 467 x 428 30.9
+// (30.9), 641 x 481 33.5 (35.4), 1025 x 513 43.2 (48), 2047 x 1023 107 (135),
+// 4095 x 2047 361 (500); batches of 32 cases of 101 to 105, 201 to 205 and 401
+// to 405 columns 35 (39), 81 (102) and 338 (381).  At most 64 rows.
 struct YmPlan {
     int width, rows;
 };

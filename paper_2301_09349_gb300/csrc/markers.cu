@@ -409,7 +409,7 @@ __device__ __forceinline__ void interp_fields(const R *__restrict__ U, long long
 // the field precision.  A chain of latencies: the cell's values are loaded
 // ahead of the weights (FP64 grids take the tabulated ones, an FP64 square
 // root costs a warp a thousand cycles), the sums share their butterflies, and
-// lane d forms component d.  Heated cylinder (FP64) 10.5 -> 5.6 us.
+// lane d forms component d.  Heated cylinder (FP64) 10.5 -> 5.2 us.
 template <int DIM> __device__ __forceinline__ float support_weight(const MarkerBuffers &m, int k,
                                                                    const int (&o)[3], float) {
     float w = 1.0f;
